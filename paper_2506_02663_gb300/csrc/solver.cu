@@ -1980,19 +1980,19 @@ amr_status wsum(amr_hierarchy* h, const double* x, const double* bc, const int* 
   return AMR_OK;
 }
 
+// h^D summed over the valid cells.  A level's invalid cells are the coarsened cells of the next
+// level's boxes (disjoint, nested in this level, edges on coarse cells), so the count is exact
+// integer arithmetic on the box extents: reading the 18.9 M flags of the 256^3 + 128^3 hierarchy
+// one by one on the host took milliseconds before the solve's first launch, twice a solve.
 double valid_volume(const amr_hierarchy* h) {
-  // number of valid cells per level times h^D (exact small integers times powers of 2)
   long double v = 0.0L;
-  size_t q = 0;
-  for (int l = 0; l < h->L; ++l) {
-    long long cnt = 0;
-    for (const PatchDesc& p : h->lev[l].patches) {
-      const long long nc = (long long)p.n[0] * p.n[1] * p.n[2];
-      for (long long i = 0; i < nc; ++i) cnt += h->im_valid[q + i];
-      q += nc;
-    }
-    v += (long double)cnt * std::pow((long double)h->lev[l].h, (long double)h->D);
-  }
+  std::vector<long long> cells(h->L + 1, 0);
+  for (int l = 0; l < h->L; ++l)
+    for (const PatchDesc& p : h->lev[l].patches) cells[l] += (long long)p.n[0] * p.n[1] * p.n[2];
+  long long children = 1;
+  for (int d = 0; d < h->D; ++d) children *= h->r;
+  for (int l = 0; l < h->L; ++l)
+    v += (long double)(cells[l] - cells[l + 1] / children) * std::pow((long double)h->lev[l].h, (long double)h->D);
   return (double)v;
 }
 
