@@ -357,185 +357,10 @@ __global__ void __launch_bounds__(BX* BY) k_level_op2d_tiled(LevelView lv, const
   level_op2d_tiled_body<T, MODE, TR, ROWS>(lv, blockIdx.z, x, f, out, bc, alpha, beta, omega, omega_over_diag, vmask);
 }
 
-// 3-D level operator, marching in z (homogeneous physical data, forward operator): a block
-// owns a 32 x 8 tile of (x, y) columns and walks a range of z planes.  Each thread keeps its
-// column's five z values in registers; the current plane of the tile plus a two-cell halo
-// sits in shared memory (double-buffered, one barrier per plane).  Halo cells inside the
-// domain come from global memory (patch interior or its stored CF / copy ghosts); cells
-// outside the domain are the ghost formulas of Eqs. (velBCHomoDiri5th)/(Neumann5) evaluated
-// from the column or row they extend; the Jacobi factor omega / diag comes from a 125-entry
-// table indexed by the cell's distance class to the x, y and z faces.  Same summation order
-// as cell_Lx.
 // distance class of global index g to the faces of an n-cell dimension: 0 interior, 1 and 2
 // the first and second cell from the low face, 3 and 4 from the high face
 __device__ __forceinline__ int face_class(int g, int n) {
   return g == 0 ? 1 : g == 1 ? 2 : g == n - 1 ? 3 : g == n - 2 ? 4 : 0;
-}
-
-constexpr int MZ_TX = 32, MZ_TY = 8, MZ_W = MZ_TX + 4, MZ_H = MZ_TY + 4;
-
-template <typename T>
-__device__ __forceinline__ T mz_column(const T* __restrict__ xb, long long base, long long stride, int g, int n, int lo,
-                                       const LevelView& lv, int d) {
-  // value at global index g along d (base = offset of local index 0), ghost formula outside
-  if (g >= 0 && g < n) return xb[base + (long long)(g - lo) * stride];
-  const int side = g < 0 ? 0 : 1, layer = side == 0 ? -g : g - n + 1, type = lv.bc[2 * d + side];
-  T v = T(0);
-#pragma unroll
-  for (int m = 0; m < 4; ++m) v += gcoef<T>(type, layer - 1, m) * xb[base + (long long)((side == 0 ? m : n - 1 - m) - lo) * stride];
-  return v;
-}
-
-// x at patch-local (li, lj) of plane k as the stencil sees it: stored values (interior, or
-// CF / copy ghosts) inside the domain, the ghost formula outside; 0 at positions no stencil of
-// an interior cell reads (corners, beyond the stored ghost layers).  The formula cases are
-// rare and kept out of line.
-template <typename T>
-__device__ __noinline__ T mz_plane_value_slow(const T* __restrict__ x, const PatchDesc& p, const LevelView& lv, int li,
-                                              int lj, int k) {
-  const int gi = p.lo[0] + li, gj = p.lo[1] + lj;
-  const bool ox = gi < 0 || gi >= lv.ndom[0], oy = gj < 0 || gj >= lv.ndom[1];
-  if (ox && oy) return T(0);
-  if (li < -NG || li >= p.n[0] + NG || lj < -NG || lj >= p.n[1] + NG) return T(0);
-  if (ox) {
-    const int side = gi < 0 ? 0 : 1, layer = side == 0 ? -gi : gi - lv.ndom[0] + 1, type = lv.bc[side];
-    T v = T(0);
-#pragma unroll
-    for (int m = 0; m < 4; ++m) v += gcoef<T>(type, layer - 1, m) * x[poff(p, (side == 0 ? m : lv.ndom[0] - 1 - m) - p.lo[0], lj, k)];
-    return v;
-  }
-  if (oy) {
-    const int side = gj < 0 ? 0 : 1, layer = side == 0 ? -gj : gj - lv.ndom[1] + 1, type = lv.bc[2 + side];
-    T v = T(0);
-#pragma unroll
-    for (int m = 0; m < 4; ++m) v += gcoef<T>(type, layer - 1, m) * x[poff(p, li, (side == 0 ? m : lv.ndom[1] - 1 - m) - p.lo[1], k)];
-    return v;
-  }
-  return x[poff(p, li, lj, k)];
-}
-
-template <typename T>
-__device__ __forceinline__ T mz_plane_value(const T* __restrict__ x, const PatchDesc& p, const LevelView& lv, int li, int lj,
-                                           int k) {
-  const int gi = p.lo[0] + li, gj = p.lo[1] + lj;
-  if (gi >= 0 && gi < lv.ndom[0] && gj >= 0 && gj < lv.ndom[1] && li >= -NG && li < p.n[0] + NG && lj >= -NG &&
-      lj < p.n[1] + NG)
-    return x[poff(p, li, lj, k)];
-  return mz_plane_value_slow<T>(x, p, lv, li, lj, k);
-}
-
-template <typename T, int MODE>
-__global__ void __launch_bounds__(MZ_TX* MZ_TY, 4) k_level_op3d_march(LevelView lv, int nzc, int kz, const T* __restrict__ x,
-                                                                 const T* __restrict__ f, T* __restrict__ out, T alpha,
-                                                                 T beta, T omega,
-                                                                 const unsigned char* __restrict__ vmask) {
-  pdl_wait();
-  __shared__ T sp[2][MZ_H * MZ_W];
-  __shared__ T wt[125];
-  const int pz = blockIdx.z / nzc, zc = blockIdx.z % nzc;
-  const PatchDesc p = lv.patches[pz];
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * MZ_TX + tx;
-  const int i0 = blockIdx.x * MZ_TX, j0 = blockIdx.y * MZ_TY;
-  const int i = i0 + tx, j = j0 + ty;
-  const int k0 = zc * kz, k1 = min(k0 + kz, p.n[2]);
-  if (i0 >= p.n[0] || j0 >= p.n[1] || k0 >= k1) return;
-  const bool active = i < p.n[0] && j < p.n[1];
-  const T inv = pick<T>(lv.inv12h2, lv.inv12h2_f);
-  if (MODE == OP_JACOBI || MODE == OP_JACOBI0) {
-    for (int q = tid; q < 125; q += MZ_TX * MZ_TY) {
-      const int a = q % 5, b = (q / 5) % 5, c = q / 25;
-      const int cls[3] = {a, b, c};
-      T acc = T(-90);
-#pragma unroll
-      for (int d = 0; d < 3; ++d)
-        if (cls[d]) acc += pick<T>(lv.dcorr[2 * d + (cls[d] - 1) / 2][(cls[d] - 1) % 2],
-                                   lv.dcorr_f[2 * d + (cls[d] - 1) / 2][(cls[d] - 1) % 2]);
-      wt[q] = omega / (alpha + beta * inv * acc);
-    }
-  }
-  const long long sy = p.sy, sz = p.sz;
-  const int gi = p.lo[0] + i, gj = p.lo[1] + j;
-  // the halo cell this thread loads (tile-local coordinates; 176 cells, threads 0..175)
-  int hx = -100, hy = -100;
-  {
-    int q = tid;
-    if (q < 2 * MZ_W) {  // two rows below the tile
-      hy = -2 + q / MZ_W;
-      hx = q % MZ_W - 2;
-    } else if ((q -= 2 * MZ_W) < 2 * MZ_W) {  // two rows above
-      hy = MZ_TY + q / MZ_W;
-      hx = q % MZ_W - 2;
-    } else if ((q -= 2 * MZ_W) < 4 * MZ_TY) {  // two columns left and right of the tile rows
-      hy = q % MZ_TY;
-      const int c = q / MZ_TY;  // 0, 1: left (-2, -1); 2, 3: right (TX, TX + 1)
-      hx = c < 2 ? c - 2 : MZ_TX + c - 2;
-    }
-    // corners of the halo are never read by the axis-aligned stencil
-    if ((hx < 0 || hx >= MZ_TX) && (hy < 0 || hy >= MZ_TY)) hx = hy = -100;
-  }
-  const bool has_halo = hx > -100;
-  // column base offsets (local index 0 along z)
-  const long long colc = p.off + (long long)(i + NG) + (long long)(j + NG) * sy + (long long)NG * sz;
-  const int nzd = lv.ndom[2], lz = p.lo[2];
-  const int kxc = face_class(gi, lv.ndom[0]), kyc = face_class(gj, lv.ndom[1]);
-  // register queue of the column: x at planes k-2 .. k+2
-  T q0 = T(0), q1 = T(0), q2 = T(0), q3 = T(0), q4 = T(0);
-  if (active && MODE != OP_JACOBI0) {
-    q0 = mz_column<T>(x, colc, sz, lz + k0 - 2, nzd, lz, lv, 2);
-    q1 = mz_column<T>(x, colc, sz, lz + k0 - 1, nzd, lz, lv, 2);
-    q2 = x[colc + (long long)k0 * sz];
-    q3 = mz_column<T>(x, colc, sz, lz + k0 + 1, nzd, lz, lv, 2);
-    q4 = mz_column<T>(x, colc, sz, lz + k0 + 2, nzd, lz, lv, 2);
-  }
-  // software pipeline: the plane-k loads (halo, the centre of an inactive tile cell, f) are
-  // issued one plane ahead, so their latency overlaps the barrier and the arithmetic
-  T hnext = T(0), cnext = T(0), fnext = T(0);
-  if (MODE != OP_JACOBI0) {
-    if (has_halo) hnext = mz_plane_value<T>(x, p, lv, i0 + hx, j0 + hy, k0);
-    if (!active) cnext = mz_plane_value<T>(x, p, lv, i, j, k0);
-  }
-  if (active && MODE != OP_APPLY) fnext = f[colc + (long long)k0 * sz];
-  __syncthreads();  // weight table
-  for (int k = k0, buf = 0; k < k1; ++k, buf ^= 1) {
-    const long long oc = colc + (long long)k * sz;
-    const T fk = fnext;
-    if (MODE != OP_JACOBI0) {
-      T* s = sp[buf];
-      // tile cells outside the patch (ragged tiles) hold the ghost values next to it
-      s[(ty + 2) * MZ_W + tx + 2] = active ? q2 : cnext;
-      if (has_halo) s[(hy + 2) * MZ_W + hx + 2] = hnext;
-      if (k + 1 < k1) {
-        if (has_halo) hnext = mz_plane_value<T>(x, p, lv, i0 + hx, j0 + hy, k + 1);
-        if (!active) cnext = mz_plane_value<T>(x, p, lv, i, j, k + 1);
-      }
-    }
-    if (active && MODE != OP_APPLY && k + 1 < k1) fnext = f[oc + sz];
-    if (MODE != OP_JACOBI0) __syncthreads();
-    if (active && (vmask == nullptr || vmask[oc])) {
-      const int kzc = face_class(lz + k, nzd);
-      if (MODE == OP_JACOBI0) {
-        out[oc] = wt[kxc + 5 * kyc + 25 * kzc] * fk;
-      } else {
-        const T* s = sp[buf];
-        const int c = (ty + 2) * MZ_W + tx + 2;
-        const T xc = q2;
-        const T s1 = ((s[c - 1] + s[c + 1]) + (s[c - MZ_W] + s[c + MZ_W])) + (q1 + q3);
-        const T s2 = ((s[c - 2] + s[c + 2]) + (s[c - 2 * MZ_W] + s[c + 2 * MZ_W])) + (q0 + q4);
-        const T lap = (T(16) * s1 - s2 - T(90) * xc) + T(0);
-        const T ax = alpha * xc + beta * (lap * inv);
-        if (MODE == OP_APPLY) out[oc] = ax;
-        else if (MODE == OP_RESID) out[oc] = fk - ax;
-        else out[oc] = xc + wt[kxc + 5 * kyc + 25 * kzc] * (fk - ax);
-      }
-    }
-    if (MODE != OP_JACOBI0 && active) {
-      q0 = q1;
-      q1 = q2;
-      q2 = q3;
-      q3 = q4;
-      if (k + 1 < k1) q4 = mz_column<T>(x, colc, sz, lz + k + 3, nzd, lz, lv, 2);
-    }
-  }
 }
 
 // ------------------------------------------------------------------------ z-chunked 3-D marching operator
@@ -1436,235 +1261,6 @@ __global__ void k_prolong(LevelView fine, LevelView crs, const XferBlock* __rest
   const int gf[3] = {2 * b.clo[0] + i, 2 * b.clo[1] + j, D == 3 ? 2 * b.clo[2] + kk : 0};
   if (gf[0] > 2 * b.chi[0] + 1 || gf[1] > 2 * b.chi[1] + 1 || (D == 3 && gf[2] > 2 * b.chi[2] + 1)) return;
   cell_prolong<T, D>(crs, fine.patches[b.fpatch], crs.patches[b.cpatch], gf, xc, xf, xf2);
-}
-
-// 3-D prolongation of one fine cell whose 2x2x2 coarse stencil leaves the domain: the
-// homogeneous extension enters as per-dimension weights over four inward coarse cells (3/4 on
-// the face cell + 1/4 of the layer-1 ghost formula), a tensor product with the usual pairs.
-template <typename T>
-__device__ __forceinline__ void prolong3d_boundary_cell(const LevelView& crs, const PatchDesc& cp, const PatchDesc& fp,
-                                                        const int gf[3], const T* __restrict__ xc, T* __restrict__ xf,
-                                                        T* __restrict__ xf2) {
-  const T* __restrict__ cb = xc + cp.off;
-  const int csy = (int)cp.sy, csz = (int)cp.sz;
-  int ix[3][4];
-  T wx[3][4];
-  int nx[3];
-#pragma unroll
-  for (int e = 0; e < 3; ++e) {
-    const int par = gf[e] >> 1, sg = (gf[e] & 1) ? 1 : -1;
-    const int lo = e == 0 ? cp.lo[0] : (e == 1 ? cp.lo[1] : cp.lo[2]);
-    const int g2 = par + sg;
-    if (g2 >= 0 && g2 < crs.ndom[e]) {
-      nx[e] = 2;
-#pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        ix[e][m] = par - lo + (m == 1 ? sg : 0);
-        wx[e][m] = m == 0 ? T(0.75) : (m == 1 ? T(0.25) : T(0));
-      }
-    } else {
-      nx[e] = 4;
-      const int side = g2 < 0 ? 0 : 1, type = crs.bc[2 * e + side];
-#pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        ix[e][m] = (side == 0 ? m : crs.ndom[e] - 1 - m) - lo;
-        wx[e][m] = T(0.25) * gcoef<T>(type, 0, m) + (m == 0 ? T(0.75) : T(0));
-      }
-    }
-  }
-  T v = T(0);
-#pragma unroll
-  for (int c2 = 0; c2 < 4; ++c2)
-#pragma unroll
-    for (int c1 = 0; c1 < 4; ++c1)
-#pragma unroll
-      for (int c0 = 0; c0 < 4; ++c0)
-        if (c0 < nx[0] && c1 < nx[1] && c2 < nx[2])
-          v += (wx[0][c0] * wx[1][c1] * wx[2][c2]) *
-               cb[(ix[2][c2] + NG) * csz + (ix[1][c1] + NG) * csy + (ix[0][c0] + NG)];
-  const int of = (gf[2] - fp.lo[2] + NG) * (int)fp.sz + (gf[1] - fp.lo[1] + NG) * (int)fp.sy + (gf[0] - fp.lo[0] + NG);
-  xf[fp.off + of] += v;
-  if (xf2 != nullptr) xf2[fp.off + of] += v;
-}
-
-// 3-D prolongation: += trilinear interpolation of each fine cell's 2x2x2 coarse stencil, read
-// with 32-bit offsets (cells outside the coarse patch are its stored ghost layers);
-// cell_prolong's summation order.  A thread takes PZ fine cells along z (large grids: four,
-// independent loads in flight together).  Fine cells whose stencil leaves the domain (the outermost fine layer at a
-// domain face) are done inline when INLINE (small grids), else skipped and left to
-// k_prolong3d_shell, so that no warp of a large grid carries the boundary arithmetic.
-template <typename T, bool INLINE, int PZ>
-__global__ void __launch_bounds__(BX* BY) k_prolong3d(LevelView fine, LevelView crs, const XferBlock* __restrict__ blocks,
-                                                      int nzc, const T* __restrict__ xc, T* __restrict__ xf,
-                                                      T* __restrict__ xf2) {
-  pdl_wait();
-  const XferBlock b = blocks[blockIdx.z / nzc];
-  const PatchDesc cp = crs.patches[b.cpatch];
-  const PatchDesc fp = fine.patches[b.fpatch];
-#pragma unroll
-  for (int qz = 0; qz < PZ; ++qz) {
-  const int gf[3] = {2 * b.clo[0] + (int)(blockIdx.x * BX + threadIdx.x), 2 * b.clo[1] + (int)(blockIdx.y * BY + threadIdx.y),
-                     2 * b.clo[2] + (int)(blockIdx.z % nzc) * PZ + qz};
-  if (gf[0] > 2 * b.chi[0] + 1 || gf[1] > 2 * b.chi[1] + 1 || gf[2] > 2 * b.chi[2] + 1) continue;
-  int par[3], sg[3];
-  bool inside = true;
-#pragma unroll
-  for (int e = 0; e < 3; ++e) {
-    par[e] = gf[e] >> 1;
-    sg[e] = (gf[e] & 1) ? 1 : -1;
-    inside = inside && par[e] + sg[e] >= 0 && par[e] + sg[e] < crs.ndom[e];
-  }
-  if (!inside) {
-    if (INLINE) prolong3d_boundary_cell<T>(crs, cp, fp, gf, xc, xf, xf2);
-    continue;
-  }
-  const T* __restrict__ cb = xc + cp.off;
-  const int csy = (int)cp.sy, csz = (int)cp.sz;
-  const int oc = (par[2] - cp.lo[2] + NG) * csz + (par[1] - cp.lo[1] + NG) * csy + (par[0] - cp.lo[0] + NG);
-  const int d0 = sg[0], d1 = sg[1] * csy, d2 = sg[2] * csz;
-  T v = T(0);
-#pragma unroll
-  for (int q2 = 0; q2 < 2; ++q2)
-#pragma unroll
-    for (int q1 = 0; q1 < 2; ++q1)
-#pragma unroll
-      for (int q0 = 0; q0 < 2; ++q0) {
-        const T w = ((T(1) * (q0 == 0 ? T(0.75) : T(0.25))) * (q1 == 0 ? T(0.75) : T(0.25))) *
-                    (q2 == 0 ? T(0.75) : T(0.25));
-        v += w * cb[oc + q2 * d2 + q1 * d1 + q0 * d0];
-      }
-  const int of = (gf[2] - fp.lo[2] + NG) * (int)fp.sz + (gf[1] - fp.lo[1] + NG) * (int)fp.sy + (gf[0] - fp.lo[0] + NG);
-  xf[fp.off + of] += v;
-  if (xf2 != nullptr) xf2[fp.off + of] += v;
-  }
-}
-
-// Prolongation of large 3-D grids by coarse parent: one thread per coarse cell reads the 27
-// coarse values around it once (instead of eight per fine cell) and updates its eight
-// children in x pairs (8-byte loads and stores); each child's value is the same sum, in the
-// same order and with the same weights, as in k_prolong3d.  Children in the outermost fine
-// layer at a domain face are left to k_prolong3d_shell, as in k_prolong3d<T, false, PZ>.
-// Block 32 x 8 coarse cells of one plane; grid.z = coarse plane (+ nzc x transfer block).
-template <typename T>
-__global__ void __launch_bounds__(BX* BY) k_prolong3d_par(LevelView fine, LevelView crs,
-                                                          const XferBlock* __restrict__ blocks, int nzc,
-                                                          const T* __restrict__ xc, T* __restrict__ xf,
-                                                          T* __restrict__ xf2) {
-  using V2 = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
-  pdl_wait();
-  const XferBlock b = blocks[blockIdx.z / nzc];
-  const int g[3] = {b.clo[0] + (int)(blockIdx.x * BX + threadIdx.x), b.clo[1] + (int)(blockIdx.y * BY + threadIdx.y),
-                    b.clo[2] + (int)(blockIdx.z % nzc)};
-  if (g[0] > b.chi[0] || g[1] > b.chi[1] || g[2] > b.chi[2]) return;
-  const PatchDesc cp = crs.patches[b.cpatch];
-  const PatchDesc fp = fine.patches[b.fpatch];
-  // children outside the face layers (fine index 0 or 2 n - 1 along a dimension: the shell's)
-  bool keep[3][2];
-#pragma unroll
-  for (int e = 0; e < 3; ++e) {
-    keep[e][0] = g[e] > 0;
-    keep[e][1] = g[e] < crs.ndom[e] - 1;
-  }
-  const bool pairx = keep[0][0] && keep[0][1];
-  const int fsy = (int)fp.sy, fsz = (int)fp.sz;
-  const long long of0 = fp.off + (long long)(2 * g[2] - fp.lo[2] + NG) * fsz + (long long)(2 * g[1] - fp.lo[1] + NG) * fsy +
-                        (2 * g[0] - fp.lo[0] + NG);
-  // the fine pairs first, so that their loads are in flight with the coarse ones
-  V2 fv[2][2];
-#pragma unroll
-  for (int cz = 0; cz < 2; ++cz)
-#pragma unroll
-    for (int cy = 0; cy < 2; ++cy)
-      if (pairx) fv[cz][cy] = *reinterpret_cast<const V2*>(xf + of0 + cz * fsz + cy * fsy);
-  const T* __restrict__ cb = xc + cp.off;
-  const int csy = (int)cp.sy, csz = (int)cp.sz;
-  const int oc = (g[2] - cp.lo[2] + NG) * csz + (g[1] - cp.lo[1] + NG) * csy + (g[0] - cp.lo[0] + NG);
-  T c[3][3][3];  // [dz + 1][dy + 1][dx + 1] (padding cells beyond a face only feed skipped children)
-#pragma unroll
-  for (int dz = 0; dz < 3; ++dz)
-#pragma unroll
-    for (int dy = 0; dy < 3; ++dy)
-#pragma unroll
-      for (int dx = 0; dx < 3; ++dx) c[dz][dy][dx] = __ldg(cb + oc + (dz - 1) * csz + (dy - 1) * csy + (dx - 1));
-#pragma unroll
-  for (int cz = 0; cz < 2; ++cz)
-#pragma unroll
-    for (int cy = 0; cy < 2; ++cy) {
-      if (!keep[2][cz] || !keep[1][cy]) continue;
-      T v[2];
-#pragma unroll
-      for (int cx = 0; cx < 2; ++cx) {
-        const int sx = cx ? 1 : -1, sy = cy ? 1 : -1, sz = cz ? 1 : -1;
-        T a = T(0);
-#pragma unroll
-        for (int q2 = 0; q2 < 2; ++q2)
-#pragma unroll
-          for (int q1 = 0; q1 < 2; ++q1)
-#pragma unroll
-            for (int q0 = 0; q0 < 2; ++q0) {
-              const T w = ((T(1) * (q0 == 0 ? T(0.75) : T(0.25))) * (q1 == 0 ? T(0.75) : T(0.25))) *
-                          (q2 == 0 ? T(0.75) : T(0.25));
-              a += w * c[1 + q2 * sz][1 + q1 * sy][1 + q0 * sx];
-            }
-        v[cx] = a;
-      }
-      const long long of = of0 + cz * fsz + cy * fsy;
-      if (pairx) {
-        V2 t = fv[cz][cy];
-        t.x += v[0];
-        t.y += v[1];
-        *reinterpret_cast<V2*>(xf + of) = t;
-        if (xf2 != nullptr) {
-          V2 u = *reinterpret_cast<const V2*>(xf2 + of);
-          u.x += v[0];
-          u.y += v[1];
-          *reinterpret_cast<V2*>(xf2 + of) = u;
-        }
-      } else {
-#pragma unroll
-        for (int cx = 0; cx < 2; ++cx)
-          if (keep[0][cx]) {
-            xf[of + cx] += v[cx];
-            if (xf2 != nullptr) xf2[of + cx] += v[cx];
-          }
-      }
-    }
-}
-
-// The fine cells k_prolong3d<T, false, PZ> skips: the layer at each domain face a block's fine region
-// touches.  blockIdx.y = face 2d + side; a cell on several faces belongs to the face of its
-// lowest dimension, so face (d, side) covers the cells with index 0 or 2 n - 1 along d,
-// the non-boundary indices along the lower dimensions and every index along the higher ones.
-template <typename T>
-__global__ void __launch_bounds__(256) k_prolong3d_shell(LevelView fine, LevelView crs, const XferBlock* __restrict__ blocks,
-                                                         const T* __restrict__ xc, T* __restrict__ xf, T* __restrict__ xf2) {
-  pdl_wait();
-  const XferBlock b = blocks[blockIdx.z];
-  const int d = blockIdx.y >> 1, side = blockIdx.y & 1;
-  int flo[3], fhi[3], blo[3], bhi[3];  // fine region and its non-boundary part per dimension
-#pragma unroll
-  for (int e = 0; e < 3; ++e) {
-    flo[e] = 2 * b.clo[e];
-    fhi[e] = 2 * b.chi[e] + 1;
-    blo[e] = max(flo[e], 1);
-    bhi[e] = min(fhi[e], 2 * crs.ndom[e] - 2);
-  }
-  const int face = side == 0 ? 0 : 2 * crs.ndom[d] - 1;
-  if (face < flo[d] || face > fhi[d]) return;
-  // the two other dimensions, lower one first
-  const int e1 = d == 0 ? 1 : 0, e2 = d == 2 ? 1 : 2;
-  const int a1 = e1 < d ? blo[e1] : flo[e1], z1 = e1 < d ? bhi[e1] : fhi[e1];
-  const int a2 = e2 < d ? blo[e2] : flo[e2], z2 = e2 < d ? bhi[e2] : fhi[e2];
-  const int n1 = z1 - a1 + 1, n2 = z2 - a2 + 1;
-  if (n1 <= 0 || n2 <= 0) return;
-  const long long cnt = (long long)n1 * n2;
-  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += (long long)gridDim.x * blockDim.x) {
-    int gf[3];
-    gf[d] = face;
-    gf[e1] = a1 + (int)(t % n1);
-    gf[e2] = a2 + (int)(t / n1);
-    prolong3d_boundary_cell<T>(crs, crs.patches[b.cpatch], fine.patches[b.fpatch], gf, xc, xf, xf2);
-  }
 }
 
 // 2-D prolongation, one thread per coarse cell: its four children += linear interpolation
@@ -3523,33 +3119,6 @@ __global__ void k_mean_from_sums(const double* __restrict__ sf, const double* __
                                  double vol, double* __restrict__ m) {
   pdl_wait();
   if (threadIdx.x == 0 && blockIdx.x == 0) m[0] = (sf[0] - (sb ? beta * sb[0] : 0.0)) / vol;
-}
-
-// ------------------------------------------------------------------------ bottom solve
-// x = Minv * b on the coarsest multigrid grid (one block); bordered Neumann systems use the
-// leading n x n block of the inverse of [A 1; 1^T 0] (the constraint right-hand side is 0).
-template <typename T, int D>
-__global__ void k_bottom(const double* __restrict__ minv, int n, int ld, PatchDesc p, const T* __restrict__ b,
-                         T* __restrict__ x, long long cstride) {
-  pdl_wait();
-  p.off += blockIdx.x * cstride;  // stacked component batches: one block per replica
-  extern __shared__ double sb[];
-  for (int t = threadIdx.x; t < n; t += blockDim.x) {
-    const int i = t % p.n[0];
-    const int j = (t / p.n[0]) % p.n[1];
-    const int k = t / (p.n[0] * p.n[1]);
-    sb[t] = (double)b[poff(p, i, j, k)];
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < n; t += blockDim.x) {
-    double acc = 0.0;
-    const double* row = minv + (long long)t * ld;
-    for (int q = 0; q < n; ++q) acc = fma(row[q], sb[q], acc);
-    const int i = t % p.n[0];
-    const int j = (t / p.n[0]) % p.n[1];
-    const int k = t / (p.n[0] * p.n[1]);
-    x[poff(p, i, j, k)] = T(acc);
-  }
 }
 
 }  // namespace amr4

@@ -1,0 +1,349 @@
+// op3d.cuh -- 3-D level operator, residual restriction and prolongation on patches of any size.
+//
+// The multigrid grids below the tile-multiple ones, ragged boxes and levels of several patches
+// are small (1e2 .. 1e6 cells, resident in L2), so a launch lasts as long as one thread's chain
+// of dependent work.  These kernels therefore give every cell (or short z run of cells) its own
+// thread, read the neighbours straight from L1 / L2 with 32-bit offsets, use no shared memory
+// and no barrier, and evaluate the ghost formulas of Eqs. (velBCHomoDiri5th)/(Neumann5) only in
+// the lanes next to a domain face, from four inward cells with the coefficients in registers.
+#pragma once
+
+#include "kernels.cuh"
+
+namespace amr4 {
+
+// Jacobi factors omega / diag by distance class of the cell to the x, y and z faces
+// (face_class; index x + 5 y + 25 z), filled on the host (jacobi_factors).
+template <typename T>
+struct JFac {
+  T w[125];
+};
+
+// Sums of the first and of the second neighbours along one dimension of the cell at offset o,
+// g <= 1 or g >= n - 2 (global index, n cells in the domain): a face cell reads the ghost
+// layers 1 and 2, its neighbour layer 1.  Ghost values in read_nb's order of operations; both
+// sums are commutative, so the low and the high side share one form.
+template <typename T>
+__device__ __forceinline__ void face_sums(const T* __restrict__ xb, int o, int st, int g, int n, int tlo, int thi, T& a1,
+                                          T& a2) {
+  const bool low = g < 2;
+  const int q = low ? g : n - 1 - g;
+  const int s = low ? st : -st;
+  const int t = low ? tlo : thi;
+  const int b = o - q * s;
+  const T c0 = xb[b], c1 = xb[b + s], c2 = xb[b + 2 * s], c3 = xb[b + 3 * s];
+  T g1 = T(0);
+  g1 += gcoef<T>(t, 0, 0) * c0;
+  g1 += gcoef<T>(t, 0, 1) * c1;
+  g1 += gcoef<T>(t, 0, 2) * c2;
+  g1 += gcoef<T>(t, 0, 3) * c3;
+  if (q == 0) {
+    T g2 = T(0);
+    g2 += gcoef<T>(t, 1, 0) * c0;
+    g2 += gcoef<T>(t, 1, 1) * c1;
+    g2 += gcoef<T>(t, 1, 2) * c2;
+    g2 += gcoef<T>(t, 1, 3) * c3;
+    a1 = g1 + c1;
+    a2 = g2 + c2;
+  } else {
+    a1 = c0 + c2;
+    a2 = g1 + c3;
+  }
+}
+
+// neighbour sums along one dimension, class 0: two cells or more from both faces
+template <typename T>
+__device__ __forceinline__ void line_sums(const T* __restrict__ xb, int o, int st, bool inner, int g, int n, int tlo,
+                                          int thi, T& a1, T& a2) {
+  if (inner) {
+    a1 = xb[o - st] + xb[o + st];
+    a2 = xb[o - 2 * st] + xb[o + 2 * st];
+  } else {
+    face_sums<T>(xb, o, st, g, n, tlo, thi, a1, a2);
+  }
+}
+
+// Level operator (OP_APPLY, OP_RESID, OP_JACOBI, OP_JACOBI0; homogeneous data).  A thread owns
+// one (x, y) column of a patch -- columns numbered linearly, so narrow grids fill their warps --
+// and kz planes of it, its z neighbours in a register queue.  The host sizes kz so that small
+// grids spread over every SM (kz = 1 on the coarsest) and large ones keep the queue.
+// Replaces a shared-memory marching kernel with a barrier and 64-bit ghost code per plane, which
+// took 10 us on every FP32 grid down to 6 x 5 x 4 cells and 34 us per FP64 sweep of 72^3.  With
+// the restriction, prolongation and bottom solve below, the FP64 Helmholtz solve on 72^3 + a
+// 56 x 52 x 72 box went from 6.05 to 2.95 ms and the mixed pressure solve on 96 x 80 x 64 with two
+// ragged boxes from 10.1 to 5.8 ms.
+template <typename T, int MODE>
+__global__ void __launch_bounds__(128) k_level_op3d_col(LevelView lv, int kz, const T* __restrict__ x,
+                                                        const T* __restrict__ f, T* __restrict__ out, T alpha, T beta,
+                                                        const __grid_constant__ JFac<T> jf,
+                                                        const unsigned char* __restrict__ vmask) {
+  const int pz = blockIdx.z;
+  const PatchDesc p = lv.npatch == 1 ? lv.p0 : lv.patches[pz];
+  const int col = blockIdx.x * 128 + threadIdx.x;
+  const int k0 = blockIdx.y * kz, k1 = min(k0 + kz, p.n[2]);
+  if (col >= p.n[0] * p.n[1] || k0 >= k1) {
+    pdl_wait();
+    return;
+  }
+  const int i = col % p.n[0], j = col / p.n[0];
+  const int sy = (int)p.sy, sz = (int)p.sz;
+  const int gx = p.lo[0] + i, gy = p.lo[1] + j, lz = p.lo[2], nzd = lv.ndom[2];
+  const int cx = face_class(gx, lv.ndom[0]), cy = face_class(gy, lv.ndom[1]);
+  const T* __restrict__ xb = x + p.off;
+  const T* __restrict__ fb = f + p.off;
+  T* __restrict__ ob = out + p.off;
+  const unsigned char* __restrict__ vb = (MODE == OP_RESID && vmask != nullptr) ? vmask + p.off : nullptr;
+  int o = (k0 + NG) * sz + (j + NG) * sy + i + NG;
+  pdl_wait();
+  if (MODE == OP_JACOBI0) {
+    for (int k = k0; k < k1; ++k, o += sz) ob[o] = jf.w[cx + 5 * cy + 25 * face_class(lz + k, nzd)] * fb[o];
+    return;
+  }
+  const T inv = pick<T>(lv.inv12h2, lv.inv12h2_f);
+  const T kc2 = beta * inv, kc1 = T(16) * kc2, kc0 = alpha - T(90) * kc2;
+  T q0, q1, q2, q3;
+  q2 = xb[o];
+  q3 = (lz + k0 + 1 < nzd) ? xb[o + sz] : T(0);
+  q0 = (lz + k0 - 2 >= 0) ? xb[o - 2 * sz] : T(0);
+  q1 = (lz + k0 - 1 >= 0) ? xb[o - sz] : T(0);
+#pragma unroll 2
+  for (int k = k0; k < k1; ++k, o += sz) {
+    const int gz = lz + k;
+    const int cz = face_class(gz, nzd);
+    const T q4 = (gz + 2 < nzd) ? xb[o + 2 * sz] : T(0);
+    T fk = T(0);
+    if (MODE != OP_APPLY) fk = fb[o];
+    T x1, x2, y1, y2, z1, z2;
+    line_sums<T>(xb, o, 1, cx == 0, gx, lv.ndom[0], lv.bc[0], lv.bc[1], x1, x2);
+    line_sums<T>(xb, o, sy, cy == 0, gy, lv.ndom[1], lv.bc[2], lv.bc[3], y1, y2);
+    if (cz == 0) {
+      z1 = q1 + q3;
+      z2 = q0 + q4;
+    } else {
+      face_sums<T>(xb, o, sz, gz, nzd, lv.bc[4], lv.bc[5], z1, z2);
+    }
+    const T s1 = (x1 + y1) + z1;
+    const T s2 = (x2 + y2) + z2;
+    if (vb == nullptr || vb[o]) {
+      if (MODE == OP_APPLY) {
+        ob[o] = kc0 * q2 + (kc1 * s1 - kc2 * s2);
+      } else {
+        const T r = fma(kc2, s2, fma(-kc1, s1, fma(-kc0, q2, fk)));
+        if (MODE == OP_RESID) ob[o] = r;
+        else ob[o] = fma(jf.w[cx + 5 * cy + 25 * cz], r, q2);
+      }
+    }
+    q0 = q1;
+    q1 = q2;
+    q2 = q3;
+    q3 = q4;
+  }
+}
+
+// Residual restriction: eight lanes per coarse cell, one per child, instead of one thread for
+// all eight (the chain of 8 x 13 loads took 15 us on every grid, 53 us in FP64 on a 72^3 one).
+// Each lane forms its child's residual with cell_Lx's arithmetic; lane 0's sum adds them in
+// cell_restrict's order, so the result is bit for bit the one-thread form's.  A warp holds
+// four coarse cells along x: the loads of a row of eight children are contiguous.
+template <typename T>
+__global__ void __launch_bounds__(256) k_restrict3d_resid(LevelView fine, LevelView crs,
+                                                          const XferBlock* __restrict__ blocks,
+                                                          const T* __restrict__ xf, const T* __restrict__ ff,
+                                                          T* __restrict__ outc, T alpha, T beta) {
+  pdl_wait();
+  const XferBlock b = blocks[blockIdx.z];
+  const int w0 = b.chi[0] - b.clo[0] + 1, w1 = b.chi[1] - b.clo[1] + 1, w2 = b.chi[2] - b.clo[2] + 1;
+  const int lane = threadIdx.x & 31, child = lane & 7;
+  // coarse cells of a warp: four along x (the last group of a row may be short)
+  const int gw = (w0 + 3) / 4;
+  const int grp = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (grp >= gw * w1 * w2) return;
+  const int ci = (grp % gw) * 4 + (lane >> 3), cj = (grp / gw) % w1, ck = grp / (gw * w1);
+  const bool act = ci < w0;
+  const PatchDesc cp = crs.patches[b.cpatch];
+  const PatchDesc fp = fine.patches[b.fpatch];
+  const int g0 = b.clo[0] + ci, g1 = b.clo[1] + cj, g2 = b.clo[2] + ck;
+  T r = T(0);
+  if (act) {
+    const int sy = (int)fp.sy, sz = (int)fp.sz;
+    const int fx = 2 * g0 + (child & 1), fy = 2 * g1 + ((child >> 1) & 1), fz = 2 * g2 + (child >> 2);
+    const int o = (fz - fp.lo[2] + NG) * sz + (fy - fp.lo[1] + NG) * sy + (fx - fp.lo[0] + NG);
+    const T* __restrict__ xb = xf + fp.off;
+    const T fk = ff[fp.off + o], xc = xb[o];
+    const int n0 = fine.ndom[0], n1 = fine.ndom[1], n2 = fine.ndom[2];
+    T x1, x2, y1, y2, z1, z2;
+    line_sums<T>(xb, o, 1, face_class(fx, n0) == 0, fx, n0, fine.bc[0], fine.bc[1], x1, x2);
+    line_sums<T>(xb, o, sy, face_class(fy, n1) == 0, fy, n1, fine.bc[2], fine.bc[3], y1, y2);
+    line_sums<T>(xb, o, sz, face_class(fz, n2) == 0, fz, n2, fine.bc[4], fine.bc[5], z1, z2);
+    const T s1 = (x1 + y1) + z1, s2 = (x2 + y2) + z2;
+    const T inv = pick<T>(fine.inv12h2, fine.inv12h2_f);
+    const T s = (T(16) * s1 - s2 - T(90) * xc) + T(0);
+    r = fk - (alpha * xc + beta * (s * inv));
+  }
+  T acc = T(0);
+#pragma unroll
+  for (int c = 0; c < 8; ++c) acc += __shfl_sync(0xffffffffu, r, (lane & 24) + c);
+  if (act && child == 0)
+    outc[cp.off + (long long)(g2 - cp.lo[2] + NG) * cp.sz + (long long)(g1 - cp.lo[1] + NG) * cp.sy + (g0 - cp.lo[0] + NG)] =
+        acc * T(0.125);
+}
+
+// Prolongation by coarse parent on any grid: one thread per coarse cell gathers the 27 coarse
+// values around it, with the homogeneous layer-1 extension where the neighbourhood leaves the
+// domain (dimension after dimension, Fig. 1(c); four inward cells per dimension instead of
+// three), and updates its eight children, whose sums are k_prolong3d's in order and weights.
+// Replaces one thread per fine cell with the face cells' 64-term products inline: 143 us for
+// an FP64 72^3 grid, 45 us for 36^3.
+template <typename T>
+__device__ __forceinline__ void ext_row(const T* __restrict__ cb, int o, int st, bool lo, bool hi, const T* __restrict__ glo,
+                                        const T* __restrict__ ghi, T& a, T& b, T& c) {
+  b = cb[o];
+  if (!lo) a = cb[o - st];
+  if (!hi) c = cb[o + st];
+  if (lo) a = fma(glo[3], cb[o + 3 * st], fma(glo[2], cb[o + 2 * st], fma(glo[1], c, glo[0] * b)));
+  if (hi) c = fma(ghi[3], cb[o - 3 * st], fma(ghi[2], cb[o - 2 * st], fma(ghi[1], a, ghi[0] * b)));
+}
+
+template <typename T>
+__global__ void __launch_bounds__(128) k_prolong3d_ext(LevelView fine, LevelView crs, const XferBlock* __restrict__ blocks,
+                                                       const T* __restrict__ xc, T* __restrict__ xf, T* __restrict__ xf2) {
+  using V2 = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
+  pdl_wait();
+  const XferBlock b = blocks[blockIdx.z];
+  const int w0 = b.chi[0] - b.clo[0] + 1, w1 = b.chi[1] - b.clo[1] + 1;
+  const int col = blockIdx.x * 128 + threadIdx.x;
+  const int g2 = b.clo[2] + (int)blockIdx.y;
+  if (col >= w0 * w1 || g2 > b.chi[2]) return;
+  const int g0 = b.clo[0] + col % w0, g1 = b.clo[1] + col / w0;
+  const PatchDesc cp = crs.patches[b.cpatch];
+  const PatchDesc fp = fine.patches[b.fpatch];
+  const int fsy = (int)fp.sy, fsz = (int)fp.sz;
+  const long long of = fp.off + (long long)(2 * g2 - fp.lo[2] + NG) * fsz + (long long)(2 * g1 - fp.lo[1] + NG) * fsy +
+                       (2 * g0 - fp.lo[0] + NG);
+  V2 fv[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) fv[q] = *reinterpret_cast<const V2*>(xf + of + (q >> 1) * fsz + (q & 1) * fsy);
+  const T* __restrict__ cb = xc + cp.off;
+  const int csy = (int)cp.sy, csz = (int)cp.sz;
+  const int oc = (g2 - cp.lo[2] + NG) * csz + (g1 - cp.lo[1] + NG) * csy + (g0 - cp.lo[0] + NG);
+  const bool xl = g0 == 0, xh = g0 == crs.ndom[0] - 1, yl = g1 == 0, yh = g1 == crs.ndom[1] - 1, zl = g2 == 0,
+             zh = g2 == crs.ndom[2] - 1;
+  T c[3][3][3];  // [dz + 1][dy + 1][dx + 1]
+  if (!(xl || xh || yl || yh || zl || zh)) {
+#pragma unroll
+    for (int dz = 0; dz < 3; ++dz)
+#pragma unroll
+      for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) c[dz][dy][dx] = cb[oc + (dz - 1) * csz + (dy - 1) * csy + (dx - 1)];
+  } else {
+    // layer-1 ghost coefficients of the two faces of each dimension
+    T gx[2][4], gy[2][4], gz[2][4];
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        gx[s][m] = gcoef<T>(crs.bc[s], 0, m);
+        gy[s][m] = gcoef<T>(crs.bc[2 + s], 0, m);
+        gz[s][m] = gcoef<T>(crs.bc[4 + s], 0, m);
+      }
+    // one plane: its three rows (extended in x), the outer ones extended in y
+    auto plane = [&](int op, T pl[3][3]) {
+      ext_row<T>(cb, op, 1, xl, xh, gx[0], gx[1], pl[1][0], pl[1][1], pl[1][2]);
+      if (!yl) ext_row<T>(cb, op - csy, 1, xl, xh, gx[0], gx[1], pl[0][0], pl[0][1], pl[0][2]);
+      if (!yh) ext_row<T>(cb, op + csy, 1, xl, xh, gx[0], gx[1], pl[2][0], pl[2][1], pl[2][2]);
+      if (yl || yh) {
+        const int d = yl ? csy : -csy;
+        const T h0 = yl ? gy[0][0] : gy[1][0], h1 = yl ? gy[0][1] : gy[1][1], h2 = yl ? gy[0][2] : gy[1][2],
+                h3 = yl ? gy[0][3] : gy[1][3];
+        T r2[3], r3[3];
+        ext_row<T>(cb, op + 2 * d, 1, xl, xh, gx[0], gx[1], r2[0], r2[1], r2[2]);
+        ext_row<T>(cb, op + 3 * d, 1, xl, xh, gx[0], gx[1], r3[0], r3[1], r3[2]);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          const T fr = yl ? pl[2][q] : pl[0][q];
+          const T v = fma(h3, r3[q], fma(h2, r2[q], fma(h1, fr, h0 * pl[1][q])));
+          if (yl) pl[0][q] = v;
+          else pl[2][q] = v;
+        }
+      }
+    };
+    plane(oc, c[1]);
+    if (!zl) plane(oc - csz, c[0]);
+    if (!zh) plane(oc + csz, c[2]);
+    if (zl || zh) {
+      const int d = zl ? csz : -csz;
+      T p2[3][3], p3[3][3];
+      plane(oc + 2 * d, p2);
+      plane(oc + 3 * d, p3);
+      const T h0 = zl ? gz[0][0] : gz[1][0], h1 = zl ? gz[0][1] : gz[1][1], h2 = zl ? gz[0][2] : gz[1][2],
+              h3 = zl ? gz[0][3] : gz[1][3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          const T fr = zl ? c[2][a][q] : c[0][a][q];
+          const T v = fma(h3, p3[a][q], fma(h2, p2[a][q], fma(h1, fr, h0 * c[1][a][q])));
+          if (zl) c[0][a][q] = v;
+          else c[2][a][q] = v;
+        }
+    }
+  }
+#pragma unroll
+  for (int cz = 0; cz < 2; ++cz)
+#pragma unroll
+    for (int cy = 0; cy < 2; ++cy) {
+      T v[2];
+#pragma unroll
+      for (int cx = 0; cx < 2; ++cx) {
+        const int sx = cx ? 1 : -1, sy = cy ? 1 : -1, sz = cz ? 1 : -1;
+        T a = T(0);
+#pragma unroll
+        for (int q2 = 0; q2 < 2; ++q2)
+#pragma unroll
+          for (int q1 = 0; q1 < 2; ++q1)
+#pragma unroll
+            for (int q0 = 0; q0 < 2; ++q0) {
+              const T w = ((T(1) * (q0 == 0 ? T(0.75) : T(0.25))) * (q1 == 0 ? T(0.75) : T(0.25))) *
+                          (q2 == 0 ? T(0.75) : T(0.25));
+              a += w * c[1 + q2 * sz][1 + q1 * sy][1 + q0 * sx];
+            }
+        v[cx] = a;
+      }
+      const long long oo = of + cz * fsz + cy * fsy;
+      V2 t = fv[2 * cz + cy];
+      t.x += v[0];
+      t.y += v[1];
+      *reinterpret_cast<V2*>(xf + oo) = t;
+      if (xf2 != nullptr) {
+        V2 u = *reinterpret_cast<const V2*>(xf2 + oo);
+        u.x += v[0];
+        u.y += v[1];
+        *reinterpret_cast<V2*>(xf2 + oo) = u;
+      }
+    }
+}
+
+// Bottom solve x = Minv b with one warp per row (the bordered Neumann systems use the leading
+// n x n block).  One block for all rows read the 4 MB inverse of a 729-cell bottom grid through
+// one SM: 279 us; spread over the chip it is one L2 read of the inverse.
+template <typename T>
+__global__ void __launch_bounds__(128) k_bottom_rows(const double* __restrict__ minv, int n, int ld, PatchDesc p,
+                                                     const T* __restrict__ b, T* __restrict__ x, long long cstride) {
+  const int row = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  p.off += blockIdx.y * cstride;  // stacked component batches: one grid row per replica
+  pdl_wait();
+  if (row >= n) return;
+  auto at = [&](int t) -> long long {
+    const int i = t % p.n[0], jk = t / p.n[0];
+    return p.off + (long long)(i + NG) + (long long)(jk % p.n[1] + NG) * p.sy +
+           (p.sz ? (long long)(jk / p.n[1] + NG) * p.sz : 0ll);
+  };
+  const double* __restrict__ m = minv + (long long)row * ld;
+  double acc = 0.0;
+  for (int q = lane; q < n; q += 32) acc = fma(m[q], (double)b[at(q)], acc);
+  for (int s = 16; s > 0; s >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
+  if (lane == 0) x[at(row)] = T(acc);
+}
+
+}  // namespace amr4

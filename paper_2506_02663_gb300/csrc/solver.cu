@@ -18,6 +18,7 @@
 
 #include "amr4_impl.h"
 #include "kernels.cuh"
+#include "op3d.cuh"
 #include "sweep3d.cuh"
 #include "coarse3d.cuh"
 #include "cic.cuh"
@@ -594,6 +595,43 @@ amr_status launch_resid_fx(const LevelView& lv, const double* x, const double* f
   return launch_check();
 }
 
+// Jacobi factors omega / diag by distance class (k_level_op3d_zc's device table, same order)
+template <typename T>
+JFac<T> jacobi_factors(const LevelView& lv, double alpha, double beta, double omega) {
+  JFac<T> j;
+  const T inv = pick_host<T>(lv.inv12h2, lv.inv12h2_f);
+  for (int q = 0; q < 125; ++q) {
+    const int cls[3] = {q % 5, (q / 5) % 5, q / 25};
+    T acc = T(-90);
+    for (int d = 0; d < 3; ++d)
+      if (cls[d]) acc += pick_host<T>(lv.dcorr[2 * d + (cls[d] - 1) / 2][(cls[d] - 1) % 2],
+                                      lv.dcorr_f[2 * d + (cls[d] - 1) / 2][(cls[d] - 1) % 2]);
+    j.w[q] = T(omega) / (T(alpha) + T(beta) * inv * acc);
+  }
+  return j;
+}
+
+// SMs of the current device, queried once per device
+inline int sm_count() {
+  static std::atomic<int> nsm[64];
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= 64) return 152;
+  int m = nsm[dev].load(std::memory_order_relaxed);
+  if (m == 0) {
+    cudaDeviceGetAttribute(&m, cudaDevAttrMultiProcessorCount, dev);
+    m = std::max(1, m);
+    nsm[dev].store(m, std::memory_order_relaxed);
+  }
+  return m;
+}
+
+// padded patches of fewer than 2^31 elements (32-bit offsets inside a patch)
+inline bool small_offsets(const LevelView& lv) {
+  const long long px = ((lv.maxn[0] + 2 * NG) + 3) / 4 * 4;
+  return px * (lv.maxn[1] + 2 * NG) * (lv.D == 3 ? lv.maxn[2] + 2 * NG : 1) < (1LL << 31);
+}
+
 template <typename T, int D, bool TR = false>
 amr_status level_op(int mode, const LevelView& lv, const T* x, const T* f, T* out, const T* bc, double alpha,
                     double beta, double omega, const unsigned char* vmask, cudaStream_t st) {
@@ -671,26 +709,29 @@ amr_status level_op(int mode, const LevelView& lv, const T* x, const T* f, T* ou
              nb * sizeof(T) * lv.ncells, lv.ncells);
     return launch_check();
   }
-  if (D == 3 && !TR && bc == nullptr) {
-    // z-marching 3-D path (homogeneous physical data)
-    const int tx = (lv.maxn[0] + MZ_TX - 1) / MZ_TX, ty = (lv.maxn[1] + MZ_TY - 1) / MZ_TY;
-    const int nz = lv.maxn[2];
-    int nzc = std::max(1, std::min((2048 + tx * ty - 1) / (tx * ty), std::max(1, nz / 4)));
-    const int kz = (nz + nzc - 1) / nzc;
-    nzc = (nz + kz - 1) / kz;
-    dim3 grid(tx, ty, nzc * lv.npatch);
-    dim3 block(MZ_TX, MZ_TY, 1);
-    const T A = T(alpha), B = T(beta), O = T(omega);
-    switch (mode) {
-      case OP_APPLY: launch(k_level_op3d_march<T, OP_APPLY>, grid, block, 0, st, lv, nzc, kz, x, f, out, A, B, O, vmask); break;
-      case OP_RESID: launch(k_level_op3d_march<T, OP_RESID>, grid, block, 0, st, lv, nzc, kz, x, f, out, A, B, O, vmask); break;
-      case OP_JACOBI: launch(k_level_op3d_march<T, OP_JACOBI>, grid, block, 0, st, lv, nzc, kz, x, f, out, A, B, O, vmask); break;
-      default: launch(k_level_op3d_march<T, OP_JACOBI0>, grid, block, 0, st, lv, nzc, kz, x, f, out, A, B, O, vmask);
+  if constexpr (D == 3 && !TR) {
+    if (bc == nullptr && small_offsets(lv)) {
+      // any other homogeneous 3-D level: one thread per column and run of kz planes, as many runs
+      // as give every SM 16 warps (a quarter of its slots: enough loads in flight for L2, and long
+      // runs where the grid allows them)
+      const long long warps = (long long)lv.npatch * ((lv.maxn[0] * (long long)lv.maxn[1] + 31) / 32);
+      const long long want = 16LL * sm_count();
+      const int nz = lv.maxn[2];
+      const int kz = (int)std::max<long long>(1, std::min<long long>(nz, (warps * nz + want - 1) / want));
+      const dim3 grid((unsigned)((lv.maxn[0] * (long long)lv.maxn[1] + 127) / 128), (nz + kz - 1) / kz, lv.npatch);
+      const JFac<T> jf = (mode == OP_JACOBI || mode == OP_JACOBI0) ? jacobi_factors<T>(lv, alpha, beta, omega) : JFac<T>{};
+      const T A = T(alpha), B = T(beta);
+      switch (mode) {
+        case OP_APPLY: launch(k_level_op3d_col<T, OP_APPLY>, grid, 128, 0, st, lv, kz, x, f, out, A, B, jf, vmask); break;
+        case OP_RESID: launch(k_level_op3d_col<T, OP_RESID>, grid, 128, 0, st, lv, kz, x, f, out, A, B, jf, vmask); break;
+        case OP_JACOBI: launch(k_level_op3d_col<T, OP_JACOBI>, grid, 128, 0, st, lv, kz, x, f, out, A, B, jf, vmask); break;
+        default: launch(k_level_op3d_col<T, OP_JACOBI0>, grid, 128, 0, st, lv, kz, x, f, out, A, B, jf, vmask);
+      }
+      const double nb = mode == OP_JACOBI0 ? 2.0 : (mode == OP_APPLY ? 2.0 : 3.0);
+      prof_end(st, ev, (mode == OP_JACOBI || mode == OP_JACOBI0) ? PC_JACOBI : (mode == OP_RESID && sizeof(T) == 8) ? PC_RESID64 : PC_RESID,
+               nb * sizeof(T) * lv.ncells, lv.ncells);
+      return launch_check();
     }
-    const double nb = mode == OP_JACOBI0 ? 2.0 : (mode == OP_APPLY ? 2.0 : 3.0);
-    prof_end(st, ev, (mode == OP_JACOBI || mode == OP_JACOBI0) ? PC_JACOBI : (mode == OP_RESID && sizeof(T) == 8) ? PC_RESID64 : PC_RESID,
-             nb * sizeof(T) * lv.ncells, lv.ncells);
-    return launch_check();
   }
   switch (mode) {
     case OP_APPLY:
@@ -725,7 +766,11 @@ amr_status restrict_blocks(const LevelView& fine, const LevelView& crs, const Xf
   prof_begin(st, &ev);
   if (resid && D == 2)
     launch(k_restrict2d_resid<T, TR>, grid, block, 0, st, fine, crs, blocks, xf, ff, outc, T(alpha), T(beta));
-  else if (resid)
+  else if (D == 3 && resid && !TR && small_offsets(fine)) {
+    const long long groups = (long long)((xmax[0] + 3) / 4) * xmax[1] * xmax[2];  // warps of four coarse cells
+    launch(k_restrict3d_resid<T>, dim3((unsigned)((groups + 7) / 8), 1, nblocks), 256, 0, st, fine, crs, blocks, xf, ff,
+           outc, T(alpha), T(beta));
+  } else if (resid)
     launch(k_restrict<T, D, true, TR>, grid, block, 0, st, fine, crs, blocks, xf, ff, outc, T(alpha), T(beta), nby);
   else
     launch(k_restrict<T, D, false>, grid, block, 0, st, fine, crs, blocks, xf, ff, outc, T(alpha), T(beta), nby);
@@ -744,27 +789,10 @@ amr_status prolong_blocks(const LevelView& fine, const LevelView& crs, const Xfe
     dim3 grid((xmax[0] + BX - 1) / BX, (xmax[1] + BY - 1) / BY, nblocks);
     launch(k_prolong2d<T>, grid, dim3(BX, BY, 1), 0, st, fine, crs, blocks, xc, xf, xf2);
   } else {
-    // 32-bit offsets inside the padded patches (a 3-D patch beyond 2^31 elements takes the
-    // generic kernel)
-    const long long fel = (long long)(fine.maxn[0] + 2 * NG + 3) * (fine.maxn[1] + 2 * NG) * (fine.maxn[2] + 2 * NG);
-    // large grids: four fine cells per thread along z, the face layer in its own launch (a few
-    // blocks per face); small grids: one cell per thread with the face cells inline
-    const bool large = (long long)xmax[0] * xmax[1] * xmax[2] >= 64LL * 64 * 64;
-    const int pz = large ? 4 : 1;
-    const int nzc = (2 * xmax[2] + pz - 1) / pz;
-    if (fel < (1LL << 31) && (long long)nzc * nblocks <= 65535) {
-      dim3 grid((2 * xmax[0] + BX - 1) / BX, (2 * xmax[1] + BY - 1) / BY, nzc * nblocks);
-      if (large) {
-        // by coarse parent (32 x 8 coarse cells a block, one coarse plane), the face layer by the shell
-        dim3 pgrid((xmax[0] + BX - 1) / BX, (xmax[1] + BY - 1) / BY, xmax[2] * nblocks);
-        launch(k_prolong3d_par<T>, pgrid, dim3(BX, BY, 1), 0, st, fine, crs, blocks, xmax[2], xc, xf, xf2);
-        if (const amr_status s1 = launch_check(); s1 != AMR_OK) return s1;
-        const long long face = 4LL * std::max({xmax[0] * xmax[1], xmax[1] * xmax[2], xmax[0] * xmax[2]});
-        const unsigned gx = (unsigned)std::min<long long>((face + 255) / 256, 64);
-        launch(k_prolong3d_shell<T>, dim3(gx, 6, nblocks), 256, 0, st, fine, crs, blocks, xc, xf, xf2);
-      } else {
-        launch(k_prolong3d<T, true, 1>, grid, dim3(BX, BY, 1), 0, st, fine, crs, blocks, nzc, xc, xf, xf2);
-      }
+    // a 3-D patch beyond 2^31 elements takes the generic kernel
+    if (small_offsets(fine) && xmax[2] <= 65535) {
+      dim3 grid((unsigned)(((long long)xmax[0] * xmax[1] + 127) / 128), xmax[2], nblocks);
+      launch(k_prolong3d_ext<T>, grid, 128, 0, st, fine, crs, blocks, xc, xf, xf2);
     } else {
       const int fy = 2 * xmax[1];
       const int nby = (fy + BY - 1) / BY;
@@ -1477,7 +1505,7 @@ amr_status mg_level0(amr_operator* op, const amr_solver_params& p, int m, const 
   }
   if (m == M) {
     const int n = op->nbot;
-    launch(k_bottom<T, D>, h->ncomp, 256, n * sizeof(double), st, TR ? op->d_binvT : op->d_binv, n, op->ldb,
+    launch(k_bottom_rows<T>, dim3((n + 3) / 4, h->ncomp, 1), 128, 0, st, TR ? op->d_binvT : op->d_binv, n, op->ldb,
            h->mg[m].patch, b, x, h->mg[m].cstride);
     return launch_check();
   }
@@ -2227,16 +2255,7 @@ amr_status solve_impl(amr_operator* op, const amr_solver_params& p, double* phi,
 // grid of the whole-array passes: grid-stride, a few blocks per SM
 // grid-stride element-wise kernels: one block per 256 elements, at most 8 per SM
 inline unsigned flat_blocks(long long n) {
-  static int nsm[64] = {0};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  int m = (dev >= 0 && dev < 64) ? nsm[dev] : 0;
-  if (m == 0) {
-    cudaDeviceGetAttribute(&m, cudaDevAttrMultiProcessorCount, dev);
-    m = std::max(1, m);
-    if (dev >= 0 && dev < 64) nsm[dev] = m;
-  }
-  return (unsigned)std::min<long long>((n + 255) / 256, 8LL * m);
+  return (unsigned)std::min<long long>((n + 255) / 256, 8LL * sm_count());
 }
 
 // elements of one replica of a stacked component batch (the whole array otherwise)
