@@ -1795,7 +1795,7 @@ __global__ void __launch_bounds__(NT) k_amr_post2d(LevelView lv, PatchDesc gp, i
     const T v = cur[(tj + j + NG) * sy + ti + i + NG];
     const int og = (tg.j0 + j + NG) * gsy + tg.i0 + i + NG;
     eg[og] += v;
-    xg[og] += v;
+    if (x != nullptr) xg[og] += v;
   });
 }
 

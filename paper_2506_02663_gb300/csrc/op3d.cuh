@@ -140,6 +140,95 @@ __global__ void __launch_bounds__(128) k_level_op3d_col(LevelView lv, int kz, co
   }
 }
 
+// ------------------------------------------------------------------------ level 0 around the refined region
+// In a composite V-cycle the correction on level 0 is zero before the level-0 multigrid except
+// under the level-1 boxes, where it is the average of the fine correction.  The level-0
+// residual r - A x then equals r outside the boxes grown by three cells (two for the stencil,
+// one more because a ghost formula reaches four cells inward).  These passes visit only that
+// region (70^3 of 256^3 cells on the benchmark's hierarchy) instead of whole fields, of which the
+// level-0 residual alone took 55 us.
+constexpr int RGN_RESID = 3;  // cells around a box where the residual differs from r
+constexpr int RGN_READ = 5;   // cells around a box that the residual or the AMRCFI windows read
+
+// cell of region t of transfer block b grown by ``grow`` cells, clipped to the domain
+template <int D>
+__device__ __forceinline__ bool region_cell(const LevelView& lv, const XferBlock& b, int grow, long long t, int g[3]) {
+  int lo[3] = {0, 0, 0}, w[3] = {1, 1, 1};
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    lo[d] = max(b.clo[d] - grow, 0);
+    w[d] = min(b.chi[d] + grow, lv.ndom[d] - 1) - lo[d] + 1;
+  }
+  if (t >= (long long)w[0] * w[1] * w[2]) return false;
+  const unsigned u = (unsigned)t;
+  g[0] = lo[0] + (int)(u % w[0]);
+  g[1] = lo[1] + (int)((u / w[0]) % w[1]);
+  g[2] = lo[2] + (int)(u / ((unsigned)w[0] * w[1]));
+  return true;
+}
+
+// x = 0 and keep = r on the regions grown by RGN_READ (r may be overwritten there afterwards;
+// idempotent where regions overlap)
+template <typename T, int D>
+__global__ void __launch_bounds__(256) k_region_begin(LevelView lv, const XferBlock* __restrict__ blocks,
+                                                      const T* __restrict__ r, T* __restrict__ x, T* __restrict__ keep) {
+  pdl_wait();
+  const XferBlock b = blocks[blockIdx.y];
+  int g[3];
+  if (!region_cell<D>(lv, b, RGN_READ, (long long)blockIdx.x * 256 + threadIdx.x, g)) return;
+  const PatchDesc p = lv.npatch == 1 ? lv.p0 : lv.patches[b.cpatch];
+  const long long o = poff(p, g[0] - p.lo[0], g[1] - p.lo[1], D == 3 ? g[2] - p.lo[2] : 0);
+  x[o] = T(0);
+  keep[o] = r[o];
+}
+
+// r = keep - A x on the valid cells of the regions grown by RGN_RESID
+template <typename T, int D>
+__global__ void __launch_bounds__(256) k_region_resid(LevelView lv, const XferBlock* __restrict__ blocks,
+                                                      const T* __restrict__ x, const T* __restrict__ keep,
+                                                      T* __restrict__ r, const unsigned char* __restrict__ vmask, T alpha,
+                                                      T beta) {
+  pdl_wait();
+  const XferBlock b = blocks[blockIdx.y];
+  int g[3];
+  if (!region_cell<D>(lv, b, RGN_RESID, (long long)blockIdx.x * 256 + threadIdx.x, g)) return;
+  const PatchDesc p = lv.npatch == 1 ? lv.p0 : lv.patches[b.cpatch];
+  const long long og = poff(p, g[0] - p.lo[0], g[1] - p.lo[1], D == 3 ? g[2] - p.lo[2] : 0);
+  if (!vmask[og]) return;
+  const T* __restrict__ xb = x + p.off;
+  const int o = (int)(og - p.off);
+  const T inv = pick<T>(lv.inv12h2, lv.inv12h2_f);
+  const T kc2 = beta * inv, kc1 = T(16) * kc2, kc0 = alpha - T(30 * D) * kc2;
+  T a1, a2, s1 = T(0), s2 = T(0);
+  line_sums<T>(xb, o, 1, face_class(g[0], lv.ndom[0]) == 0, g[0], lv.ndom[0], lv.bc[0], lv.bc[1], a1, a2);
+  s1 += a1;
+  s2 += a2;
+  line_sums<T>(xb, o, (int)p.sy, face_class(g[1], lv.ndom[1]) == 0, g[1], lv.ndom[1], lv.bc[2], lv.bc[3], a1, a2);
+  s1 += a1;
+  s2 += a2;
+  if (D == 3) {
+    line_sums<T>(xb, o, (int)p.sz, face_class(g[2], lv.ndom[2]) == 0, g[2], lv.ndom[2], lv.bc[4], lv.bc[5], a1, a2);
+    s1 += a1;
+    s2 += a2;
+  }
+  r[og] = fma(kc2, s2, fma(-kc1, s1, fma(-kc0, xb[o], keep[og])));
+}
+
+// copy (add = 0) or add (add = 1) src into dst on the regions grown by ``grow``; adding is
+// done on the boxes themselves only (grow = 0: disjoint)
+template <typename T, int D>
+__global__ void __launch_bounds__(256) k_region_move(LevelView lv, const XferBlock* __restrict__ blocks, int grow,
+                                                     const T* __restrict__ src, T* __restrict__ dst, int add) {
+  pdl_wait();
+  const XferBlock b = blocks[blockIdx.y];
+  int g[3];
+  if (!region_cell<D>(lv, b, grow, (long long)blockIdx.x * 256 + threadIdx.x, g)) return;
+  const PatchDesc p = lv.npatch == 1 ? lv.p0 : lv.patches[b.cpatch];
+  const long long o = poff(p, g[0] - p.lo[0], g[1] - p.lo[1], D == 3 ? g[2] - p.lo[2] : 0);
+  if (add) dst[o] += src[o];
+  else dst[o] = src[o];
+}
+
 // Residual restriction: eight lanes per coarse cell, one per child, instead of one thread for
 // all eight (the chain of 8 x 13 loads took 15 us on every grid, 53 us in FP64 on a 72^3 one).
 // Each lane forms its child's residual with cell_Lx's arithmetic; lane 0's sum adds them in

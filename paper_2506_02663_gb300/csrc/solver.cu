@@ -1770,6 +1770,20 @@ amr_status vcycle_corr_T(amr_operator* op, const amr_solver_params& p, const T* 
   return AMR_OK;
 }
 
+// Restriction of a single-patch fine level's residual over its single-patch coarse level by the
+// bulk-copy kernel (the arithmetic of k_restrict3d_resid).
+template <typename T>
+amr_status bulk_restrict_level(const LevelView& fine, const LevelView& crs, const T* x, const T* f, T* outc, double alpha,
+                               double beta, cudaStream_t st) {
+  cudaEvent_t ev;
+  prof_begin(st, &ev);
+  TRY((launch_sw<T, OP_RESTRICT>(fine, x, f, (T*)nullptr, T(alpha), T(beta), T(0), nullptr, st, nullptr, outc, &crs.p0,
+                                 crs.cstride)));
+  const double cc = fine.ncells / 8.0;
+  prof_end(st, ev, PC_RESTRICT, (2.0 * 8 + 1.0) * sizeof(T) * cc, cc * 8);
+  return AMR_OK;
+}
+
 // ---------------------------------------------------------------- composite V-cycle
 // Correction form: given the composite residual r (covered cells), S.X receives the
 // V-cycle's approximation of A^{-1} r (homogeneous data).
@@ -1789,30 +1803,60 @@ bool blocked_amr_level(const amr_operator* op, const amr_solver_params& p, int l
   return true;
 }
 
+// What happens to the V-cycle's input and to the covered cells of its output:
+//   VC_SCRATCH_R  the level-0 part of r may be overwritten (the caller recomputes it)
+//   VC_COVERED    S.X is also wanted on level-0 cells under the level-1 boxes
+enum { VC_SCRATCH_R = 1, VC_COVERED = 2 };
+
+// S.X doubles as the finest level's correction E_L and as level 0's E_0 (valid cells: X = E
+// on every level), so neither is accumulated separately; the whole-field passes that did so
+// (four memsets, a copy of r, the level-0 residual, E -> X) took 180 us of a 256^3 + 128^3
+// V-cycle (pressure solve 25.7 -> 22.5 ms, 18 cycles).  Buffers whose stencils read stored coarse-fine ghosts keep them zero: T1 and T2
+// are never given ghost values, E and X have theirs cleared here.
 template <typename T, int D>
-amr_status vcycle_corr(amr_operator* op, const amr_solver_params& p, const T* r, cudaStream_t st) {
+amr_status vcycle_corr(amr_operator* op, const amr_solver_params& p, const T* r, cudaStream_t st, int flags) {
   amr_hierarchy* h = op->h;
   Scratch<T>& S = scratch<T>(op);
   const int L = h->L - 1;
   const size_t bytes = (size_t)h->nelems * sizeof(T);
-  CK(cudaMemsetAsync(S.E, 0, bytes, st));
-  CK(cudaMemsetAsync(S.X, 0, bytes, st));
-  CK(cudaMemsetAsync(S.T1, 0, bytes, st));
-  CK(cudaMemsetAsync(S.T2, 0, bytes, st));
+  if (p.nu1 < 1) {  // no down sweep writes the corrections: all of them start from zero
+    CK(cudaMemsetAsync(S.E, 0, bytes, st));
+    CK(cudaMemsetAsync(S.X, 0, bytes, st));
+  }
+  if (L == 0) return mg_level0<T, D>(op, p, 0, r, S.X, S.T1, st);
   for (int c = 0; c < h->ncomp; ++c) {
     long long a, b;
     level_range(h, L, a, b, c);
     CK(cudaMemcpyAsync(S.R + a, r + a, (size_t)(b - a) * sizeof(T), cudaMemcpyDeviceToDevice, st));
+    for (int l = 1; l < L && p.nu1 >= 1; ++l) {
+      level_range(h, l, a, b, c);
+      CK(cudaMemsetAsync(S.X + a, 0, (size_t)(b - a) * sizeof(T), st));
+    }
   }
   std::vector<LevelView> lv(h->L);
   for (int l = 0; l <= L; ++l) lv[l] = level_view(h, l, op->bc);
   const double a_ = op->alpha, b_ = op->beta;
+  // level 0: its right-hand side is r itself, changed around the boxes only (kept in S.R)
+  T* const r0 = const_cast<T*>(r);
+  const DeviceLists& d0 = h->lev[0].dev;
+  auto region_grid = [&](int grow) {
+    long long n = 1;
+    for (int d = 0; d < D; ++d) n *= std::min(d0.xfer_max[d] + 2 * grow, lv[0].ndom[d]);
+    return dim3((unsigned)((n + 255) / 256), (unsigned)d0.nxfer, 1);
+  };
+  launch(k_region_begin<T, D>, region_grid(RGN_READ), 256, 0, st, lv[0], d0.xfer, r, S.X, S.R);
+  TRY(launch_check());
+  auto corr = [&](int l) { return l == L ? S.X : S.E; };  // correction of level l >= 1
+  auto acc = [&](int l) { return l == L ? (T*)nullptr : S.X; };  // its accumulated copy, if any
   // ---- down
   for (int l = L; l >= 1; --l) {
     const DeviceLists& cl = h->lev[l - 1].dev;
+    T* E = corr(l);
+    T* const rc = l == 1 ? r0 : S.R;  // right-hand side of level l - 1
     bool deferred = false;
+    if (h->lev[l].dev.ncfi) TRY(cfi_fill<T, D>(h, l, E, E, true, st));  // zero coarse-fine ghosts
     if (blocked_amr_level<T, D>(op, p, l)) {
-      // one launch: nu1 sweeps from zero (zero CF ghosts) into E_l, X_l += E_l, and the
+      // one launch: nu1 sweeps from zero (zero CF ghosts) into E_l (and X_l), and the
       // mean of the fine residual R_l - A_l E_l into R_{l-1} on the covered cells
       const PatchDesc& fp = h->lev[l].patches[0];
       const PatchDesc& cpd = h->lev[l - 1].patches[h->lev[l - 1].xfer[0].cpatch];
@@ -1822,14 +1866,24 @@ amr_status vcycle_corr(amr_operator* op, const amr_solver_params& p, const T* r,
       cudaEvent_t ev;
       prof_begin(st, &ev);
       launch_down2d<T>(tt, p.nu1, grid, blk_smem_fx<T>(fp.n, p.nu1, true), st, lv[l], fp, cpd, tt, tt, hd, p.nu1,
-                       (const T*)S.R, S.E, S.X, S.R, T(a_), T(b_), T(p.omega), ood);
+                       (const T*)S.R, E, acc(l), rc, T(a_), T(b_), T(p.omega), ood);
       TRY(launch_check());
-      prof_end(st, ev, PC_DOWN, (3.0 + 0.25) * sizeof(T) * (double)fp.n[0] * fp.n[1]);  // f in; e, x, coarse f out
+      prof_end(st, ev, PC_DOWN, ((acc(l) ? 3.0 : 2.0) + 0.25) * sizeof(T) * (double)fp.n[0] * fp.n[1]);
     } else {
-      TRY(smooth_from_zero<T, D>(h, l, lv[l], S.R, S.E, S.T1, p.nu1, a_, b_, p.omega, true, st));
-      TRY(axpy<T, T, D>(lv[l], S.E, S.X, (T*)nullptr, 1.0, st));
-      TRY(copy_fill<T>(h, l, S.E, st));
-      deferred = true;  // the fine residual's mean is restricted after the level-(l-1) residual
+      TRY(smooth_from_zero<T, D>(h, l, lv[l], S.R, E, S.T1, p.nu1, a_, b_, p.omega, true, st));
+      if (acc(l)) TRY(axpy<T, T, D>(lv[l], E, acc(l), (T*)nullptr, 1.0, st));
+      TRY(copy_fill<T>(h, l, E, st));
+      deferred = true;
+    }
+    if (deferred && l == 1) {
+      // the mean of the fine residual R_1 - A_1 E_1 (zero CF ghosts) on the covered cells; the
+      // level-0 residual below writes the valid cells only
+      if (D == 3 && lv[0].npatch == lv[0].ncomp && sw_eligible(lv[1]) && lv[1].maxn[2] % 2 == 0 &&
+          tile_rows_for(lv[1], sizeof(T)) == TILE_BULK) {
+        TRY(bulk_restrict_level<T>(lv[1], lv[0], E, S.R, rc, a_, b_, st));
+      } else {
+        TRY(restrict_blocks<T, D>(lv[1], lv[0], cl.xfer, cl.nxfer, cl.xfer_max, true, E, S.R, rc, a_, b_, st));
+      }
     }
     // valid cells of level l-1: composite residual r - A^comp X
     for (int m = l - 1; m >= 0; --m) {
@@ -1839,45 +1893,55 @@ amr_status vcycle_corr(amr_operator* op, const amr_solver_params& p, const T* r,
     }
     if (l - 1 >= 1) TRY(cfi_fill<T, D>(h, l - 1, S.X, S.X, false, st));
     TRY(copy_fill<T>(h, l - 1, S.X, st));
-    TRY(cfi_fill<T, D>(h, l, S.X, S.X, false, st));
-    TRY(copy_fill<T>(h, l, S.X, st));
-    if (deferred) {
+    if (deferred && l > 1) {
       // every cell of level l-1, then its invalid cells overwritten by the mean of the fine
-      // residual R_l - A_l E_l (zero CF ghosts): the same values as the masked residual
-      // after the restriction, without the mask (the restriction reads neither array the
-      // level-(l-1) residual writes)
+      // residual R_l - A_l E_l (zero CF ghosts, hence before E_L = X_L gets its own)
       TRY(level_op<T, D>(OP_RESID, lv[l - 1], S.X, r, S.R, nullptr, a_, b_, 0.0, nullptr, st));
       if (D == 3 && lv[l - 1].npatch == lv[l - 1].ncomp && sw_eligible(lv[l]) && lv[l].maxn[2] % 2 == 0 &&
           tile_rows_for(lv[l], sizeof(T)) == TILE_BULK) {
-        // a single-patch fine level over a single-patch coarse level: the bulk-copy
-        // restriction (the arithmetic of k_restrict)
-        cudaEvent_t ev;
-        prof_begin(st, &ev);
-        TRY((launch_sw<T, OP_RESTRICT>(lv[l], S.E, S.R, (T*)nullptr, T(a_), T(b_), T(0), nullptr, st, nullptr, S.R,
-                                       &lv[l - 1].p0, lv[l - 1].cstride)));
-        const double cc = lv[l].ncells / 8.0;
-        prof_end(st, ev, PC_RESTRICT, (2.0 * 8 + 1.0) * sizeof(T) * cc, cc * 8);
+        TRY(bulk_restrict_level<T>(lv[l], lv[l - 1], E, S.R, S.R, a_, b_, st));
       } else {
-        TRY(restrict_blocks<T, D>(lv[l], lv[l - 1], cl.xfer, cl.nxfer, cl.xfer_max, true, S.E, S.R, S.R, a_, b_, st));
+        TRY(restrict_blocks<T, D>(lv[l], lv[l - 1], cl.xfer, cl.nxfer, cl.xfer_max, true, E, S.R, S.R, a_, b_, st));
       }
-    } else {
+    } else if (l > 1) {
       TRY(level_op<T, D>(OP_RESID, lv[l - 1], S.X, r, S.R, nullptr, a_, b_, 0.0, h->d_valid, st));
+    } else {
+      launch(k_region_resid<T, D>, region_grid(RGN_RESID), 256, 0, st, lv[0], d0.xfer, S.X, S.R, r0, h->d_valid, T(a_),
+             T(b_));
+      TRY(launch_check());
     }
+    TRY(cfi_fill<T, D>(h, l, S.X, S.X, false, st));
+    TRY(copy_fill<T>(h, l, S.X, st));
     P3<T> xc{{S.X, S.X, S.X}}, xf{{S.X, S.X, S.X}}, nb{{nullptr, nullptr, nullptr}};
-    TRY(reflux<T, D>(h, l - 1, lv[l - 1], lv[l], xc, xf, nb, S.R, -b_, 0, st));
+    TRY(reflux<T, D>(h, l - 1, lv[l - 1], lv[l], xc, xf, nb, rc, -b_, 0, st));
   }
   // ---- level 0: single-level V-cycle on all of level 0
-  TRY(mg_level0<T, D>(op, p, 0, S.R, S.E, S.T1, st));
-  TRY(axpy<T, T, D>(lv[0], S.E, S.X, (T*)nullptr, 1.0, st));
+  if (flags & VC_COVERED) {
+    launch(k_region_move<T, D>, region_grid(0), 256, 0, st, lv[0], d0.xfer, 0, (const T*)S.X, S.E, 0);
+    TRY(launch_check());
+  }
+  for (int c = 0; c < h->ncomp && p.nu1 < 1; ++c) {
+    long long a, b;
+    level_range(h, 0, a, b, c);
+    CK(cudaMemsetAsync(S.X + a, 0, (size_t)(b - a) * sizeof(T), st));
+  }
+  TRY(mg_level0<T, D>(op, p, 0, r0, S.X, S.T1, st));
+  if (!(flags & VC_SCRATCH_R)) {
+    launch(k_region_move<T, D>, region_grid(RGN_RESID), 256, 0, st, lv[0], d0.xfer, (int)RGN_RESID, (const T*)S.R, r0, 0);
+    TRY(launch_check());
+  }
   // ---- up
   for (int l = 1; l <= L; ++l) {
     const DeviceLists& cl = h->lev[l - 1].dev;
-    TRY(copy_fill<T>(h, l - 1, S.E, st));
-    TRY(prolong_blocks<T, D>(lv[l], lv[l - 1], cl.xfer, cl.nxfer, cl.xfer_max, S.E, S.E, S.X, st));
-    TRY(cfi_fill<T, D>(h, l, S.E, S.E, false, st));
-    TRY(copy_fill<T>(h, l, S.E, st));
-    TRY(level_op<T, D>(OP_RESID, lv[l], S.E, S.R, S.R, nullptr, a_, b_, 0.0, nullptr, st));
-    if (blocked_amr_level<T, D>(op, p, l) && p.nu2 >= 1) {
+    T* E = corr(l);
+    T* const Ec = l == 1 ? S.X : S.E;
+    TRY(copy_fill<T>(h, l - 1, Ec, st));
+    TRY(prolong_blocks<T, D>(lv[l], lv[l - 1], cl.xfer, cl.nxfer, cl.xfer_max, Ec, E, acc(l), st));
+    TRY(cfi_fill<T, D>(h, l, Ec, E, false, st));
+    TRY(copy_fill<T>(h, l, E, st));
+    TRY(level_op<T, D>(OP_RESID, lv[l], E, S.R, S.R, nullptr, a_, b_, 0.0, nullptr, st));
+    if (p.nu2 < 1) continue;
+    if (blocked_amr_level<T, D>(op, p, l)) {
       // one launch: nu2 sweeps from zero on R_l (zero CF ghosts), added to E_l and X_l
       const PatchDesc& fp = h->lev[l].patches[0];
       const int tt = blk_tile(fp.n), hu = 2 * p.nu2;
@@ -1886,13 +1950,17 @@ amr_status vcycle_corr(amr_operator* op, const amr_solver_params& p, const T* r,
       cudaEvent_t ev;
       prof_begin(st, &ev);
       launch_post2d<T>(tt, p.nu2, grid, blk_smem_fx<T>(fp.n, p.nu2, false), st, lv[l], fp, tt, tt, hu, p.nu2,
-                       (const T*)S.R, S.E, S.X, T(a_), T(b_), T(p.omega), ood);
+                       (const T*)S.R, E, acc(l), T(a_), T(b_), T(p.omega), ood);
       TRY(launch_check());
-      prof_end(st, ev, PC_UP, 5.0 * sizeof(T) * (double)fp.n[0] * fp.n[1]);  // r in; e, x read and written
+      prof_end(st, ev, PC_UP, (acc(l) ? 5.0 : 3.0) * sizeof(T) * (double)fp.n[0] * fp.n[1]);  // r in; e (and x) read and written
     } else {
       TRY(smooth_from_zero<T, D>(h, l, lv[l], S.R, S.T1, S.T2, p.nu2, a_, b_, p.omega, true, st));
-      TRY(axpy<T, T, D>(lv[l], S.T1, S.E, S.X, 1.0, st));
+      TRY(axpy<T, T, D>(lv[l], S.T1, E, acc(l), 1.0, st));
     }
+  }
+  if (flags & VC_COVERED) {
+    launch(k_region_move<T, D>, region_grid(0), 256, 0, st, lv[0], d0.xfer, 0, (const T*)S.E, S.X, 1);
+    TRY(launch_check());
   }
   return AMR_OK;
 }
@@ -2174,7 +2242,7 @@ amr_status ensure_inner(amr_operator* op) {
 template <int D>
 amr_status mixed_correction(amr_operator* op, const amr_solver_params& p, cudaStream_t st) {
   Scratch<float>& S = op->s32;
-  TRY((vcycle_corr<float, D>(op, p, S.rin, st)));
+  TRY((vcycle_corr<float, D>(op, p, S.rin, st, cpr_of(p) <= 1 ? VC_SCRATCH_R : 0)));
   if (cpr_of(p) <= 1) return AMR_OK;
   if (op->inner_x == nullptr || op->inner_r == nullptr) {
     set_error("correction-cycle buffers were not allocated before the solve");
@@ -2184,7 +2252,7 @@ amr_status mixed_correction(amr_operator* op, const amr_solver_params& p, cudaSt
   for (int c = 1; c < cpr_of(p); ++c) {
     std::swap(S.X, op->inner_x);
     TRY(composite_op<D>(op, OP_RESID, op->inner_x, (const float*)S.rin, op->inner_r, (const float*)nullptr, st));
-    TRY((vcycle_corr<float, D>(op, p, op->inner_r, st)));
+    TRY((vcycle_corr<float, D>(op, p, op->inner_r, st, VC_SCRATCH_R)));
     for (int l = 0; l < h->L; ++l)
       TRY((axpy<float, float, D>(level_view(h, l, nullptr), op->inner_x, S.X, (float*)nullptr, 1.0, st)));
   }
@@ -2238,7 +2306,7 @@ amr_status solve_impl(amr_operator* op, const amr_solver_params& p, double* phi,
       for (int l = 0; l < h->L; ++l) TRY(axpy<float, double, D>(level_view(h, l, nullptr), S.X, phi, (double*)nullptr, 1.0, st));
     } else {
       Scratch<double>& S = op->s64;
-      TRY(vcycle_corr<double, D>(op, p, op->Res, st));
+      TRY(vcycle_corr<double, D>(op, p, op->Res, st, VC_SCRATCH_R));
       for (int l = 0; l < h->L; ++l) TRY(axpy<double, double, D>(level_view(h, l, nullptr), S.X, phi, (double*)nullptr, 1.0, st));
     }
   }
@@ -2294,7 +2362,7 @@ amr_status iteration_body(amr_operator* op, int prec, const amr_solver_params& p
            active);
   } else {
     Scratch<double>& Sd = op->s64;
-    TRY(vcycle_corr<double, D>(op, p, op->Res, st));
+    TRY(vcycle_corr<double, D>(op, p, op->Res, st, VC_SCRATCH_R));
     launch(k_update_valid<double>, grid, 256, 0, st, n, (const double*)Sd.X, phi, (const unsigned char*)h->d_valid,
            rbits, active);
   }
@@ -2547,7 +2615,7 @@ amr_status vcycle_impl(amr_operator* op, const amr_solver_params& p, double* phi
   amr_hierarchy* h = op->h;
   TRY(ensure_scratch<double>(op));
   TRY(composite_op<D>(op, OP_RESID, phi, f, op->Res, bc, st));
-  TRY(vcycle_corr<double, D>(op, p, op->Res, st));
+  TRY(vcycle_corr<double, D>(op, p, op->Res, st, VC_SCRATCH_R | VC_COVERED));
   for (int l = 0; l < h->L; ++l) TRY(axpy<double, double, D>(level_view(h, l, nullptr), op->s64.X, phi, (double*)nullptr, 1.0, st));
   return AMR_OK;
 }
