@@ -994,6 +994,9 @@ amr_status ensure_scratch(amr_operator* op) {
   } else {
     TRY((autotune_tiles<T, 3>(op, 0)));
   }
+  // the clears above run on the default stream, which the solves' non-blocking streams do not
+  // wait for: a solve could start before its scratch is zero
+  CK(cudaStreamSynchronize(0));
   return AMR_OK;
 }
 
@@ -2220,7 +2223,8 @@ amr_status ensure_inner(amr_operator* op) {
   float* a = nullptr;
   float* b = nullptr;
   if (cudaMalloc(&a, bytes) != cudaSuccess || cudaMalloc(&b, bytes) != cudaSuccess ||
-      cudaMemset(a, 0, bytes) != cudaSuccess || cudaMemset(b, 0, bytes) != cudaSuccess) {
+      cudaMemset(a, 0, bytes) != cudaSuccess || cudaMemset(b, 0, bytes) != cudaSuccess ||
+      cudaStreamSynchronize(0) != cudaSuccess) {  // non-blocking streams do not wait for the clears
     cudaFree(a);
     cudaFree(b);
     cudaGetLastError();
@@ -3326,7 +3330,8 @@ amr_status batch_stacked(amr_operator* const* ops, int n, const amr_solver_param
     }
     if (s1 == AMR_OK) s1 = dalloc(&c->f, c->hs->nelems);
     if (s1 == AMR_OK && (cudaMemset(c->phi, 0, c->hs->nelems * sizeof(double)) != cudaSuccess ||
-                         cudaMemset(c->f, 0, c->hs->nelems * sizeof(double)) != cudaSuccess))
+                         cudaMemset(c->f, 0, c->hs->nelems * sizeof(double)) != cudaSuccess ||
+                         cudaStreamSynchronize(0) != cudaSuccess))
       s1 = AMR_ERR_CUDA;
     lead->stack = c.release();
     if (s1 != AMR_OK) {
@@ -3871,6 +3876,7 @@ amr_status amr_operator_create(amr_hierarchy* h, double alpha, double beta, cons
   CK(cudaMemset(op->F, 0, ne * sizeof(double)));
   CK(cudaMemset(op->Res, 0, ne * sizeof(double)));
   CK(cudaMemset(op->Tmp, 0, ne * sizeof(double)));
+  CK(cudaStreamSynchronize(0));  // a solve may run on a stream that does not wait for the default one
   *out = op.release();
   return AMR_OK;
 }
