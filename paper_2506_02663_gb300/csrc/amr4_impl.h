@@ -82,6 +82,22 @@ struct CfiGroup {
   signed char pad;
 };
 
+// A rectangle of up to 8 x 8 coarse parents on one face of a fine patch (3-D, ratio 2) whose
+// windows lie in one coarse patch and are centred along the face: the folds along the normal
+// and along the first tangential dimension are shared by the parents of the rectangle.
+// Strides are in elements; bit a + 8 b of mask: parent (a, b) has ghosts.
+constexpr int CFI_TILE = 8;
+struct CfiTile {
+  long long src;            // first window cell: normal window start, two cells before parent (0, 0)
+  long long dst;            // child 0 of parent (0, 0)
+  int sn, s1, s2;           // coarse strides: normal, first and second tangential dimension
+  int fn, f1, f2;           // fine strides
+  int n1, n2;               // parents
+  int posn;                 // the parent's place in the normal window
+  int pad;
+  unsigned long long mask;
+};
+
 // One coarse-fine interface face of a level (Sec. 6.4, Eq. correctingFaceAvg): the CF ghost
 // of the first layer across it, step = side x the patch stride along the face normal (the
 // interior cell next to the face is ghost - step, the second ghost layer ghost + step), the
@@ -134,6 +150,10 @@ struct DeviceLists {
   long long ncfi = 0;
   CfiGroup* cfig = nullptr;  // the same ghosts grouped by coarse parent (ratio 2)
   long long ncfig = 0;
+  CfiTile* cfit = nullptr;   // the groups that form regular face rectangles (3-D)
+  int ncfit = 0;
+  CfiGroup* cfir = nullptr;  // the other groups (slid or multi-patch windows, partial parents)
+  long long ncfir = 0;
   CopyEntry* copy = nullptr;
   long long ncopy = 0;
   CicFace* cicf = nullptr;  // coarse-fine interface faces, grouped by connected component
@@ -144,14 +164,7 @@ struct DeviceLists {
   int* cic_ccstart = nullptr;      // chunks of component c: [ccstart[c], ccstart[c+1])
   double* cic_psum = nullptr;      // one partial sum per chunk
   int ncic_chunks = 0;
-  // 3-D interface ghosts: the distinct coarse cells of the level's AMRCFI windows (field
-  // offsets, ascending) and scratch for their two time combinations, indexed by offset -
-  // cic_base over the coarse level's span; made by the first amr_cic_ghosts call
-  long long* cic_band = nullptr;
-  long long ncic_band = 0;
-  long long cic_base = 0;
-  double* cic_y = nullptr;  // 2 x cic_span doubles
-  long long cic_span = 0;
+  bool cic_seen = false;  // a 3-D interface-ghost call was made outside a stream capture
   long long* cic_slot = nullptr;  // per face, see LevelHost::cic_slot
   RefluxEntry* reflux = nullptr;
   long long nreflux = 0;

@@ -2,8 +2,10 @@
 // field layout, index maps (Eq. validRegion, Fig. 1 (b)-(c)), and the device work lists for
 // ghost filling (copy / AMRCFI, Sec. 5.2), refluxing (COH-3) and level transfers.
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstring>
+#include <map>
 #include <memory>
 #include <numeric>
 #include <stdexcept>
@@ -296,7 +298,7 @@ static void group_cic_faces(LevelHost& L, const std::vector<int>& im_component, 
 }
 
 static std::vector<CfiGroup> cfi_groups(const std::vector<CfiEntry>& cfi, const std::vector<long long>& key, int r,
-                                        int D) {
+                                        int D, std::vector<const CfiEntry*>* first = nullptr) {
   std::vector<CfiGroup> out;
   if (r != 2 || cfi.empty() || key.size() != cfi.size()) return out;
   std::vector<size_t> ord(cfi.size());
@@ -316,9 +318,82 @@ static std::vector<CfiGroup> cfi_groups(const std::vector<CfiEntry>& cfi, const 
       g.dst[c] = e.dst;
     }
     out.push_back(g);
+    if (first != nullptr) first->push_back(&e0);
     i = j;
   }
   return out;
+}
+
+// Face rectangles of the groups whose window lies in one coarse patch, centred along the face,
+// with all eight children at their regular places; the other groups go to ``rest``.
+static void cfi_tiles(const std::vector<CfiGroup>& groups, const std::vector<const CfiEntry*>& first,
+                      const LevelHost& fine, const LevelHost& crs, std::vector<CfiTile>& tiles, std::vector<CfiGroup>& rest) {
+  struct Parent {
+    int a, b;  // tangential coordinates (padded, coarse patch)
+    long long src, dst;
+  };
+  struct Bucket {
+    const CfiEntry* e;
+    std::vector<Parent> ps;
+  };
+  std::map<std::array<int, 6>, Bucket> buckets;  // fine patch, dimension, side, coarse patch, normal coordinate, place
+  for (size_t i = 0; i < groups.size(); ++i) {
+    const CfiGroup& g = groups[i];
+    const CfiEntry& e = *first[i];
+    const int d = e.dir, t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
+    bool ok = g.src >= 0 && g.pos[t1] == 2 && g.pos[t2] == 2;
+    const PatchDesc& fp = fine.patches[e.fpatch];
+    for (int c = 0; c < 8 && ok; ++c)
+      ok = g.dst[c] >= 0 && g.dst[c] == g.dst[0] + (c & 1) + ((c >> 1) & 1) * fp.sy + (c >> 2) * fp.sz;
+    if (!ok) {
+      rest.push_back(g);
+      continue;
+    }
+    const PatchDesc& cp = crs.patches[g.cpatch];
+    const long long rel = g.src - cp.off;
+    const int w[3] = {(int)(rel % cp.sy), (int)(rel % cp.sz / cp.sy), (int)(rel / cp.sz)};  // window start
+    Bucket& b = buckets[{e.fpatch, d, e.layer > 0 ? 1 : 0, g.cpatch, w[d], g.pos[d]}];
+    b.e = &e;
+    b.ps.push_back({w[t1], w[t2], g.src, g.dst[0]});
+  }
+  for (auto& kv : buckets) {
+    Bucket& b = kv.second;
+    const int d = b.e->dir, t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
+    const PatchDesc& fp = fine.patches[b.e->fpatch];
+    const PatchDesc& cp = crs.patches[kv.first[3]];
+    const long long cs[3] = {1, cp.sy, cp.sz}, fs[3] = {1, fp.sy, fp.sz};
+    int a0 = b.ps[0].a, b0 = b.ps[0].b;
+    for (const Parent& p : b.ps) {
+      a0 = std::min(a0, p.a);
+      b0 = std::min(b0, p.b);
+    }
+    std::map<std::pair<int, int>, std::vector<const Parent*>> cells;
+    for (const Parent& p : b.ps) cells[{(p.b - b0) / CFI_TILE, (p.a - a0) / CFI_TILE}].push_back(&p);
+    for (auto& c : cells) {
+      int la = c.second[0]->a, ha = la, lb = c.second[0]->b, hb = lb;
+      for (const Parent* p : c.second) {
+        la = std::min(la, p->a);
+        ha = std::max(ha, p->a);
+        lb = std::min(lb, p->b);
+        hb = std::max(hb, p->b);
+      }
+      const Parent& q = *c.second[0];
+      CfiTile t{};
+      t.src = q.src - (q.a - la) * cs[t1] - (q.b - lb) * cs[t2];
+      t.dst = q.dst - 2 * (q.a - la) * fs[t1] - 2 * (q.b - lb) * fs[t2];
+      t.sn = (int)cs[d];
+      t.s1 = (int)cs[t1];
+      t.s2 = (int)cs[t2];
+      t.fn = (int)fs[d];
+      t.f1 = (int)fs[t1];
+      t.f2 = (int)fs[t2];
+      t.n1 = ha - la + 1;
+      t.n2 = hb - lb + 1;
+      t.posn = kv.first[5];
+      for (const Parent* p : c.second) t.mask |= 1ull << ((p->a - la) + CFI_TILE * (p->b - lb));
+      tiles.push_back(t);
+    }
+  }
 }
 
 namespace {
@@ -897,9 +972,19 @@ amr_status upload_hierarchy(amr_hierarchy* h, std::string& err) {
       L.dev.cfi = upload(L.cfi);
       L.dev.ncfi = (long long)L.cfi.size();
       {
-        const std::vector<CfiGroup> g = cfi_groups(L.cfi, L.cfi_key, h->r, h->D);
+        std::vector<const CfiEntry*> first;
+        const std::vector<CfiGroup> g = cfi_groups(L.cfi, L.cfi_key, h->r, h->D, &first);
         L.dev.cfig = upload(g);
         L.dev.ncfig = (long long)g.size();
+        if (h->D == 3 && !g.empty()) {
+          std::vector<CfiTile> tiles;
+          std::vector<CfiGroup> rest;
+          cfi_tiles(g, first, L, h->lev[l - 1], tiles, rest);
+          L.dev.cfit = upload(tiles);
+          L.dev.ncfit = (int)tiles.size();
+          L.dev.cfir = upload(rest);
+          L.dev.ncfir = (long long)rest.size();
+        }
       }
       L.dev.cfi_side = upload(L.cfi_side);
       L.dev.copy = upload(L.copy);
@@ -949,6 +1034,8 @@ void free_hierarchy(amr_hierarchy* h) {
     cudaFree(L.d_patches);
     cudaFree(L.dev.cfi);
     cudaFree(L.dev.cfig);
+    cudaFree(L.dev.cfit);
+    cudaFree(L.dev.cfir);
     cudaFree(L.dev.cfi_side);
     cudaFree(L.dev.copy);
     cudaFree(L.dev.cicf);
@@ -956,9 +1043,7 @@ void free_hierarchy(amr_hierarchy* h) {
     cudaFree(L.dev.cic_chunks);
     cudaFree(L.dev.cic_ccstart);
     cudaFree(L.dev.cic_psum);
-    cudaFree(L.dev.cic_band);
     cudaFree(L.dev.cic_slot);
-    cudaFree(L.dev.cic_y);
     cudaFree(L.dev.reflux);
     cudaFree(L.dev.xfer);
   }

@@ -1094,6 +1094,81 @@ __global__ void k_cfi_grp(const CfiGroup* __restrict__ list, long long n, const 
     if (g.dst[c] >= 0) xf[g.dst[c]] = acc[c & 1][(c >> 1) & 1][c >> 2];
 }
 
+// AMRCFI of face rectangles (CfiTile), one block per rectangle: the window columns fold along
+// the face normal (both children), the folded plane along the first tangential dimension, then
+// along the second.  The first two folds serve every parent whose window holds the column, so a
+// parent costs about 92 multiply-adds instead of 390 by itself; in FP64 their rate bounds the
+// pass (interface conditions of a 128^3 box, three components: 197 -> 72 us a call).  NS = 1: one field; NS = 4: the fields at four times, combined by two rows of weights
+// after the normal fold (value and time derivative; AMRCFI and the combination are linear).
+template <typename T, int NS>
+struct CfiSource {
+  const T* x[NS];
+  T w[2][NS];  // NS = 4: weights of the value and of the derivative
+};
+
+template <typename T, int NS>
+__global__ void __launch_bounds__(128) k_cfi_tile(const CfiTile* __restrict__ tiles, CfiSource<T, NS> s, T* out0, T* out1) {
+  constexpr int NR = NS == 1 ? 1 : 2, M = CFI_TILE + CFI_W - 1;
+  __shared__ T fa[NR][2][M][M + 1];            // [row][normal child][second][first tangential column]
+  __shared__ T fb[NR][2][M][2 * CFI_TILE];     // folded along the first tangential dimension
+  pdl_wait();
+  const CfiTile t = tiles[blockIdx.x];
+  const int tid = threadIdx.x;
+  const int m1 = t.n1 + CFI_W - 1, m2 = t.n2 + CFI_W - 1;
+  const int nr = (NS == 1 || out1 == nullptr) ? 1 : 2;
+  const int bn = 2 * t.posn * CFI_W, bt = 4 * CFI_W;  // weights of the normal window; of a centred one
+  for (int q = tid; q < m1 * m2; q += 128) {
+    const int j1 = q % m1, j2 = q / m1;
+    const long long o = t.src + (long long)j1 * t.s1 + (long long)j2 * t.s2;
+    T f[NS][2];
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+      T v[CFI_W];
+#pragma unroll
+      for (int c = 0; c < CFI_W; ++c) v[c] = s.x[i][o + (long long)c * t.sn];
+      f[i][0] = f[i][1] = T(0);
+#pragma unroll
+      for (int c = 0; c < CFI_W; ++c) {
+        f[i][0] += cfiw<T>(bn + c) * v[c];
+        f[i][1] += cfiw<T>(bn + CFI_W + c) * v[c];
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        T v = f[0][h];
+        if (NS > 1) {
+          v = s.w[r][0] * f[0][h];
+#pragma unroll
+          for (int i = 1; i < NS; ++i) v += s.w[r][i] * f[i][h];
+        }
+        fa[r][h][j2][j1] = v;
+      }
+  }
+  __syncthreads();
+  const int w1 = 2 * t.n1, w2 = 2 * t.n2;
+  for (int q = tid; q < w1 * m2 * 2 * nr; q += 128) {
+    const int o1 = q % w1, u = q / w1, j2 = u % m2, hr = u / m2, h = hr & 1, r = hr >> 1;
+    const T* __restrict__ a = &fa[r][h][j2][o1 >> 1];
+    const int b = bt + (o1 & 1) * CFI_W;
+    T v = T(0);
+#pragma unroll
+    for (int c = 0; c < CFI_W; ++c) v += cfiw<T>(b + c) * a[c];
+    fb[r][h][j2][o1] = v;
+  }
+  __syncthreads();
+  for (int q = tid; q < w1 * w2 * 2 * nr; q += 128) {
+    const int o1 = q % w1, u = q / w1, o2 = u % w2, hr = u / w2, h = hr & 1, r = hr >> 1;
+    if (!((t.mask >> ((o1 >> 1) + CFI_TILE * (o2 >> 1))) & 1ull)) continue;
+    const int b = bt + (o2 & 1) * CFI_W;
+    T v = T(0);
+#pragma unroll
+    for (int c = 0; c < CFI_W; ++c) v += cfiw<T>(b + c) * fb[r][h][(o2 >> 1) + c][o1];
+    (r == 0 ? out0 : out1)[t.dst + (long long)h * t.fn + (long long)o1 * t.f1 + (long long)o2 * t.f2] = v;
+  }
+}
+
 template <typename T>
 __global__ void k_copy(const CopyEntry* __restrict__ list, long long n, T* __restrict__ x) {
   pdl_wait();

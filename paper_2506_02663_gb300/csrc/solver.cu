@@ -811,8 +811,21 @@ amr_status cfi_fill(const amr_hierarchy* h, int l, const T* xc, T* xf, bool zero
   if (dl.ncfi == 0) return AMR_OK;
   const int nt = 128;
   if (dl.ncfig > 0) {  // ratio 2: by coarse parent
-    launch(k_cfi_grp<T, D>, (unsigned)((dl.ncfig + nt - 1) / nt), nt, 0, st, dl.cfig, dl.ncfig, dl.cfi_side,
-           h->lev[l - 1].d_patches, xc, xf, zero ? 1 : 0);
+    const CfiGroup* list = dl.cfig;
+    long long n = dl.ncfig;
+    if (D == 3 && !zero) {
+      if (dl.ncfit > 0) {
+        CfiSource<T, 1> s{};
+        s.x[0] = xc;
+        launch(k_cfi_tile<T, 1>, dl.ncfit, 128, 0, st, dl.cfit, s, xf, (T*)nullptr);
+        TRY(launch_check());
+      }
+      list = dl.cfir;
+      n = dl.ncfir;
+    }
+    if (n == 0) return AMR_OK;
+    launch(k_cfi_grp<T, D>, (unsigned)((n + nt - 1) / nt), nt, 0, st, list, n, dl.cfi_side, h->lev[l - 1].d_patches, xc, xf,
+           zero ? 1 : 0);
     return launch_check();
   }
   launch(k_cfi<T, D>, (unsigned)((dl.ncfi + nt - 1) / nt), nt, 0, st, dl.cfi, dl.ncfi, dl.cfi_side, h->lev[l - 1].d_patches,
@@ -3464,55 +3477,17 @@ void cic_weights(double k, double eta, double w[2][4]) {
     for (int i = 0; i < 4; ++i) w[r][i] = m[r][3 - i];
 }
 
-// The distinct coarse cells of level l's AMRCFI windows and the scratch for their time
-// combinations (3-D, ratio 2), made once per level on the first call that needs them.  The
-// scratch spans the coarse level's patches (2 doubles per element of that span).
-amr_status cic_band(amr_hierarchy* h, int l, cudaStream_t st) {
+// A 3-D level's first interface-ghost call must come before any stream capture.
+amr_status cic_first_call(amr_hierarchy* h, int l, cudaStream_t st) {
   LevelHost& L = h->lev[l];
-  if (L.dev.cic_y) return AMR_OK;
+  if (L.dev.cic_seen) return AMR_OK;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   CK(cudaStreamIsCapturing(st, &cs));
   if (cs != cudaStreamCaptureStatusNone) {
-    set_error("amr_cic_ghosts: the first call for a 3-D level allocates its scratch and must come before any "
-              "stream capture");
+    set_error("amr_cic_ghosts: the first call for a 3-D level must come before any stream capture");
     return AMR_ERR_INVALID_ARG;
   }
-  const LevelHost& C = h->lev[l - 1];
-  long long lo = -1, hi = 0;
-  for (const PatchDesc& p : C.patches) {
-    lo = lo < 0 ? p.off : std::min(lo, p.off);
-    hi = std::max(hi, p.off + p.sz * (p.n[2] + 2 * NG));
-  }
-  std::vector<unsigned char> mark((size_t)(hi - lo), 0);
-  for (const CfiEntry& e : L.cfi) {
-    if (e.src >= 0) {
-      const PatchDesc& cp = C.patches[e.cpatch];
-      for (int c2 = 0; c2 < CFI_W; ++c2)
-        for (int c1 = 0; c1 < CFI_W; ++c1)
-          for (int c0 = 0; c0 < CFI_W; ++c0) mark[(size_t)(e.src + c0 + c1 * cp.sy + c2 * cp.sz - lo)] = 1;
-    } else {
-      const long long* s = &L.cfi_side[(size_t)(-1 - e.src) * 125];
-      for (int q = 0; q < 125; ++q) mark[(size_t)(s[q] - lo)] = 1;
-    }
-  }
-  std::vector<long long> band;
-  for (size_t i = 0; i < mark.size(); ++i)
-    if (mark[i]) band.push_back(lo + (long long)i);
-  long long* d_band = nullptr;
-  double* d_y = nullptr;
-  if (cudaMalloc(&d_band, sizeof(long long) * std::max<size_t>(band.size(), 1)) != cudaSuccess ||
-      cudaMalloc(&d_y, sizeof(double) * 2 * (size_t)(hi - lo)) != cudaSuccess) {
-    cudaFree(d_band);
-    cudaGetLastError();
-    set_error("amr_cic_ghosts: scratch allocation failed");
-    return AMR_ERR_OOM;
-  }
-  CK(cudaMemcpy(d_band, band.data(), sizeof(long long) * band.size(), cudaMemcpyHostToDevice));
-  L.dev.cic_band = d_band;
-  L.dev.ncic_band = (long long)band.size();
-  L.dev.cic_base = lo;
-  L.dev.cic_span = hi - lo;
-  L.dev.cic_y = d_y;
+  L.dev.cic_seen = true;
   return AMR_OK;
 }
 
@@ -3528,21 +3503,26 @@ amr_status cic_ghosts_impl(amr_hierarchy* h, int l, const double* const* xt, dou
   CicTimes ct{};
   for (int i = 0; i < 4; ++i) ct.x[i] = xt[i];
   cic_weights(k, eta, ct.w);
-  const int nt = 128;
+  const CfiGroup* rest = dl.cfig;
+  long long nrest = dl.ncfig;
   if (D == 3) {
-    TRY(cic_band(h, l, st));
-    double* y0 = dl.cic_y;
-    double* y1 = rate ? dl.cic_y + dl.cic_span : nullptr;
-    launch(k_cic_combine, (unsigned)((dl.ncic_band + 255) / 256), 256, 0, st, dl.cic_band, dl.ncic_band,
-           dl.cic_base, ct, y0, y1);
-    TRY(launch_check());
-    launch(k_cic_grp3, (unsigned)((dl.ncfig * CIC_LANES + CIC_GRP_THREADS - 1) / CIC_GRP_THREADS),
-           CIC_GRP_THREADS, 0, st, dl.cfig, dl.ncfig, dl.cfi_side, h->lev[l - 1].d_patches, (const double*)y0,
-           (const double*)y1, dl.cic_base, v, rate);
-  } else {
-    launch(k_cic_grp<D>, (unsigned)((dl.ncfig + nt - 1) / nt), nt, 0, st, dl.cfig, dl.ncfig, dl.cfi_side,
-           h->lev[l - 1].d_patches, ct, v, rate);
+    TRY(cic_first_call(h, l, st));
+    rest = dl.cfir;
+    nrest = dl.ncfir;
+    if (dl.ncfit > 0) {
+      CfiSource<double, 4> s{};
+      for (int i = 0; i < 4; ++i) {
+        s.x[i] = xt[i];
+        for (int r = 0; r < 2; ++r) s.w[r][i] = ct.w[r][i];
+      }
+      launch(k_cfi_tile<double, 4>, dl.ncfit, 128, 0, st, dl.cfit, s, v, rate);
+      TRY(launch_check());
+    }
   }
+  if (nrest == 0) return AMR_OK;
+  const int nt = 32;  // few groups: one warp per block spreads them over the SMs
+  launch(k_cic_grp<D>, (unsigned)((nrest + nt - 1) / nt), nt, 0, st, rest, nrest, dl.cfi_side, h->lev[l - 1].d_patches, ct,
+         v, rate);
   return launch_check();
 }
 
