@@ -2022,16 +2022,45 @@ amr_status composite_op(amr_operator* op, int mode, T* x, const T* f, T* out, co
   return AMR_OK;
 }
 
-template <typename T, int D>
-amr_status maxnorm(amr_hierarchy* h, const T* x, bool use_mask, double* out_host, cudaStream_t st) {
+// grid of the whole-array passes: grid-stride, at most 8 blocks per SM
+inline unsigned flat_blocks(long long n) { return (unsigned)std::min<long long>((n + 255) / 256, 8LL * sm_count()); }
+
+// elements of one replica of a stacked component batch (the whole array otherwise)
+inline long long rep_elems(const amr_hierarchy* h) { return h->ncomp > 1 ? h->cstride : h->nelems; }
+
+// 16-byte accesses: the caller's field may start anywhere (a view of a larger buffer)
+inline bool flat_vec(long long n, const void* a, const void* b = nullptr) {
+  return n % 4 == 0 && reinterpret_cast<uintptr_t>(a) % 16 == 0 && reinterpret_cast<uintptr_t>(b) % 16 == 0;
+}
+
+// valid-cell max-norm of x into acc[c] (not cleared here) for each of nc runs of n elements,
+// and (rin given) x rounded to FP32
+inline amr_status norm_flat(const amr_hierarchy* h, long long n, int nc, const double* x, float* rin,
+                            unsigned long long* acc, cudaStream_t st) {
+  const unsigned char* m = h->d_valid;
+  if (flat_vec(n, x, rin)) launch(k_norm_convert<4>, dim3(flat_blocks(n / 4), nc, 1), 256, 0, st, n, x, m, rin, acc);
+  else launch(k_norm_convert<1>, dim3(flat_blocks(n), nc, 1), 256, 0, st, n, x, m, rin, acc);
+  return launch_check();
+}
+
+// phi += x on the valid cells
+template <typename S>
+amr_status update_flat(const amr_hierarchy* h, const S* x, double* phi, unsigned long long* acc_clear, const int* active,
+                       cudaStream_t st) {
+  const long long n = rep_elems(h);
+  const unsigned char* m = h->d_valid;
+  if (flat_vec(n, x, phi))
+    launch(k_update_valid<S, 4>, dim3(flat_blocks(n / 4), h->ncomp, 1), 256, 0, st, n, x, phi, m, acc_clear, active);
+  else
+    launch(k_update_valid<S, 1>, dim3(flat_blocks(n), h->ncomp, 1), 256, 0, st, n, x, phi, m, acc_clear, active);
+  return launch_check();
+}
+
+// max-norm of x over the valid cells of every level, read back; rin (nullable) receives x in FP32
+inline amr_status maxnorm(amr_hierarchy* h, const double* x, double* out_host, cudaStream_t st, float* rin = nullptr) {
   unsigned long long* acc = reinterpret_cast<unsigned long long*>(h->d_scalar);
   CK(cudaMemsetAsync(acc, 0, sizeof(unsigned long long), st));
-  for (int l = 0; l < h->L; ++l) {
-    LevelView lv = level_view(h, l, nullptr);
-    Geo g = geo_of(lv);
-    launch(k_maxnorm<T, D>, g.grid, g.block, 0, st, lv, g.nby, x, use_mask ? h->d_valid : nullptr, acc);
-    TRY(launch_check());
-  }
+  TRY(norm_flat(h, h->nelems, 1, x, rin, acc, st));
   CK(cudaMemcpyAsync(h->h_scalar, acc, sizeof(double), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   *out_host = h->h_scalar[0];
@@ -2174,19 +2203,6 @@ amr_status neumann_fix_T(amr_hierarchy* h, double* x, double* m_host, cudaStream
   return AMR_OK;
 }
 
-// max-norm over valid cells into *out (IEEE bits, atomicMax); no host readback
-template <typename T, int D>
-amr_status maxnorm_dev(amr_hierarchy* h, const T* x, unsigned long long* out, cudaStream_t st) {
-  CK(cudaMemsetAsync(out, 0, sizeof(unsigned long long), st));
-  for (int l = 0; l < h->L; ++l) {
-    LevelView lv = level_view(h, l, nullptr);
-    Geo g = geo_of(lv);
-    launch(k_maxnorm<T, D>, g.grid, g.block, 0, st, lv, g.nby, x, h->d_valid, out);
-    TRY(launch_check());
-  }
-  return AMR_OK;
-}
-
 // Bounded wait of about ``ns`` nanoseconds (at most 2^20 polls of the global timer).
 __global__ void k_headstart(unsigned long long ns) {
   pdl_wait();
@@ -2294,7 +2310,7 @@ amr_status solve_impl(amr_operator* op, const amr_solver_params& p, double* phi,
   if (p.zero_initial) CK(cudaMemsetAsync(phi, 0, bytes, st));
   TRY(avgdown_all<D>(h, op->F, st));
   double fn = 0.0;
-  TRY(maxnorm<double, D>(h, op->F, true, &fn, st));
+  TRY(maxnorm(h, op->F, &fn, st));
   loc.rhs_norm = fn;
   const double tol = std::max(p.rtol * fn, p.atol);
   if (p.precision == AMR_MIXED) TRY(ensure_scratch<float>(op));
@@ -2305,7 +2321,7 @@ amr_status solve_impl(amr_operator* op, const amr_solver_params& p, double* phi,
   int it = 0;
   for (;; ++it) {
     TRY(composite_op<D>(op, OP_RESID, phi, op->F, op->Res, bc, st));
-    TRY(maxnorm<double, D>(h, op->Res, true, &res, st));
+    TRY(maxnorm(h, op->Res, &res, st, p.precision == AMR_MIXED ? op->s32.rin : nullptr));
     if (it < 64) loc.res_history[it] = res;
     if (!std::isfinite(res)) { result = AMR_ERR_NONFINITE; set_error("residual is not finite"); break; }
     if (res <= tol) { result = AMR_OK; break; }
@@ -2317,14 +2333,11 @@ amr_status solve_impl(amr_operator* op, const amr_solver_params& p, double* phi,
       TRY(launch_check());
     }
     if (p.precision == AMR_MIXED) {
-      Scratch<float>& S = op->s32;
-      for (int l = 0; l < h->L; ++l) TRY(convert<double, float, D>(level_view(h, l, nullptr), op->Res, S.rin, st));
       TRY(mixed_correction<D>(op, p, st));
-      for (int l = 0; l < h->L; ++l) TRY(axpy<float, double, D>(level_view(h, l, nullptr), S.X, phi, (double*)nullptr, 1.0, st));
+      TRY(update_flat<float>(h, op->s32.X, phi, nullptr, nullptr, st));
     } else {
-      Scratch<double>& S = op->s64;
       TRY(vcycle_corr<double, D>(op, p, op->Res, st, VC_SCRATCH_R));
-      for (int l = 0; l < h->L; ++l) TRY(axpy<double, double, D>(level_view(h, l, nullptr), S.X, phi, (double*)nullptr, 1.0, st));
+      TRY(update_flat<double>(h, op->s64.X, phi, nullptr, nullptr, st));
     }
   }
   loc.vcycles = it * (p.precision == AMR_MIXED ? cpr_of(p) : 1);
@@ -2337,23 +2350,11 @@ amr_status solve_impl(amr_operator* op, const amr_solver_params& p, double* phi,
 
 // One V-cycle iteration of the solve loop (V-cycle on op->Res, phi += correction, new
 // residual and its norm), all stream-ordered on st; used inside the captured while-body.
-// grid of the whole-array passes: grid-stride, a few blocks per SM
-// grid-stride element-wise kernels: one block per 256 elements, at most 8 per SM
-inline unsigned flat_blocks(long long n) {
-  return (unsigned)std::min<long long>((n + 255) / 256, 8LL * sm_count());
-}
-
-// elements of one replica of a stacked component batch (the whole array otherwise)
-inline long long rep_elems(const amr_hierarchy* h) { return h->ncomp > 1 ? h->cstride : h->nelems; }
-
 // valid-cell max-norm of x into acc[c] for every replica c, and (rin given) x rounded to FP32
 inline amr_status norm_convert_field(amr_operator* op, const double* x, float* rin, unsigned long long* acc,
                                      cudaStream_t st) {
   amr_hierarchy* h = op->h;
-  const long long n = rep_elems(h);
-  launch(k_norm_convert, dim3(flat_blocks(n), h->ncomp, 1), 256, 0, st, n, x, (const unsigned char*)h->d_valid, rin,
-         acc);
-  return launch_check();
+  return norm_flat(h, rep_elems(h), h->ncomp, x, rin, acc, st);
 }
 
 // valid-cell max-norm of op->Res into acc (per replica), and (mixed precision) its FP32 copy
@@ -2369,21 +2370,14 @@ amr_status iteration_body(amr_operator* op, int prec, const amr_solver_params& p
                           cudaStream_t st) {
   amr_hierarchy* h = op->h;
   unsigned long long* rbits = h->d_cnorm;
-  const long long n = rep_elems(h);
-  const dim3 grid(flat_blocks(n), h->ncomp, 1);
   const int* active = h->ncomp > 1 ? op->d_active : nullptr;  // converged replicas keep their phi
   if (prec == AMR_MIXED) {
-    Scratch<float>& Sf = op->s32;
     TRY(mixed_correction<D>(op, p, st));
-    launch(k_update_valid<float>, grid, 256, 0, st, n, (const float*)Sf.X, phi, (const unsigned char*)h->d_valid, rbits,
-           active);
+    TRY(update_flat<float>(h, op->s32.X, phi, rbits, active, st));
   } else {
-    Scratch<double>& Sd = op->s64;
     TRY(vcycle_corr<double, D>(op, p, op->Res, st, VC_SCRATCH_R));
-    launch(k_update_valid<double>, grid, 256, 0, st, n, (const double*)Sd.X, phi, (const unsigned char*)h->d_valid,
-           rbits, active);
+    TRY(update_flat<double>(h, op->s64.X, phi, rbits, active, st));
   }
-  TRY(launch_check());
   TRY(composite_op<D>(op, OP_RESID, phi, op->F, op->Res, bc, st));
   return norm_convert(op, prec, rbits, st);
 }
@@ -2588,7 +2582,7 @@ amr_status solve_transpose_impl(amr_operator* op, const amr_solver_params& p, do
   // mean zero); A^T lambda = F^T g and 1^T lambda = 0 (F^T again at the end)
   if (op->neumann) TRY(neumann_fix_T<D>(h, op->F, &loc.removed_mean, st));
   double gn = 0.0;
-  TRY((maxnorm<double, D>(h, g, true, &gn, st)));
+  TRY(maxnorm(h, g, &gn, st));
   loc.rhs_norm = gn;
   const double tol = std::max(p.rtol * gn, p.atol);
   amr_status result = AMR_ERR_NOT_CONVERGED;
@@ -2597,19 +2591,17 @@ amr_status solve_transpose_impl(amr_operator* op, const amr_solver_params& p, do
   for (;; ++it) {
     TRY((composite_AT<double, D>(op, lam, st)));
     TRY((transpose_residual<double, D>(op, -1, g, op->Res, st)));
-    TRY((maxnorm<double, D>(h, op->Res, true, &res, st)));
+    TRY(maxnorm(h, op->Res, &res, st, p.precision == AMR_MIXED ? op->s32.rin : nullptr));
     if (it < 64) loc.res_history[it] = res;
     if (!std::isfinite(res)) { result = AMR_ERR_NONFINITE; set_error("residual is not finite"); break; }
     if (res <= tol) { result = AMR_OK; break; }
     if (it >= p.max_vcycles) { set_error("max_vcycles reached"); break; }
     if (p.precision == AMR_MIXED) {
-      Scratch<float>& Sf = op->s32;
-      for (int l = 0; l < h->L; ++l) TRY((convert<double, float, D>(level_view(h, l, nullptr), op->Res, Sf.rin, st)));
-      TRY((vcycle_corr_T<float, D>(op, p, Sf.rin, st)));
-      for (int l = 0; l < h->L; ++l) TRY((axpy<float, double, D>(level_view(h, l, nullptr), Sf.X, lam, (double*)nullptr, 1.0, st)));
+      TRY((vcycle_corr_T<float, D>(op, p, op->s32.rin, st)));
+      TRY(update_flat<float>(h, op->s32.X, lam, nullptr, nullptr, st));
     } else {
       TRY((vcycle_corr_T<double, D>(op, p, op->Res, st)));
-      for (int l = 0; l < h->L; ++l) TRY((axpy<double, double, D>(level_view(h, l, nullptr), op->s64.X, lam, (double*)nullptr, 1.0, st)));
+      TRY(update_flat<double>(h, op->s64.X, lam, nullptr, nullptr, st));
     }
   }
   if (op->neumann) TRY(neumann_fix_T<D>(h, lam, nullptr, st));
@@ -4048,8 +4040,7 @@ amr_status amr_residual(amr_operator* op, double* phi, const double* f, double* 
   TRY(DISPATCH(op->h, composite_op, op, OP_RESID, phi, f, res, bc, S(stream)));
   if (norm) {
     amr_hierarchy* h = op->h;
-    if (h->D == 2) TRY((maxnorm<double, 2>(h, res, true, norm, S(stream))));
-    else TRY((maxnorm<double, 3>(h, res, true, norm, S(stream))));
+    TRY(maxnorm(h, res, norm, S(stream)));
   }
   return AMR_OK;
 }
