@@ -263,6 +263,119 @@ __device__ __forceinline__ void cell_level_op(const LevelView& lv, const PatchDe
   }
 }
 
+// distance class of global index g to the faces of an n-cell dimension: 0 interior, 1 and 2
+// the first and second cell from the low face, 3 and 4 from the high face
+__device__ __forceinline__ int face_class(int g, int n) {
+  return g == 0 ? 1 : g == 1 ? 2 : g == n - 1 ? 3 : g == n - 2 ? 4 : 0;
+}
+
+// Jacobi factors omega / diag by distance class of the cell to the x, y [and z] faces
+// (face_class; index x + 5 y [+ 25 z]), filled on the host (jacobi_factors).
+template <typename T, int D>
+struct JFac {
+  T w[D == 3 ? 125 : 25];
+};
+
+// Sums of the first and of the second neighbours along one dimension of the cell at offset o,
+// g <= 1 or g >= n - 2 (global index, n cells in the domain): a face cell reads the ghost
+// layers 1 and 2, its neighbour layer 1.  Ghost values in read_nb's order of operations; both
+// sums are commutative, so the low and the high side share one form.
+template <typename T>
+__device__ __forceinline__ void face_sums(const T* __restrict__ xb, int o, int st, int g, int n, int tlo, int thi, T& a1,
+                                          T& a2) {
+  const bool low = g < 2;
+  const int q = low ? g : n - 1 - g;
+  const int s = low ? st : -st;
+  const int t = low ? tlo : thi;
+  const int b = o - q * s;
+  const T c0 = xb[b], c1 = xb[b + s], c2 = xb[b + 2 * s], c3 = xb[b + 3 * s];
+  T g1 = T(0);
+  g1 += gcoef<T>(t, 0, 0) * c0;
+  g1 += gcoef<T>(t, 0, 1) * c1;
+  g1 += gcoef<T>(t, 0, 2) * c2;
+  g1 += gcoef<T>(t, 0, 3) * c3;
+  if (q == 0) {
+    T g2 = T(0);
+    g2 += gcoef<T>(t, 1, 0) * c0;
+    g2 += gcoef<T>(t, 1, 1) * c1;
+    g2 += gcoef<T>(t, 1, 2) * c2;
+    g2 += gcoef<T>(t, 1, 3) * c3;
+    a1 = g1 + c1;
+    a2 = g2 + c2;
+  } else {
+    a1 = c0 + c2;
+    a2 = g1 + c3;
+  }
+}
+
+// neighbour sums along one dimension, class 0: two cells or more from both faces
+template <typename T>
+__device__ __forceinline__ void line_sums(const T* __restrict__ xb, int o, int st, bool inner, int g, int n, int tlo,
+                                          int thi, T& a1, T& a2) {
+  if (inner) {
+    a1 = xb[o - st] + xb[o + st];
+    a2 = xb[o - 2 * st] + xb[o + 2 * st];
+  } else {
+    face_sums<T>(xb, o, st, g, n, tlo, thi, a1, a2);
+  }
+}
+
+// The transposed operator's sums along one dimension (cell_Lx with TR): zero outside the domain,
+// and in the four cells next to a face ``ex`` gathers the ghost coefficients of the two rows
+// that read the ghosts.  i: patch-local index, n: domain, [plo, plo + pn): the patch.
+template <typename T>
+__device__ __forceinline__ void trans_sums(const T* __restrict__ xb, int o, int st, int i, int n, int plo, int pn, int tlo,
+                                           int thi, T& a1, T& a2, T& ex) {
+  const int g = plo + i;
+  const T m1 = g >= 1 ? xb[o - st] : T(0), p1 = g + 1 < n ? xb[o + st] : T(0);
+  const T m2 = g >= 2 ? xb[o - 2 * st] : T(0), p2 = g + 2 < n ? xb[o + 2 * st] : T(0);
+  a1 = m1 + p1;
+  a2 = m2 + p2;
+  if (g <= 3 && plo == 0) {
+    const int f = o - i * st;
+    const T w1 = T(16) * xb[f] - xb[f + st], w2 = -xb[f];
+    ex += gcoef<T>(tlo, 0, g) * w1 + gcoef<T>(tlo, 1, g) * w2;
+  }
+  const int m = n - 1 - g;
+  if (m <= 3 && plo + pn == n) {
+    const int f = o + (pn - 1 - i) * st;
+    const T w1 = T(16) * xb[f] - xb[f - st], w2 = -xb[f];
+    ex += gcoef<T>(thi, 0, m) * w1 + gcoef<T>(thi, 1, m) * w2;
+  }
+}
+
+// f - A x (or f - A^T x) coefficients and sums of one cell near a face, 2-D, homogeneous data
+template <typename T, int MODE, bool TR>
+__device__ __forceinline__ void edge_op2d(const LevelView& lv, const PatchDesc& p, int i, int j, const T* __restrict__ x,
+                                          const T* __restrict__ f, T* __restrict__ out, T alpha, T beta,
+                                          const JFac<T, 2>& jf) {
+  const int sy = (int)p.sy, o = (j + NG) * sy + i + NG;
+  const int gx = p.lo[0] + i, gy = p.lo[1] + j;
+  const int cx = face_class(gx, lv.ndom[0]), cy = face_class(gy, lv.ndom[1]);
+  if (MODE == OP_JACOBI0) {
+    out[p.off + o] = jf.w[cx + 5 * cy] * f[p.off + o];
+    return;
+  }
+  const T* __restrict__ xb = x + p.off;
+  const T xc = xb[o];
+  T fk = T(0);
+  if (MODE != OP_APPLY) fk = f[p.off + o];
+  T x1, x2, y1, y2, ex = T(0);
+  if (TR) {
+    trans_sums<T>(xb, o, 1, i, lv.ndom[0], p.lo[0], p.n[0], lv.bc[0], lv.bc[1], x1, x2, ex);
+    trans_sums<T>(xb, o, sy, j, lv.ndom[1], p.lo[1], p.n[1], lv.bc[2], lv.bc[3], y1, y2, ex);
+  } else {
+    line_sums<T>(xb, o, 1, cx == 0, gx, lv.ndom[0], lv.bc[0], lv.bc[1], x1, x2);
+    line_sums<T>(xb, o, sy, cy == 0, gy, lv.ndom[1], lv.bc[2], lv.bc[3], y1, y2);
+  }
+  const T s1 = x1 + y1, s2 = x2 + y2;
+  const T inv = pick<T>(lv.inv12h2, lv.inv12h2_f);
+  const T ax = alpha * xc + beta * (((T(16) * s1 - s2 - T(60) * xc) + ex) * inv);
+  if (MODE == OP_APPLY) out[p.off + o] = ax;
+  else if (MODE == OP_RESID) out[p.off + o] = fk - ax;
+  else out[p.off + o] = xc + jf.w[cx + 5 * cy] * (fk - ax);
+}
+
 template <typename T, int D, int MODE, bool TR = false>
 __global__ void __launch_bounds__(BX* BY) k_level_op(LevelView lv, int nby, const T* __restrict__ x,
                                                      const T* __restrict__ f, T* __restrict__ out,
@@ -286,7 +399,8 @@ template <typename T, int MODE, bool TR, int ROWS>
 __device__ __forceinline__ void level_op2d_tiled_body(const LevelView& lv, int pz, const T* __restrict__ x,
                                                       const T* __restrict__ f, T* __restrict__ out,
                                                       const T* __restrict__ bc, T alpha, T beta, T omega,
-                                                      T omega_over_diag, const unsigned char* __restrict__ vmask) {
+                                                      T omega_over_diag, const unsigned char* __restrict__ vmask,
+                                                      const JFac<T, 2>& jf) {
   const PatchDesc p = lv.patches[pz];
   const int i = blockIdx.x * BX + threadIdx.x;
   const int j0 = (blockIdx.y * BY + threadIdx.y) * ROWS;
@@ -302,7 +416,9 @@ __device__ __forceinline__ void level_op2d_tiled_body(const LevelView& lv, int p
       const int j = j0 + r;
       if (j >= p.n[1]) return;
       if (vmask != nullptr && vmask[poff(p, i, j, 0)] == 0) continue;
-      cell_level_op<T, 2, MODE, TR>(lv, p, i, j, 0, x, f, out, bc, alpha, beta, omega);
+      if (bc != nullptr)
+        cell_level_op<T, 2, MODE, TR>(lv, p, i, j, 0, x, f, out, bc, alpha, beta, omega);
+      else edge_op2d<T, MODE, TR>(lv, p, i, j, x, f, out, alpha, beta, jf);
     }
     return;
   }
@@ -352,15 +468,10 @@ template <typename T, int MODE, bool TR, int ROWS>
 __global__ void __launch_bounds__(BX* BY) k_level_op2d_tiled(LevelView lv, const T* __restrict__ x,
                                                              const T* __restrict__ f, T* __restrict__ out,
                                                              const T* __restrict__ bc, T alpha, T beta, T omega,
-                                                             T omega_over_diag, const unsigned char* __restrict__ vmask) {
+                                                             T omega_over_diag, const unsigned char* __restrict__ vmask,
+                                                             const __grid_constant__ JFac<T, 2> jf) {
   pdl_wait();
-  level_op2d_tiled_body<T, MODE, TR, ROWS>(lv, blockIdx.z, x, f, out, bc, alpha, beta, omega, omega_over_diag, vmask);
-}
-
-// distance class of global index g to the faces of an n-cell dimension: 0 interior, 1 and 2
-// the first and second cell from the low face, 3 and 4 from the high face
-__device__ __forceinline__ int face_class(int g, int n) {
-  return g == 0 ? 1 : g == 1 ? 2 : g == n - 1 ? 3 : g == n - 2 ? 4 : 0;
+  level_op2d_tiled_body<T, MODE, TR, ROWS>(lv, blockIdx.z, x, f, out, bc, alpha, beta, omega, omega_over_diag, vmask, jf);
 }
 
 // ------------------------------------------------------------------------ z-chunked 3-D marching operator
@@ -2398,7 +2509,7 @@ __global__ void __launch_bounds__(BX* BY) k_resid2d_b(const BResid* __restrict__
   const BResid& e = d[blockIdx.z];
   if (!active[e.p] || (int)blockIdx.x >= e.tiles_x || (int)blockIdx.y >= e.tiles_y) return;
   level_op2d_tiled_body<double, OP_RESID, false, ROWS>(e.lv, 0, e.x, e.f, e.out, nullptr, e.alpha, e.beta, 0.0, 0.0,
-                                                       nullptr);
+                                                       nullptr, JFac<double, 2>{});
 }
 
 // block-wide max of IEEE bits (non-negative doubles) into *acc

@@ -12,58 +12,7 @@
 
 namespace amr4 {
 
-// Jacobi factors omega / diag by distance class of the cell to the x, y and z faces
-// (face_class; index x + 5 y + 25 z), filled on the host (jacobi_factors).
-template <typename T>
-struct JFac {
-  T w[125];
-};
-
-// Sums of the first and of the second neighbours along one dimension of the cell at offset o,
-// g <= 1 or g >= n - 2 (global index, n cells in the domain): a face cell reads the ghost
-// layers 1 and 2, its neighbour layer 1.  Ghost values in read_nb's order of operations; both
-// sums are commutative, so the low and the high side share one form.
-template <typename T>
-__device__ __forceinline__ void face_sums(const T* __restrict__ xb, int o, int st, int g, int n, int tlo, int thi, T& a1,
-                                          T& a2) {
-  const bool low = g < 2;
-  const int q = low ? g : n - 1 - g;
-  const int s = low ? st : -st;
-  const int t = low ? tlo : thi;
-  const int b = o - q * s;
-  const T c0 = xb[b], c1 = xb[b + s], c2 = xb[b + 2 * s], c3 = xb[b + 3 * s];
-  T g1 = T(0);
-  g1 += gcoef<T>(t, 0, 0) * c0;
-  g1 += gcoef<T>(t, 0, 1) * c1;
-  g1 += gcoef<T>(t, 0, 2) * c2;
-  g1 += gcoef<T>(t, 0, 3) * c3;
-  if (q == 0) {
-    T g2 = T(0);
-    g2 += gcoef<T>(t, 1, 0) * c0;
-    g2 += gcoef<T>(t, 1, 1) * c1;
-    g2 += gcoef<T>(t, 1, 2) * c2;
-    g2 += gcoef<T>(t, 1, 3) * c3;
-    a1 = g1 + c1;
-    a2 = g2 + c2;
-  } else {
-    a1 = c0 + c2;
-    a2 = g1 + c3;
-  }
-}
-
-// neighbour sums along one dimension, class 0: two cells or more from both faces
-template <typename T>
-__device__ __forceinline__ void line_sums(const T* __restrict__ xb, int o, int st, bool inner, int g, int n, int tlo,
-                                          int thi, T& a1, T& a2) {
-  if (inner) {
-    a1 = xb[o - st] + xb[o + st];
-    a2 = xb[o - 2 * st] + xb[o + 2 * st];
-  } else {
-    face_sums<T>(xb, o, st, g, n, tlo, thi, a1, a2);
-  }
-}
-
-// Level operator (OP_APPLY, OP_RESID, OP_JACOBI, OP_JACOBI0; homogeneous data).  A thread owns
+// Level operator (OP_APPLY, OP_RESID, OP_JACOBI, OP_JACOBI0; homogeneous data; TR: its transpose).  A thread owns
 // one (x, y) column of a patch -- columns numbered linearly, so narrow grids fill their warps --
 // and kz planes of it, its z neighbours in a register queue.  The host sizes kz so that small
 // grids spread over every SM (kz = 1 on the coarsest) and large ones keep the queue.
@@ -72,14 +21,14 @@ __device__ __forceinline__ void line_sums(const T* __restrict__ xb, int o, int s
 // the restriction, prolongation and bottom solve below, the FP64 Helmholtz solve on 72^3 + a
 // 56 x 52 x 72 box went from 6.05 to 2.95 ms and the mixed pressure solve on 96 x 80 x 64 with two
 // ragged boxes from 10.1 to 5.8 ms.
-template <typename T, int MODE>
+template <typename T, int MODE, bool TR>
 __global__ void __launch_bounds__(128) k_level_op3d_col(LevelView lv, int kz, const T* __restrict__ x,
-                                                        const T* __restrict__ f, T* __restrict__ out, T alpha, T beta,
-                                                        const __grid_constant__ JFac<T> jf,
+                                                        const T* f, T* out, T alpha, T beta,
+                                                        const __grid_constant__ JFac<T, 3> jf,
                                                         const unsigned char* __restrict__ vmask) {
   const int pz = blockIdx.z;
   const PatchDesc p = lv.npatch == 1 ? lv.p0 : lv.patches[pz];
-  const int col = blockIdx.x * 128 + threadIdx.x;
+  const int col = blockIdx.x * blockDim.x + threadIdx.x;
   const int k0 = blockIdx.y * kz, k1 = min(k0 + kz, p.n[2]);
   if (col >= p.n[0] * p.n[1] || k0 >= k1) {
     pdl_wait();
@@ -89,9 +38,10 @@ __global__ void __launch_bounds__(128) k_level_op3d_col(LevelView lv, int kz, co
   const int sy = (int)p.sy, sz = (int)p.sz;
   const int gx = p.lo[0] + i, gy = p.lo[1] + j, lz = p.lo[2], nzd = lv.ndom[2];
   const int cx = face_class(gx, lv.ndom[0]), cy = face_class(gy, lv.ndom[1]);
+  const bool inx = gx >= 4 && gx <= lv.ndom[0] - 5, iny = gy >= 4 && gy <= lv.ndom[1] - 5;  // transposed: no ghost rows
   const T* __restrict__ xb = x + p.off;
-  const T* __restrict__ fb = f + p.off;
-  T* __restrict__ ob = out + p.off;
+  const T* fb = f + p.off;  // may be out (in-place residual)
+  T* ob = out + p.off;
   const unsigned char* __restrict__ vb = (MODE == OP_RESID && vmask != nullptr) ? vmask + p.off : nullptr;
   int o = (k0 + NG) * sz + (j + NG) * sy + i + NG;
   pdl_wait();
@@ -113,22 +63,46 @@ __global__ void __launch_bounds__(128) k_level_op3d_col(LevelView lv, int kz, co
     const T q4 = (gz + 2 < nzd) ? xb[o + 2 * sz] : T(0);
     T fk = T(0);
     if (MODE != OP_APPLY) fk = fb[o];
-    T x1, x2, y1, y2, z1, z2;
-    line_sums<T>(xb, o, 1, cx == 0, gx, lv.ndom[0], lv.bc[0], lv.bc[1], x1, x2);
-    line_sums<T>(xb, o, sy, cy == 0, gy, lv.ndom[1], lv.bc[2], lv.bc[3], y1, y2);
-    if (cz == 0) {
-      z1 = q1 + q3;
-      z2 = q0 + q4;
+    T x1, x2, y1, y2, z1, z2, ex = T(0);
+    if (TR) {
+      if (inx) {
+        x1 = xb[o - 1] + xb[o + 1];
+        x2 = xb[o - 2] + xb[o + 2];
+      } else {
+        trans_sums<T>(xb, o, 1, i, lv.ndom[0], p.lo[0], p.n[0], lv.bc[0], lv.bc[1], x1, x2, ex);
+      }
+      if (iny) {
+        y1 = xb[o - sy] + xb[o + sy];
+        y2 = xb[o - 2 * sy] + xb[o + 2 * sy];
+      } else {
+        trans_sums<T>(xb, o, sy, j, lv.ndom[1], p.lo[1], p.n[1], lv.bc[2], lv.bc[3], y1, y2, ex);
+      }
+      if (gz >= 4 && gz <= nzd - 5) {
+        z1 = q1 + q3;
+        z2 = q0 + q4;
+      } else {
+        trans_sums<T>(xb, o, sz, k, nzd, lz, p.n[2], lv.bc[4], lv.bc[5], z1, z2, ex);
+      }
     } else {
-      face_sums<T>(xb, o, sz, gz, nzd, lv.bc[4], lv.bc[5], z1, z2);
+      line_sums<T>(xb, o, 1, cx == 0, gx, lv.ndom[0], lv.bc[0], lv.bc[1], x1, x2);
+      line_sums<T>(xb, o, sy, cy == 0, gy, lv.ndom[1], lv.bc[2], lv.bc[3], y1, y2);
+      if (cz == 0) {
+        z1 = q1 + q3;
+        z2 = q0 + q4;
+      } else {
+        face_sums<T>(xb, o, sz, gz, nzd, lv.bc[4], lv.bc[5], z1, z2);
+      }
     }
     const T s1 = (x1 + y1) + z1;
     const T s2 = (x2 + y2) + z2;
     if (vb == nullptr || vb[o]) {
       if (MODE == OP_APPLY) {
-        ob[o] = kc0 * q2 + (kc1 * s1 - kc2 * s2);
+        T v = kc0 * q2 + (kc1 * s1 - kc2 * s2);
+        if (TR) v = fma(kc2, ex, v);
+        ob[o] = v;
       } else {
-        const T r = fma(kc2, s2, fma(-kc1, s1, fma(-kc0, q2, fk)));
+        T r = fma(kc2, s2, fma(-kc1, s1, fma(-kc0, q2, fk)));
+        if (TR) r = fma(-kc2, ex, r);
         if (MODE == OP_RESID) ob[o] = r;
         else ob[o] = fma(jf.w[cx + 5 * cy + 25 * cz], r, q2);
       }
@@ -300,7 +274,7 @@ __global__ void __launch_bounds__(128) k_prolong3d_ext(LevelView fine, LevelView
   pdl_wait();
   const XferBlock b = blocks[blockIdx.z];
   const int w0 = b.chi[0] - b.clo[0] + 1, w1 = b.chi[1] - b.clo[1] + 1;
-  const int col = blockIdx.x * 128 + threadIdx.x;
+  const int col = blockIdx.x * blockDim.x + threadIdx.x;
   const int g2 = b.clo[2] + (int)blockIdx.y;
   if (col >= w0 * w1 || g2 > b.chi[2]) return;
   const int g0 = b.clo[0] + col % w0, g1 = b.clo[1] + col / w0;

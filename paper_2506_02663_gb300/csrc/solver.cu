@@ -21,6 +21,7 @@
 #include "op3d.cuh"
 #include "sweep3d.cuh"
 #include "coarse3d.cuh"
+#include "mgcluster.cuh"
 #include "cic.cuh"
 #include "migrate.cuh"
 
@@ -596,17 +597,17 @@ amr_status launch_resid_fx(const LevelView& lv, const double* x, const double* f
 }
 
 // Jacobi factors omega / diag by distance class (k_level_op3d_zc's device table, same order)
-template <typename T>
-JFac<T> jacobi_factors(const LevelView& lv, double alpha, double beta, double omega) {
-  JFac<T> j;
+template <typename T, int D>
+JFac<T, D> jacobi_factors(const LevelView& lv, double alpha, double beta, double omega) {
+  JFac<T, D> j;
   const T inv = pick_host<T>(lv.inv12h2, lv.inv12h2_f);
-  for (int q = 0; q < 125; ++q) {
+  for (int q = 0; q < (D == 3 ? 125 : 25); ++q) {
     const int cls[3] = {q % 5, (q / 5) % 5, q / 25};
-    T acc = T(-90);
-    for (int d = 0; d < 3; ++d)
+    T acc = T(-30 * D);
+    for (int d = 0; d < D; ++d)
       if (cls[d]) acc += pick_host<T>(lv.dcorr[2 * d + (cls[d] - 1) / 2][(cls[d] - 1) % 2],
                                       lv.dcorr_f[2 * d + (cls[d] - 1) / 2][(cls[d] - 1) % 2]);
-    j.w[q] = T(omega) / (T(alpha) + T(beta) * inv * acc);
+    j.w[q] = T(omega) / std::fma(T(beta) * inv, acc, T(alpha));  // the device tables' contraction, on every host
   }
   return j;
 }
@@ -647,11 +648,12 @@ amr_status level_op(int mode, const LevelView& lv, const T* x, const T* f, T* ou
     dim3 grid((lv.maxn[0] + BX - 1) / BX, (lv.maxn[1] + BY * rows - 1) / (BY * rows), lv.npatch);
     dim3 block(BX, BY, 1);
     const T A = T(alpha), B = T(beta), O = T(omega);
+    const JFac<T, 2> jf = (mode == OP_JACOBI || mode == OP_JACOBI0) ? jacobi_factors<T, 2>(lv, alpha, beta, omega) : JFac<T, 2>{};
 #define LAUNCH_TILED(M)                                                                                     \
   do {                                                                                                      \
-    if (rows == 4) launch(k_level_op2d_tiled<T, M, TR, 4>, grid, block, 0, st, lv, x, f, out, bc, A, B, O, ood, vmask); \
-    else if (rows == 2) launch(k_level_op2d_tiled<T, M, TR, 2>, grid, block, 0, st, lv, x, f, out, bc, A, B, O, ood, vmask); \
-    else launch(k_level_op2d_tiled<T, M, TR, 1>, grid, block, 0, st, lv, x, f, out, bc, A, B, O, ood, vmask); \
+    if (rows == 4) launch(k_level_op2d_tiled<T, M, TR, 4>, grid, block, 0, st, lv, x, f, out, bc, A, B, O, ood, vmask, jf); \
+    else if (rows == 2) launch(k_level_op2d_tiled<T, M, TR, 2>, grid, block, 0, st, lv, x, f, out, bc, A, B, O, ood, vmask, jf); \
+    else launch(k_level_op2d_tiled<T, M, TR, 1>, grid, block, 0, st, lv, x, f, out, bc, A, B, O, ood, vmask, jf); \
   } while (0)
     switch (mode) {
       case OP_APPLY: LAUNCH_TILED(OP_APPLY); break;
@@ -709,23 +711,24 @@ amr_status level_op(int mode, const LevelView& lv, const T* x, const T* f, T* ou
              nb * sizeof(T) * lv.ncells, lv.ncells);
     return launch_check();
   }
-  if constexpr (D == 3 && !TR) {
-    if (bc == nullptr && small_offsets(lv)) {
+  if constexpr (D == 3) {
+    if (bc == nullptr && (!TR || vmask == nullptr) && small_offsets(lv)) {
       // any other homogeneous 3-D level: one thread per column and run of kz planes, as many runs
       // as give every SM 16 warps (a quarter of its slots: enough loads in flight for L2, and long
       // runs where the grid allows them)
       const long long warps = (long long)lv.npatch * ((lv.maxn[0] * (long long)lv.maxn[1] + 31) / 32);
-      const long long want = 16LL * sm_count();
+      const long long want = 32LL * sm_count();
       const int nz = lv.maxn[2];
       const int kz = (int)std::max<long long>(1, std::min<long long>(nz, (warps * nz + want - 1) / want));
-      const dim3 grid((unsigned)((lv.maxn[0] * (long long)lv.maxn[1] + 127) / 128), (nz + kz - 1) / kz, lv.npatch);
-      const JFac<T> jf = (mode == OP_JACOBI || mode == OP_JACOBI0) ? jacobi_factors<T>(lv, alpha, beta, omega) : JFac<T>{};
+      constexpr int cb = 64;
+      const dim3 grid((unsigned)((lv.maxn[0] * (long long)lv.maxn[1] + cb - 1) / cb), (nz + kz - 1) / kz, lv.npatch);
+      const JFac<T, 3> jf = (mode == OP_JACOBI || mode == OP_JACOBI0) ? jacobi_factors<T, 3>(lv, alpha, beta, omega) : JFac<T, 3>{};
       const T A = T(alpha), B = T(beta);
       switch (mode) {
-        case OP_APPLY: launch(k_level_op3d_col<T, OP_APPLY>, grid, 128, 0, st, lv, kz, x, f, out, A, B, jf, vmask); break;
-        case OP_RESID: launch(k_level_op3d_col<T, OP_RESID>, grid, 128, 0, st, lv, kz, x, f, out, A, B, jf, vmask); break;
-        case OP_JACOBI: launch(k_level_op3d_col<T, OP_JACOBI>, grid, 128, 0, st, lv, kz, x, f, out, A, B, jf, vmask); break;
-        default: launch(k_level_op3d_col<T, OP_JACOBI0>, grid, 128, 0, st, lv, kz, x, f, out, A, B, jf, vmask);
+        case OP_APPLY: launch(k_level_op3d_col<T, OP_APPLY, TR>, grid, cb, 0, st, lv, kz, x, f, out, A, B, jf, vmask); break;
+        case OP_RESID: launch(k_level_op3d_col<T, OP_RESID, TR>, grid, cb, 0, st, lv, kz, x, f, out, A, B, jf, vmask); break;
+        case OP_JACOBI: launch(k_level_op3d_col<T, OP_JACOBI, TR>, grid, cb, 0, st, lv, kz, x, f, out, A, B, jf, vmask); break;
+        default: launch(k_level_op3d_col<T, OP_JACOBI0, TR>, grid, cb, 0, st, lv, kz, x, f, out, A, B, jf, vmask);
       }
       const double nb = mode == OP_JACOBI0 ? 2.0 : (mode == OP_APPLY ? 2.0 : 3.0);
       prof_end(st, ev, (mode == OP_JACOBI || mode == OP_JACOBI0) ? PC_JACOBI : (mode == OP_RESID && sizeof(T) == 8) ? PC_RESID64 : PC_RESID,
@@ -791,8 +794,9 @@ amr_status prolong_blocks(const LevelView& fine, const LevelView& crs, const Xfe
   } else {
     // a 3-D patch beyond 2^31 elements takes the generic kernel
     if (small_offsets(fine) && xmax[2] <= 65535) {
-      dim3 grid((unsigned)(((long long)xmax[0] * xmax[1] + 127) / 128), xmax[2], nblocks);
-      launch(k_prolong3d_ext<T>, grid, 128, 0, st, fine, crs, blocks, xc, xf, xf2);
+      constexpr int nt = 64;
+      dim3 grid((unsigned)(((long long)xmax[0] * xmax[1] + nt - 1) / nt), xmax[2], nblocks);
+      launch(k_prolong3d_ext<T>, grid, nt, 0, st, fine, crs, blocks, xc, xf, xf2);
     } else {
       const int fy = 2 * xmax[1];
       const int nby = (fy + BY - 1) / BY;
@@ -809,7 +813,7 @@ template <typename T, int D>
 amr_status cfi_fill(const amr_hierarchy* h, int l, const T* xc, T* xf, bool zero, cudaStream_t st) {
   const DeviceLists& dl = h->lev[l].dev;
   if (dl.ncfi == 0) return AMR_OK;
-  const int nt = 128;
+  const int nt = 32;  // one warp per block: a few hundred warps of FP64 work spread over every SM
   if (dl.ncfig > 0) {  // ratio 2: by coarse parent
     const CfiGroup* list = dl.cfig;
     long long n = dl.ncfig;
@@ -856,7 +860,7 @@ amr_status reflux(const amr_hierarchy* h, int l, const LevelView& crs, const Lev
                   P3<T> bcs, T* out, double coef, int kind, cudaStream_t st) {
   const DeviceLists& dl = h->lev[l].dev;
   if (dl.nreflux == 0) return AMR_OK;
-  const int nt = 128;
+  const int nt = 32;  // as above
   launch(k_reflux_p3<T, D>, (unsigned)((dl.nreflux + nt - 1) / nt), nt, 0, st, crs, fine, dl.reflux, dl.nreflux, xc, xf,
                                                                          bcs, out, T(coef), kind);
   return launch_check();
@@ -1498,6 +1502,161 @@ amr_status coarse_cluster(amr_operator* op, const amr_solver_params& p, int m0, 
 }
 static_assert(sizeof(CoarseCluster) + sizeof(CoarsePtrs<double>) < 30000, "kernel parameter block too large");
 
+// ---------------------------------------------------------------- cluster coarse end in shared memory
+// Blocks per cluster of k_mg_cluster: 16 where the device schedules a cluster that large with
+// this much shared memory, else 8 (queried once per device and kernel).
+constexpr size_t MC_SMEM = 160 * 1024;  // shared memory per block the grids may take
+template <typename T, int D, bool TR>
+int mg_cluster_size() {
+  static std::mutex mu;
+  static std::map<int, int> cache;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lock(mu);
+  auto it = cache.find(dev);
+  if (it != cache.end()) return it->second;
+  int cs = 0;
+  if (cudaFuncSetAttribute(k_mg_cluster<T, D, TR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MC_SMEM) == cudaSuccess &&
+      cudaFuncSetAttribute(k_mg_cluster<T, D, TR>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
+    for (int want : {16, 8}) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(want, 1, 1);
+      cfg.blockDim = dim3(MC_THREADS, 1, 1);
+      cfg.dynamicSmemBytes = MC_SMEM;
+      cudaLaunchAttribute a[1];
+      a[0].id = cudaLaunchAttributeClusterDimension;
+      a[0].val.clusterDim.x = want;
+      a[0].val.clusterDim.y = 1;
+      a[0].val.clusterDim.z = 1;
+      cfg.attrs = a;
+      cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, k_mg_cluster<T, D, TR>, &cfg) == cudaSuccess && n >= 1) {
+        cs = want;
+        break;
+      }
+    }
+  cudaGetLastError();
+  cache[dev] = cs;
+  return cs;
+}
+
+// Grids of the cluster V-cycle from m on: slabs per block and their shared-memory offsets.
+// Returns the bytes per block, 0 when grid m cannot start it.  A grid takes as many blocks as
+// keep ``min_cells`` cells each (below that remote reads cost more than the extra block saves).
+template <typename T, int D>
+size_t mg_cluster_layout(const amr_hierarchy* h, int m, int cs, int min_cells, MgCluster<T, D>* c) {
+  const int M = (int)h->mg.size() - 1;
+  if (M - m + 1 > MC_MAX || m >= M) return 0;
+  long long off = 0;
+  for (int q = 0; q <= M - m; ++q) {
+    const MgGrid& g = h->mg[m + q];
+    const int ns = g.n[D - 1], P = g.n[0] * (D == 3 ? g.n[1] : 1);
+    for (int d = 0; d < D; ++d)
+      if (q < M - m && g.n[d] < 8) return 0;  // both faces' cells have bands of their own
+    const int R = std::min(ns, std::max((ns + cs - 1) / cs, (min_cells + P - 1) / P));
+    const int mul = (65536 + R - 1) / R;
+    for (int k = 0; k < ns; ++k)
+      if (((k * mul) >> 16) != k / R) return 0;
+    if (c != nullptr) {
+      for (int d = 0; d < 3; ++d) c->n[q][d] = g.n[d];
+      c->R[q] = R;
+      c->mul[q] = mul;
+      c->off[q] = (int)off;
+    }
+    off += 3ll * R * P;
+    if (off * (long long)sizeof(T) > (long long)MC_SMEM) return 0;
+  }
+  return (size_t)off * sizeof(T);
+}
+
+// First grid of the cluster V-cycle, -1 for none: the finest within the size limit.  FP64 work
+// is bound by 16 SMs' FP64 rate beyond about 4096 cells (2-D; a sweep launched over the whole
+// chip is faster there), FP32 work by the 16 SMs' issue slots beyond about 32^3 cells.
+constexpr long long MC_CELLS64 = 4096, MC_CELLS32 = 32768;
+constexpr int MC_MIN = 64;  // cells a block takes at least (64: poisson 64^2 1.98 ms; 32: 1.97, 128: 2.01, 1024 with FP32 grids: 3 % slower)
+template <typename T, int D, bool TR>
+int mg_cluster_m0(const amr_operator* op) {
+  const amr_hierarchy* h = op->h;
+  if (h->ncomp != 1 || op->nbot > MC_BOT) return -1;
+  const int cs = mg_cluster_size<T, D, TR>();
+  if (cs == 0) return -1;
+  int m0 = -1;
+  for (int m = (int)h->mg.size() - 2; m >= 0; --m) {
+    const MgGrid& g = h->mg[m];
+    if ((long long)g.n[0] * g.n[1] * g.n[2] > (sizeof(T) == 8 ? MC_CELLS64 : MC_CELLS32)) break;
+    if (mg_cluster_layout<T, D>(h, m, cs, MC_MIN, nullptr) == 0) break;
+    m0 = m;
+  }
+  return m0;
+}
+
+template <typename T, int D, bool TR>
+amr_status mg_cluster(amr_operator* op, const amr_solver_params& p, int m0, const T* b, T* x, cudaStream_t st) {
+  const amr_hierarchy* h = op->h;
+  const int cs = mg_cluster_size<T, D, TR>();
+  MgCluster<T, D> c{};
+  const size_t smem = mg_cluster_layout<T, D>(h, m0, cs, MC_MIN, &c);
+  c.ng = (int)h->mg.size() - m0;
+  c.nu1 = p.nu1;
+  c.nu2 = p.nu2;
+  c.nbot = op->nbot;
+  c.ldb = op->ldb;
+  c.minv = TR ? op->d_binvT : op->d_binv;
+  c.gp = h->mg[m0].patch;
+  c.alpha = T(op->alpha);
+  for (int q = 0; q < c.ng; ++q) {
+    const LevelView lv = mg_view(h, m0 + q, op->bc);
+    c.kc[q] = T(op->beta) * pick_host<T>(lv.inv12h2, lv.inv12h2_f);
+    const JFac<T, D> jf = jacobi_factors<T, D>(lv, op->alpha, op->beta, p.omega);
+    std::memcpy(c.wt[q], jf.w, sizeof(jf.w));
+  }
+  // bands per dimension: rows 0 and 1 of the 1-D operator with the ghost formulas substituted
+  const double in[5] = {-1.0, 16.0, -30.0, 16.0, -1.0};
+  for (int d = 0; d < D; ++d) {
+    for (int q = 0; q < 5; ++q) c.band[d][0][q] = T(in[q]);
+    for (int side = 0; side < 2; ++side) {
+      const int t = op->bc[2 * d + side] == 1 ? 1 : 0;
+      double row[6][8] = {};  // rows 0 .. 5 over cells 0 .. 7 from the face
+      for (int i = 0; i < 6; ++i)
+        for (int q = 0; q < 5; ++q) {
+          const int e = i + q - 2;
+          if (e >= 0) row[i][e] += in[q];
+          else
+            for (int k = 0; k < 4; ++k) row[i][k] += in[q] * HG[t][-e - 1][k];
+        }
+      for (int i = 0; i < (TR ? 4 : 2); ++i)
+        for (int k = 0; k < 6; ++k) c.band[d][1 + 4 * side + i][k] = T(TR ? row[k][i] : row[i][k]);
+    }
+    for (int side = 0; side < 2; ++side)
+      for (int k = 0; k < 4; ++k) c.ghost[2 * d + side][k] = T(HG[op->bc[2 * d + side] == 1 ? 1 : 0][0][k]);
+  }
+  cudaEvent_t ev;
+  prof_begin(st, &ev);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cs, 1, 1);
+  cfg.blockDim = dim3(MC_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cs;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_mg_cluster<T, D, TR>, c, b, x);
+  if (e != cudaSuccess && g_launch_err == cudaSuccess) g_launch_err = e;
+  TRY(launch_check());
+  const MgGrid& g = h->mg[m0];
+  const double cells = (double)g.n[0] * g.n[1] * g.n[2];
+  prof_end(st, ev, PC_COARSE, 2.0 * sizeof(T) * cells, cells);  // read f, write x of the top grid
+  return AMR_OK;
+}
+static_assert(sizeof(MgCluster<double, 3>) < 30000, "kernel parameter block too large");
+
 // ---------------------------------------------------------------- level-0 multigrid
 template <typename T, int D, bool TR = false>
 amr_status mg_level0(amr_operator* op, const amr_solver_params& p, int m, const T* b, T* x, T* t, cudaStream_t st) {
@@ -1511,11 +1670,16 @@ amr_status mg_level0(amr_operator* op, const amr_solver_params& p, int m, const 
     TRY((fused_config<T, D, TR>(op, m0, bytes)));
     if (m == m0) return fused_coarse<T, D, TR>(op, p, m0, bytes, b, x, st);
   }
+  // default: the coarse end in one cluster's shared memory (FP32 2-D forward V-cycles with blocked
+  // legs keep their one-block coarse kernels)
+  if (p.fuse_coarse == 0 && p.nu1 >= 1 && !(D == 2 && sizeof(T) == 4 && !TR && p.temporal_blocking) &&
+      m == mg_cluster_m0<T, D, TR>(op))
+    return mg_cluster<T, D, TR>(op, p, m, b, x, st);
   if constexpr (D == 3) {
     // fuse_coarse = 2: the coarse end of the pyramid in one cluster launch
     if (p.fuse_coarse == 2 && h->ncomp == 1 && m == coarse_cluster_m0(h))
       return coarse_cluster<T, D, TR>(op, p, m, b, x, t, st);
-    // default: a 16^3, 8^3, 4^3 coarse end of an FP32 forward V-cycle in one block
+    // where no cluster can be scheduled: a 16^3, 8^3, 4^3 coarse end of an FP32 forward V-cycle in one block
     if constexpr (sizeof(T) == 4 && !TR)
       if (p.fuse_coarse == 0 && p.nu1 >= 1 && cube_pyramid(op, m)) return cube_coarse<T>(op, p, m, b, x, st);
   }
