@@ -1678,6 +1678,16 @@ __device__ __forceinline__ T lap_smem(const T* __restrict__ a, int o, int sy) {
   return (T(16) * s1 - s2 - T(60) * xc) + T(0);
 }
 
+// f - (alpha x + beta L x) at smem offset o: kc0 = alpha - 60 kc2, kc1 = 16 kc2, kc2 = beta /
+// (12 h^2); the operations of the streamed legs (stream2d.cuh), so that a leg's result does not
+// depend on which of the two forms runs it
+template <typename T>
+__device__ __forceinline__ T resid_smem(const T* __restrict__ a, int o, int sy, T f, T kc0, T kc1, T kc2) {
+  const T s1 = (a[o - 1] + a[o + 1]) + (a[o - sy] + a[o + sy]);
+  const T s2 = (a[o - 2] + a[o + 2]) + (a[o - 2 * sy] + a[o + 2 * sy]);
+  return fma(kc2, s2, fma(-kc1, s1, fma(-kc0, a[o], f)));
+}
+
 // f(i, j) for every cell of a w x h box of a block (rows of 32 threads, NT in all).  RM = 0: rows of 32
 // threads stride over the box; RM > 0 (w, h <= RM, a compile-time bound): one linear pass
 // over RM x RM positions with a fixed trip count, positions outside the box skipped.
@@ -1708,7 +1718,7 @@ template <typename T, bool ZERO, int RM = 0, int NT = 256>
 __device__ __forceinline__ T* smooth_region(const LevelView& lv, const TileGeom& tg, const JacobiTable& jt, int sy,
                                             T* cur, T* oth, const T* __restrict__ sb, int nu, T alpha, T beta,
                                             const Team& tm) {
-  const T inv = pick<T>(lv.inv12h2, lv.inv12h2_f);
+  const T kc2 = beta * pick<T>(lv.inv12h2, lv.inv12h2_f), kc1 = T(16) * kc2, kc0 = fma(T(-60), kc2, alpha);
   if constexpr (RM > 0) {
     constexpr int SY = RM + 2 * NG;
     const bool face = tg.fl0 | tg.fh0 | tg.fl1 | tg.fh1;
@@ -1729,9 +1739,7 @@ __device__ __forceinline__ T* smooth_region(const LevelView& lv, const TileGeom&
         if (zero) {
           oth[o] = w * sb[o];
         } else {
-          const T xc = cur[o];
-          const T ax = alpha * xc + beta * (lap_smem(cur, o, SY) * inv);
-          oth[o] = xc + w * (sb[o] - ax);
+          oth[o] = fma(w, resid_smem(cur, o, SY, sb[o], kc0, kc1, kc2), cur[o]);
         }
       });
       __syncthreads();
@@ -1760,9 +1768,7 @@ __device__ __forceinline__ T* smooth_region(const LevelView& lv, const TileGeom&
         if (zero) {
           oth[o] = w * sb[o];
         } else {
-          const T xc = cur[o];
-          const T ax = alpha * xc + beta * (lap_smem(cur, o, sy) * inv);
-          oth[o] = xc + w * (sb[o] - ax);
+          oth[o] = fma(w, resid_smem(cur, o, sy, sb[o], kc0, kc1, kc2), cur[o]);
         }
       }
     }
@@ -1814,7 +1820,7 @@ __device__ __forceinline__ void mg_down2d_body(const LevelView& lv, const PatchD
     region_ghosts(lv, tg, cur, sy, c0, d0, c1, d1, tm);
     __syncthreads();
   }
-  const T inv = pick<T>(lv.inv12h2, lv.inv12h2_f);
+  const T kc2 = beta * pick<T>(lv.inv12h2, lv.inv12h2_f), kc1 = T(16) * kc2, kc0 = fma(T(-60), kc2, alpha);
   const int cw = tg.tw / 2, ch = tg.th / 2;
   const int csy = (int)gcp.sy;
   T* __restrict__ cg = bcn + gcp.off;
@@ -1825,8 +1831,7 @@ __device__ __forceinline__ void mg_down2d_body(const LevelView& lv, const PatchD
 #pragma unroll
       for (int q0 = 0; q0 < 2; ++q0) {
         const int o = (tj + 2 * cj + q1 + NG) * sy + (ti + 2 * ci + q0 + NG);
-        const T xc = cur[o];
-        acc += sb[o] - (alpha * xc + beta * (lap_smem(cur, o, sy) * inv));
+        acc += resid_smem(cur, o, sy, sb[o], kc0, kc1, kc2);
       }
     cg[(((gp.lo[1] + tg.j0) >> 1) - gcp.lo[1] + cj + NG) * csy + ((gp.lo[0] + tg.i0) >> 1) - gcp.lo[0] + ci + NG] =
         acc * T(0.25);

@@ -22,6 +22,7 @@
 #include "sweep3d.cuh"
 #include "coarse3d.cuh"
 #include "mgcluster.cuh"
+#include "stream2d.cuh"
 #include "cic.cuh"
 #include "migrate.cuh"
 
@@ -1242,6 +1243,52 @@ size_t blk_smem_fx(const int* n, int nu, bool down) {
   return (size_t)3 * rm * rm * sizeof(T);
 }
 
+// Streamed legs (k_leg2d): FP32, four sweeps, columns in groups of four, whole coarse rows.
+// Below LEG_MIN_CELLS a leg has too few strips and rows to fill the chip and the tiled form,
+// with a block per 16^2 cells, is faster.
+constexpr long long LEG_MIN_CELLS = 768ll * 768;
+inline bool leg_shape(const int* n) { return n[0] % 4 == 0 && n[1] % 2 == 0 && n[0] >= 16 && n[1] >= 16; }
+template <typename T>
+bool leg_ok(const int* n, int nu) {
+  return sizeof(T) == 4 && nu == LEG_NU && leg_shape(n) && (long long)n[0] * n[1] >= LEG_MIN_CELLS;
+}
+
+// Geometry and coefficients of one streamed leg; ``share``: warps it should split into.
+inline Leg2D make_leg(int mode, const LevelView& lv, const LevelView* cv, const PatchDesc& gp, const PatchDesc& gcp,
+                      double alpha, double beta, double omega, long long share) {
+  Leg2D d{};
+  d.gp = gp;
+  d.gcp = gcp;
+  d.nd0 = lv.ndom[0];
+  d.nd1 = lv.ndom[1];
+  const int hx = mode == LEG_DOWN ? leg_hx<LEG_DOWN>() : leg_hx<LEG_UP>();
+  d.ns = leg_strips(gp.n[0], hx);
+  // rows per chunk: as many chunks as the share allows, at least 32 rows each (18 are halo)
+  const long long nch = std::max<long long>(1, share / d.ns);
+  d.ch = (int)std::max<long long>(32, (gp.n[1] + nch - 1) / nch + 1 & ~1ll);
+  d.nch = (gp.n[1] + d.ch - 1) / d.ch;
+  d.kc2 = (float)beta * lv.inv12h2_f;
+  d.kc1 = 16.0f * d.kc2;
+  d.kc0 = std::fma(-60.0f, d.kc2, (float)alpha);
+  const JFac<float, 2> jf = jacobi_factors<float, 2>(lv, alpha, beta, omega);
+  std::memcpy(d.wt, jf.w, sizeof(d.wt));
+  d.wt[0] = (float)(omega / (alpha - 60.0 * beta * lv.inv12h2));  // as the tiled legs' table
+  for (int f = 0; f < 4; ++f) {
+    const int e = f / 2;
+    const bool face = f % 2 == 0 ? gp.lo[e] == 0 : gp.lo[e] + gp.n[e] == lv.ndom[e];
+    for (int l = 0; l < 2; ++l)
+      for (int m = 0; m < 4; ++m) d.g[f][l][m] = face ? (float)HG[lv.bc[f] == 1 ? 1 : 0][l][m] : 0.0f;
+    for (int m = 0; m < 4; ++m) d.cg[f][m] = cv != nullptr ? (float)HG[cv->bc[f] == 1 ? 1 : 0][0][m] : 0.0f;
+  }
+  return d;
+}
+inline long long leg_share() { return 12ll * sm_count(); }  // resident warps: three blocks of four per SM
+template <int MODE>
+amr_status launch_leg(const Leg2D& d, cudaStream_t st) {
+  launch(k_leg2d<MODE>, (unsigned)((d.ns * d.nch + LEG_WARPS - 1) / LEG_WARPS), 32 * LEG_WARPS, 0, st, d);
+  return launch_check();
+}
+
 template <typename T>
 amr_status blk_attrs() {
   static bool done = false;
@@ -1709,15 +1756,32 @@ amr_status mg_level0(amr_operator* op, const amr_solver_params& p, int m, const 
     cudaEvent_t ev;
     prof_begin(st, &ev);
     (void)blk;
-    launch_down2d<T>(tt, p.nu1, grid, blk_smem_fx<T>(g.n, p.nu1, true), st, lv, g.patch, gc.patch, tt, tt, hd, p.nu1, b, t,
-                     (T*)nullptr, S.mb[m + 1], T(op->alpha), T(op->beta), T(p.omega), ood);
-    TRY(launch_check());
+    if (leg_ok<T>(g.n, p.nu1)) {
+      Leg2D d = make_leg(LEG_DOWN, lv, nullptr, g.patch, gc.patch, op->alpha, op->beta, p.omega, leg_share());
+      d.b = b + g.patch.off;
+      d.xo = t + g.patch.off;
+      d.bcn = S.mb[m + 1] + gc.patch.off;
+      TRY(launch_leg<LEG_DOWN>(d, st));
+    } else {
+      launch_down2d<T>(tt, p.nu1, grid, blk_smem_fx<T>(g.n, p.nu1, true), st, lv, g.patch, gc.patch, tt, tt, hd, p.nu1, b, t,
+                       (T*)nullptr, S.mb[m + 1], T(op->alpha), T(op->beta), T(p.omega), ood);
+      TRY(launch_check());
+    }
     prof_end(st, ev, PC_DOWN, (2.0 + 0.25) * sizeof(T) * cells);  // read f, write x, write coarse f
     TRY(mg_level0<T, D, TR>(op, p, m + 1, S.mb[m + 1], S.mx[m + 1], S.mt[m + 1], st));
     prof_begin(st, &ev);
-    launch_up2d<T>(tt, p.nu2, grid, blk_smem_fx<T>(g.n, p.nu2, false), st, lv, cv, g.patch, gc.patch, tt, tt, hu, p.nu2,
-                   (const T*)S.mx[m + 1], (const T*)b, (const T*)t, x, T(op->alpha), T(op->beta), T(p.omega), ood);
-    TRY(launch_check());
+    if (leg_ok<T>(g.n, p.nu2)) {
+      Leg2D d = make_leg(LEG_UP, lv, &cv, g.patch, gc.patch, op->alpha, op->beta, p.omega, leg_share());
+      d.b = b + g.patch.off;
+      d.xi = t + g.patch.off;
+      d.xc = S.mx[m + 1] + gc.patch.off;
+      d.xo = x + g.patch.off;
+      TRY(launch_leg<LEG_UP>(d, st));
+    } else {
+      launch_up2d<T>(tt, p.nu2, grid, blk_smem_fx<T>(g.n, p.nu2, false), st, lv, cv, g.patch, gc.patch, tt, tt, hu, p.nu2,
+                     (const T*)S.mx[m + 1], (const T*)b, (const T*)t, x, T(op->alpha), T(op->beta), T(p.omega), ood);
+      TRY(launch_check());
+    }
     prof_end(st, ev, PC_UP, (3.0 + 0.25) * sizeof(T) * cells);  // read x, f, coarse x; write x
     return AMR_OK;
   }
@@ -2045,9 +2109,22 @@ amr_status vcycle_corr(amr_operator* op, const amr_solver_params& p, const T* r,
       dim3 grid((fp.n[0] + tt - 1) / tt, (fp.n[1] + tt - 1) / tt, 1);
       cudaEvent_t ev;
       prof_begin(st, &ev);
-      launch_down2d<T>(tt, p.nu1, grid, blk_smem_fx<T>(fp.n, p.nu1, true), st, lv[l], fp, cpd, tt, tt, hd, p.nu1,
-                       (const T*)S.R, E, acc(l), rc, T(a_), T(b_), T(p.omega), ood);
-      TRY(launch_check());
+      bool streamed = false;
+      if constexpr (sizeof(T) == 4 && D == 2)
+        if (leg_ok<T>(fp.n, p.nu1)) {
+          streamed = true;
+          Leg2D d = make_leg(LEG_DOWN, lv[l], nullptr, fp, cpd, a_, b_, p.omega, leg_share());
+          d.b = S.R + fp.off;
+          d.xo = E + fp.off;
+          d.x2 = acc(l) ? acc(l) + fp.off : nullptr;
+          d.bcn = rc + cpd.off;
+          TRY(launch_leg<LEG_DOWN>(d, st));
+        }
+      if (!streamed) {
+        launch_down2d<T>(tt, p.nu1, grid, blk_smem_fx<T>(fp.n, p.nu1, true), st, lv[l], fp, cpd, tt, tt, hd, p.nu1,
+                         (const T*)S.R, E, acc(l), rc, T(a_), T(b_), T(p.omega), ood);
+        TRY(launch_check());
+      }
       prof_end(st, ev, PC_DOWN, ((acc(l) ? 3.0 : 2.0) + 0.25) * sizeof(T) * (double)fp.n[0] * fp.n[1]);
     } else {
       TRY(smooth_from_zero<T, D>(h, l, lv[l], S.R, E, S.T1, p.nu1, a_, b_, p.omega, true, st));
@@ -2129,9 +2206,21 @@ amr_status vcycle_corr(amr_operator* op, const amr_solver_params& p, const T* r,
       dim3 grid((fp.n[0] + tt - 1) / tt, (fp.n[1] + tt - 1) / tt, 1);
       cudaEvent_t ev;
       prof_begin(st, &ev);
-      launch_post2d<T>(tt, p.nu2, grid, blk_smem_fx<T>(fp.n, p.nu2, false), st, lv[l], fp, tt, tt, hu, p.nu2,
-                       (const T*)S.R, E, acc(l), T(a_), T(b_), T(p.omega), ood);
-      TRY(launch_check());
+      bool streamed = false;
+      if constexpr (sizeof(T) == 4 && D == 2)
+        if (leg_ok<T>(fp.n, p.nu2)) {
+          streamed = true;
+          Leg2D d = make_leg(LEG_POST, lv[l], nullptr, fp, fp, a_, b_, p.omega, leg_share());
+          d.b = S.R + fp.off;
+          d.xo = E + fp.off;
+          d.x2 = acc(l) ? acc(l) + fp.off : nullptr;
+          TRY(launch_leg<LEG_POST>(d, st));
+        }
+      if (!streamed) {
+        launch_post2d<T>(tt, p.nu2, grid, blk_smem_fx<T>(fp.n, p.nu2, false), st, lv[l], fp, tt, tt, hu, p.nu2,
+                         (const T*)S.R, E, acc(l), T(a_), T(b_), T(p.omega), ood);
+        TRY(launch_check());
+      }
       prof_end(st, ev, PC_UP, (acc(l) ? 5.0 : 3.0) * sizeof(T) * (double)fp.n[0] * fp.n[1]);  // r in; e (and x) read and written
     } else {
       TRY(smooth_from_zero<T, D>(h, l, lv[l], S.R, S.T1, S.T2, p.nu2, a_, b_, p.omega, true, st));
@@ -3043,6 +3132,7 @@ struct BatchPlan {
   int n = 0, kmax = 0;
   std::vector<BatchGroup> down, up;  // per (m, tile) group, down in increasing m, up in decreasing m
   BatchGroup coarse, resid, flat;
+  Leg2D* d_leg = nullptr;  // streamed legs (groups with tt = 0)
   BDown* d_down = nullptr;
   BUp* d_up = nullptr;
   BCoarse* d_coarse = nullptr;
@@ -3058,7 +3148,7 @@ struct BatchPlan {
   long long launches_pre = 0, launches_body = 0;
   void release() {
     if (exec) cudaGraphExecDestroy(exec);
-    cudaFree(d_down); cudaFree(d_up); cudaFree(d_coarse); cudaFree(d_resid); cudaFree(d_flat);
+    cudaFree(d_leg); cudaFree(d_down); cudaFree(d_up); cudaFree(d_coarse); cudaFree(d_resid); cudaFree(d_flat);
     cudaFree(d_active); cudaFree(d_bits); cudaFree(d_stats);
     if (h_stats) cudaFreeHost(h_stats);
     if (h_bits) cudaFreeHost(h_bits);
@@ -3095,6 +3185,10 @@ amr_status upload(D** dst, const std::vector<D>& v) {
 // where the halo recomputation of a tile (a 36^2 region for 16^2 cells, 52^2 for 32^2) is
 // the cost, so the batch takes 32^2 tiles
 inline int batch_tile(const int*) { return 32; }
+// smallest extent of a streamed leg in a batch: a leg of a smaller grid is bound by one warp's
+// 50 dependent row steps (96 problems of 64^2 .. 512^2: 7.4 ms with 300, 7.7 ms without
+// streaming, 8.4 ms with 200, 9.3 ms with 96)
+constexpr int LEG_BATCH_MIN = 300;
 
 // descriptors of every phase, grouped into launches
 amr_status build_batch_lists(BatchPlan& B) {
@@ -3113,13 +3207,54 @@ amr_status build_batch_lists(BatchPlan& B) {
   auto group_of = [](std::vector<BatchGroup>& gs, int off, int cnt, int tx, int ty, int tt) {
     if (cnt > 0) gs.push_back(BatchGroup{off, cnt, tx, ty, tt});
   };
+  // streamed legs of depth m: one entry per problem, rows split so that the launch fills the chip
+  std::vector<Leg2D> leg;
+  auto streamed = [&](int k, int m, int nu) {
+    const int* n = B.ops[k]->h->mg[m].n;
+    return nu == LEG_NU && leg_shape(n) && n[0] >= LEG_BATCH_MIN && n[1] >= LEG_BATCH_MIN;
+  };
+  auto leg_group = [&](int m, int mode) {
+    const int off = (int)leg.size(), nu = mode == LEG_DOWN ? p.nu1 : p.nu2;
+    long long rows = 0;  // strip rows of the launch
+    for (int k = 0; k < B.n; ++k)
+      if (K[k] > m && streamed(k, m, nu)) {
+        const int* n = B.ops[k]->h->mg[m].n;
+        rows += (long long)leg_strips(n[0], mode == LEG_DOWN ? leg_hx<LEG_DOWN>() : leg_hx<LEG_UP>()) * n[1];
+      }
+    int blocks = 0;
+    for (int k = 0; k < B.n; ++k) {
+      if (K[k] <= m || !streamed(k, m, nu)) continue;
+      amr_operator* op = B.ops[k];
+      amr_hierarchy* h = op->h;
+      Scratch<float>& S = op->s32;
+      const LevelView lv = mg_view(h, m, op->bc), cv = mg_view(h, m + 1, op->bc);
+      const PatchDesc &gp = h->mg[m].patch, &gcp = h->mg[m + 1].patch;
+      const int ns = leg_strips(gp.n[0], mode == LEG_DOWN ? leg_hx<LEG_DOWN>() : leg_hx<LEG_UP>());
+      const long long share = std::max<long long>(1, leg_share() * ns * gp.n[1] / std::max<long long>(1, rows));
+      Leg2D d = make_leg(mode, lv, &cv, gp, gcp, op->alpha, op->beta, p.omega, share);
+      d.p = k;
+      d.b = (m == 0 ? S.rin : S.mb[m]) + gp.off;
+      if (mode == LEG_DOWN) {
+        d.xo = (m == 0 ? S.T1 : S.mt[m]) + gp.off;
+        d.bcn = S.mb[m + 1] + gcp.off;
+      } else {
+        d.xi = (m == 0 ? S.T1 : S.mt[m]) + gp.off;
+        d.xc = S.mx[m + 1] + gcp.off;
+        d.xo = (m == 0 ? S.E : S.mx[m]) + gp.off;
+      }
+      blocks = std::max(blocks, (d.ns * d.nch + LEG_WARPS - 1) / LEG_WARPS);
+      leg.push_back(d);
+    }
+    group_of(mode == LEG_DOWN ? B.down : B.up, off, (int)leg.size() - off, blocks, 1, 0);
+  };
   // down legs m = 0 .. kmax-1 and up legs m = kmax-1 .. 0, each split by tile edge
-  for (int m = 0; m < B.kmax; ++m)
+  for (int m = 0; m < B.kmax; ++m) {
+    leg_group(m, LEG_DOWN);
     for (int tt : {16, 32}) {
       const int off = (int)down.size();
       int tx = 0, ty = 0;
       for (int k = 0; k < B.n; ++k) {
-        if (K[k] <= m) continue;
+        if (K[k] <= m || streamed(k, m, p.nu1)) continue;
         amr_operator* op = B.ops[k];
         amr_hierarchy* h = op->h;
         if (batch_tile(h->mg[m].n) != tt) continue;
@@ -3147,12 +3282,14 @@ amr_status build_batch_lists(BatchPlan& B) {
       }
       group_of(B.down, off, (int)down.size() - off, tx, ty, tt);
     }
-  for (int m = B.kmax - 1; m >= 0; --m)
+  }
+  for (int m = B.kmax - 1; m >= 0; --m) {
+    leg_group(m, LEG_UP);
     for (int tt : {16, 32}) {
       const int off = (int)up.size();
       int tx = 0, ty = 0;
       for (int k = 0; k < B.n; ++k) {
-        if (K[k] <= m) continue;
+        if (K[k] <= m || streamed(k, m, p.nu2)) continue;
         amr_operator* op = B.ops[k];
         amr_hierarchy* h = op->h;
         if (batch_tile(h->mg[m].n) != tt) continue;
@@ -3182,6 +3319,7 @@ amr_status build_batch_lists(BatchPlan& B) {
       }
       group_of(B.up, off, (int)up.size() - off, tx, ty, tt);
     }
+  }
   int rtx = 0, rty = 0;
   long long nmax = 0;
   for (int k = 0; k < B.n; ++k) {
@@ -3250,6 +3388,12 @@ amr_status batch_body(BatchPlan& B, cudaGraphConditionalHandle handle, cudaStrea
   constexpr int RD16 = 16 + 4 * BLK_FX_NU + 4, RD32 = 32 + 4 * BLK_FX_NU + 4;
   constexpr int RU16 = 16 + 4 * BLK_FX_NU, RU32 = 32 + 4 * BLK_FX_NU;
   for (const BatchGroup& g : B.down) {
+    if (g.tt == 0) {
+      launch(k_leg2d_b<LEG_DOWN>, dim3(g.tx, g.cnt, 1), 32 * LEG_WARPS, 0, st, (const Leg2D*)(B.d_leg + g.off),
+             (const int*)B.d_active);
+      TRY(launch_check());
+      continue;
+    }
     const int rm = g.tt == 16 ? RD16 : RD32;
     const size_t smem = (size_t)3 * (rm + 2 * NG) * (rm + 2 * NG) * sizeof(float);
     dim3 grid(g.tx, g.ty, g.cnt);
@@ -3261,6 +3405,12 @@ amr_status batch_body(BatchPlan& B, cudaGraphConditionalHandle handle, cudaStrea
          (const BCoarse*)B.d_coarse, (const int*)B.d_active);
   TRY(launch_check());
   for (const BatchGroup& g : B.up) {
+    if (g.tt == 0) {
+      launch(k_leg2d_b<LEG_UP>, dim3(g.tx, g.cnt, 1), 32 * LEG_WARPS, 0, st, (const Leg2D*)(B.d_leg + g.off),
+             (const int*)B.d_active);
+      TRY(launch_check());
+      continue;
+    }
     const int rm = g.tt == 16 ? RU16 : RU32;
     const size_t smem = (size_t)3 * (rm + 2 * NG) * (rm + 2 * NG) * sizeof(float);
     dim3 grid(g.tx, g.ty, g.cnt);
