@@ -169,6 +169,8 @@ inline bool sw_eligible(const LevelView& lv) {
   return px * (lv.maxn[1] + 2 * NG) * (lv.maxn[2] + 2 * NG) < (1LL << 31);
 }
 constexpr int TILE_BULK = 8;  // tile-table code of the bulk-copy 3-D kernel
+constexpr int TILE_COL = 16;  // and of the one-thread-per-column kernel (k_level_op3d_col): FP32 sweeps of 64^3 take
+                              // 5.0 us against 6.0 z-chunked and 11.1 bulk-copy, of 128^3 12.2 / 10.6 / 8.6
 
 void free_stack(amr_operator* op);  // stacked component batches (defined with amr_batch_solve)
 
@@ -425,9 +427,12 @@ void launch_zc(const LevelView& lv, const T* x, const T* f, T* out, T A, T B, T 
          vmask, gate);
 }
 
+// tile rows per consumer warp: four where the z neighbours are kept in registers
+template <typename T, int M>
+constexpr int sw_rw() { return sw3_zqueue<T, M>() ? 4 : SW_RW; }
 template <typename T, int M>
 constexpr auto sw_kernel() {
-  return k_sweep3d<T, M, SW_TY, SW_RW, SW_S>;
+  return k_sweep3d<T, M, SW_TY, sw_rw<T, M>(), SW_S>;
 }
 template <typename T>
 amr_status sw_attrs() {
@@ -503,7 +508,7 @@ amr_status launch_sw(const LevelView& lv, const T* x, const T* f, T* out, T A, T
                      long long ccs = 0) {
   TRY(sw_attrs<T>());
   constexpr size_t smem = sw3::smem_bytes<T, M, SW_TY, SW_S>();
-  constexpr int threads = 32 * (SW_TY / SW_RW + 2);
+  constexpr int threads = 32 * (SW_TY / sw_rw<T, M>() + 2);
   CUtensorMap tmx{}, tmf{};
   const int nc = std::max(1, lv.ncomp);  // stacked component batches: one part of the grid per replica
   if (M != OP_JACOBI0) TRY(encode_patch_tmap<T>(&tmx, x, lv.p0, SW_TY + 4, nc, lv.cstride));
@@ -692,9 +697,10 @@ amr_status level_op(int mode, const LevelView& lv, const T* x, const T* f, T* ou
              nb * sizeof(T) * lv.ncells, lv.ncells);
     return AMR_OK;
   }
-  if (D == 3 && !TR && bc == nullptr && (vmask == nullptr || mode == OP_RESID) && zc_eligible(lv, 2)) {
+  const int tile3 = D == 3 && !TR ? tile_rows_for(lv, sizeof(T)) : 0;
+  if (D == 3 && !TR && bc == nullptr && (vmask == nullptr || mode == OP_RESID) && zc_eligible(lv, 2) && tile3 != TILE_COL) {
     // z-chunked marching path; rows per thread from the autotuner's table
-    const int R = (tile_rows_for(lv, sizeof(T)) == 4 && zc_eligible(lv, 4)) ? 4 : 2;
+    const int R = (tile3 == 4 && zc_eligible(lv, 4)) ? 4 : 2;
     const T A = T(alpha), B = T(beta), O = T(omega);
 #define LAUNCH_ZC(M)                                                                                    \
   do {                                                                                                  \
@@ -1049,6 +1055,7 @@ amr_status autotune_tiles(amr_operator* op, cudaStream_t st) {
     const LevelView& lv = c.lv;
     std::vector<int> variants = D == 3 ? std::vector<int>{2} : std::vector<int>{1, 2, 4};
     if (D == 3 && zc_eligible(lv, 4)) variants.push_back(4);
+    if (D == 3 && zc_eligible(lv, 2) && lv.ncells <= 4194304.0) variants.push_back(TILE_COL);
     if (D == 3 && sw_eligible(lv)) variants.push_back(TILE_BULK);
     if (variants.size() < 2) continue;  // nothing to choose
     const long long key = tile_key(lv, sizeof(T));
@@ -1078,7 +1085,7 @@ amr_status autotune_tiles(amr_operator* op, cudaStream_t st) {
         std::lock_guard<std::mutex> lock(g_tile_mu);
         g_tile_table.pop_back();
       }
-      // a larger tile (or the bulk-copy kernel) must win by 5 %: timing back-to-back sweeps
+        // a larger tile (or the bulk-copy kernel) must win by 5 %: timing back-to-back sweeps
       // flatters it (warmer L2)
       if (ms < 0.95f * best) { best = ms; best_rows = rows; }
     }
@@ -1788,7 +1795,7 @@ amr_status mg_level0(amr_operator* op, const amr_solver_params& p, int m, const 
   }
   TRY(smooth_from_zero<T, D, TR>(h, 0, lv, b, x, t, p.nu1, op->alpha, op->beta, p.omega, false, st));
   const int xm[3] = {h->mg[m + 1].n[0], h->mg[m + 1].n[1], h->mg[m + 1].n[2]};
-  if (D == 3 && !TR && sw_eligible(lv) && lv.maxn[2] % 2 == 0 && tile_rows_for(lv, sizeof(T)) == TILE_BULK) {
+  if (D == 3 && !TR && sw_eligible(lv) && lv.maxn[2] % 2 == 0) {
     // the residual restriction by the bulk-copy kernel (same arithmetic as k_restrict)
     cudaEvent_t ev;
     prof_begin(st, &ev);
@@ -2136,8 +2143,7 @@ amr_status vcycle_corr(amr_operator* op, const amr_solver_params& p, const T* r,
     if (deferred && l == 1) {
       // the mean of the fine residual R_1 - A_1 E_1 (zero CF ghosts) on the covered cells; the
       // level-0 residual below writes the valid cells only
-      if (D == 3 && lv[0].npatch == lv[0].ncomp && sw_eligible(lv[1]) && lv[1].maxn[2] % 2 == 0 &&
-          tile_rows_for(lv[1], sizeof(T)) == TILE_BULK) {
+      if (D == 3 && lv[0].npatch == lv[0].ncomp && sw_eligible(lv[1]) && lv[1].maxn[2] % 2 == 0) {
         TRY(bulk_restrict_level<T>(lv[1], lv[0], E, S.R, rc, a_, b_, st));
       } else {
         TRY(restrict_blocks<T, D>(lv[1], lv[0], cl.xfer, cl.nxfer, cl.xfer_max, true, E, S.R, rc, a_, b_, st));
@@ -2155,8 +2161,7 @@ amr_status vcycle_corr(amr_operator* op, const amr_solver_params& p, const T* r,
       // every cell of level l-1, then its invalid cells overwritten by the mean of the fine
       // residual R_l - A_l E_l (zero CF ghosts, hence before E_L = X_L gets its own)
       TRY(level_op<T, D>(OP_RESID, lv[l - 1], S.X, r, S.R, nullptr, a_, b_, 0.0, nullptr, st));
-      if (D == 3 && lv[l - 1].npatch == lv[l - 1].ncomp && sw_eligible(lv[l]) && lv[l].maxn[2] % 2 == 0 &&
-          tile_rows_for(lv[l], sizeof(T)) == TILE_BULK) {
+      if (D == 3 && lv[l - 1].npatch == lv[l - 1].ncomp && sw_eligible(lv[l]) && lv[l].maxn[2] % 2 == 0) {
         TRY(bulk_restrict_level<T>(lv[l], lv[l - 1], E, S.R, S.R, a_, b_, st));
       } else {
         TRY(restrict_blocks<T, D>(lv[l], lv[l - 1], cl.xfer, cl.nxfer, cl.xfer_max, true, E, S.R, S.R, a_, b_, st));
