@@ -1271,9 +1271,11 @@ inline Leg2D make_leg(int mode, const LevelView& lv, const LevelView* cv, const 
   d.nd1 = lv.ndom[1];
   const int hx = mode == LEG_DOWN ? leg_hx<LEG_DOWN>() : leg_hx<LEG_UP>();
   d.ns = leg_strips(gp.n[0], hx);
-  // rows per chunk: as many chunks as the share allows, at least 32 rows each (18 are halo)
+  // rows per chunk: as many chunks as the share allows, at least 16 rows each (18 are halo): a row
+  // takes about as long with one warp per scheduler as with three, so a short chunk pays even though
+  // half of it is halo (4096^2 solve with a least chunk of 8, 16, 32 rows: 15.2, 14.3, 15.3 ms)
   const long long nch = std::max<long long>(1, share / d.ns);
-  d.ch = (int)std::max<long long>(32, (gp.n[1] + nch - 1) / nch + 1 & ~1ll);
+  d.ch = (int)std::max<long long>(16, (gp.n[1] + nch - 1) / nch + 1 & ~1ll);
   d.nch = (gp.n[1] + d.ch - 1) / d.ch;
   d.kc2 = (float)beta * lv.inv12h2_f;
   d.kc1 = 16.0f * d.kc2;
@@ -1293,7 +1295,8 @@ inline Leg2D make_leg(int mode, const LevelView& lv, const LevelView* cv, const 
 inline long long leg_share() { return 12ll * sm_count(); }  // resident warps: three blocks of four per SM
 template <int MODE>
 amr_status launch_leg(const Leg2D& d, cudaStream_t st) {
-  launch(k_leg2d<MODE>, (unsigned)((d.ns * d.nch + LEG_WARPS - 1) / LEG_WARPS), 32 * LEG_WARPS, 0, st, d);
+  launch(k_leg2d<MODE>, (unsigned)((d.ns * d.nch + LEG_WARPS - 1) / LEG_WARPS), 32 * LEG_WARPS, leg_smem_bytes<MODE>(), st,
+         d);
   return launch_check();
 }
 
@@ -1308,6 +1311,11 @@ amr_status blk_attrs() {
   CK(cudaFuncSetAttribute(k_mg_coarse2d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
   CK(cudaFuncSetAttribute(k_mg_coarse2d_sq<T, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
   CK(cudaFuncSetAttribute(k_mg_coarse2d_sq<T, 48>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  CK(cudaFuncSetAttribute(k_leg2d<LEG_DOWN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)leg_smem_bytes<LEG_DOWN>()));
+  CK(cudaFuncSetAttribute(k_leg2d<LEG_UP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)leg_smem_bytes<LEG_UP>()));
+  CK(cudaFuncSetAttribute(k_leg2d<LEG_POST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)leg_smem_bytes<LEG_POST>()));
+  CK(cudaFuncSetAttribute(k_leg2d_b<LEG_DOWN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)leg_smem_bytes<LEG_DOWN>()));
+  CK(cudaFuncSetAttribute(k_leg2d_b<LEG_UP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)leg_smem_bytes<LEG_UP>()));
   done = true;
   return AMR_OK;
 }
@@ -3429,8 +3437,8 @@ amr_status batch_body(BatchPlan& B, cudaGraphConditionalHandle handle, cudaStrea
   constexpr int RU16 = 16 + 4 * BLK_FX_NU, RU32 = 32 + 4 * BLK_FX_NU;
   for (const BatchGroup& g : B.down) {
     if (g.tt == 0) {
-      launch(k_leg2d_b<LEG_DOWN>, dim3(g.tx, g.cnt, 1), 32 * LEG_WARPS, 0, st, (const Leg2D*)(B.d_leg + g.off),
-             (const int*)B.d_active);
+      launch(k_leg2d_b<LEG_DOWN>, dim3(g.tx, g.cnt, 1), 32 * LEG_WARPS, leg_smem_bytes<LEG_DOWN>(), st,
+             (const Leg2D*)(B.d_leg + g.off), (const int*)B.d_active);
       TRY(launch_check());
       continue;
     }
@@ -3446,8 +3454,8 @@ amr_status batch_body(BatchPlan& B, cudaGraphConditionalHandle handle, cudaStrea
   TRY(launch_check());
   for (const BatchGroup& g : B.up) {
     if (g.tt == 0) {
-      launch(k_leg2d_b<LEG_UP>, dim3(g.tx, g.cnt, 1), 32 * LEG_WARPS, 0, st, (const Leg2D*)(B.d_leg + g.off),
-             (const int*)B.d_active);
+      launch(k_leg2d_b<LEG_UP>, dim3(g.tx, g.cnt, 1), 32 * LEG_WARPS, leg_smem_bytes<LEG_UP>(), st,
+             (const Leg2D*)(B.d_leg + g.off), (const int*)B.d_active);
       TRY(launch_check());
       continue;
     }

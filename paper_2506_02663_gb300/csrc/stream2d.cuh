@@ -26,7 +26,9 @@ enum { LEG_DOWN = 0, LEG_UP = 1, LEG_POST = 2 };
 constexpr int LEG_NU = 4;        // sweeps per pass
 constexpr int LEG_W = 128;       // columns of a strip (four per lane)
 constexpr int LEG_WARPS = 4;     // warps per block
-constexpr int LEG_RING = 16;     // rows of f kept per warp (10 needed)
+constexpr int LEG_RING = 16;     // rows of f kept per warp (ten in use, LEG_AHEAD on their way)
+constexpr int LEG_AHEAD = 4;     // rows requested ahead of their step
+constexpr int LEG_CRING = 8;     // up: coarse rows kept per warp
 
 struct Leg2D {
   PatchDesc gp, gcp;             // the level's patch and the coarser one's
@@ -75,6 +77,19 @@ __device__ __forceinline__ float4 ldrow(const float* __restrict__ g) {  // four 
   const float2 a = *reinterpret_cast<const float2*>(g), b = *reinterpret_cast<const float2*>(g + 2);
   return make_float4(a.x, a.y, b.x, b.y);
 }
+// asynchronous copy of four cells (8-byte aligned) into the lane's own slot; zeros where !on
+__device__ __forceinline__ void cprow(float4* s, const float* g, bool on) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(s);
+  const int n = on ? 8 : 0;
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(g), "r"(n) : "memory");
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d + 8), "l"(g + (on ? 2 : 0)), "r"(n) : "memory");
+}
+template <typename V>
+__device__ __forceinline__ void cpone(V* s, const float* g, bool on) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(s);
+  const int n = on ? (int)sizeof(V) : 0;
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(d), "l"(g), "n"(sizeof(V)), "r"(n) : "memory");
+}
 __device__ __forceinline__ void strow(float* g, float4 v) {
   *reinterpret_cast<float2*>(g) = make_float2(v.x, v.y);
   *reinterpret_cast<float2*>(g + 2) = make_float2(v.z, v.w);
@@ -85,8 +100,16 @@ template <int MODE>
 struct LegRun {
   static constexpr int HX = leg_hx<MODE>(), HY = leg_hy<MODE>(), LAG = leg_lag<MODE>();
   static constexpr int NWIN = MODE == LEG_POST ? 3 : 4;
+  // shared memory of a warp, every entry private to one lane (no barriers)
+  struct Smem {
+    float4 f[LEG_RING][32];                                  // right-hand side rows
+    float4 x[MODE == LEG_UP || MODE == LEG_POST ? 5 : 1][32];  // up: iterate rows; post: rows of xo
+    float4 y[MODE == LEG_UP ? 1 : 5][32];                    // rows of the second target
+    float2 c[MODE == LEG_UP ? LEG_CRING : 1][32];            // up: coarse rows
+    float e[MODE == LEG_UP ? LEG_CRING : 1][2];              // up: the coarse cells beyond the strip
+  };
   const Leg2D& L;
-  float4* ring;  // this lane's column of the f ring (stride 32)
+  Smem& S;
   int lane, c0, n0, n1;
   bool act, xl, xh, xface;  // lane holds cells; lane at the low / high x edge; strip touches one
   float kc0, kc1, kc2;
@@ -94,7 +117,7 @@ struct LegRun {
   int sy, fo;               // row pitch; offset of (c0, row 0) inside the patch
   float4 W[4][5];
   float4 hg, rp;            // ghost row held for the next step; residual of the even row
-  int y0, y1;               // rows this warp stores
+  int y0, y1, tend;         // rows this warp stores; steps end
   bool cols;                // the lane's columns are stored
 
   // residual of the row c between rows m1, m2 (below) and p1, p2 (above)
@@ -121,7 +144,7 @@ struct LegRun {
   __device__ __forceinline__ float4 fma4(float4 w, float4 r, float4 c) const {
     return make_float4(fmaf(w.x, r.x, c.x), fmaf(w.y, r.y, c.y), fmaf(w.z, r.z, c.z), fmaf(w.w, r.w, c.w));
   }
-  __device__ __forceinline__ float4 fring(int k) const { return ring[(k & (LEG_RING - 1)) * 32]; }
+  __device__ __forceinline__ float4 fring(int k) const { return S.f[k & (LEG_RING - 1)][lane]; }
   // factors of row k
   __device__ __forceinline__ float4 factors(int k) const {
     const int cy = face_class(L.gp.lo[1] + k, L.nd1);
@@ -130,18 +153,18 @@ struct LegRun {
     return make_float4(L.wt[face_class(g, L.nd0) + 5 * cy], L.wt[face_class(g + 1, L.nd0) + 5 * cy],
                        L.wt[face_class(g + 2, L.nd0) + 5 * cy], L.wt[face_class(g + 3, L.nd0) + 5 * cy]);
   }
-  // a finished iterate row
-  __device__ __forceinline__ void store(int k, float4 v) const {
+  // a finished iterate row; sl: the slot its targets' old values wait in (-1: read them here)
+  __device__ __forceinline__ void store(int k, float4 v, int sl) const {
     if (!cols || k < y0 || k >= y1) return;
     const int o = fo + k * sy;
     if (MODE == LEG_POST) {
-      const float4 e = leg2::ldrow(L.xo + o);
+      const float4 e = sl < 0 ? leg2::ldrow(L.xo + o) : S.x[MODE == LEG_POST && sl > 0 ? sl : 0][lane];
       leg2::strow(L.xo + o, make_float4(e.x + v.x, e.y + v.y, e.z + v.z, e.w + v.w));
     } else {
       leg2::strow(L.xo + o, v);
     }
     if (MODE != LEG_UP && L.x2 != nullptr) {
-      const float4 e = leg2::ldrow(L.x2 + o);
+      const float4 e = sl < 0 ? leg2::ldrow(L.x2 + o) : S.y[MODE != LEG_UP && sl > 0 ? sl : 0][lane];
       leg2::strow(L.x2 + o, make_float4(e.x + v.x, e.y + v.y, e.z + v.z, e.w + v.w));
     }
   }
@@ -234,39 +257,53 @@ struct LegRun {
     return L.xc[(k + NG) * (int)L.gcp.sy + c + NG];
   }
 
-  struct Row {  // the global reads of one step, one step ahead
-    float4 f, x;
-    float2 ca, cb;
-    float ea, eb;
-  };
-  __device__ __forceinline__ Row read(int t) const {
-    Row r;
-    r.f = r.x = make_float4(0.f, 0.f, 0.f, 0.f);
-    r.ca = r.cb = make_float2(0.f, 0.f);
-    r.ea = r.eb = 0.f;
-    if (t < n1) {
-      if (act) {
-        r.f = leg2::ldrow(L.b + fo + t * sy);
-        if (MODE == LEG_UP) r.x = leg2::ldrow(L.xi + fo + t * sy);
-      }
+  // Requests what step t needs, into slot PH of the five-row rings: row t of f (up: of xi, and
+  // the coarse row that step t is the first to use), the old values of the row it finishes.
+  template <int PH>
+  __device__ __forceinline__ void request(int t) {
+    if (t < n1 && t < tend) {
+      const bool on = act;
+      leg2::cprow(&S.f[t & (LEG_RING - 1)][lane], on ? L.b + fo + t * sy : L.b, on);
       if (MODE == LEG_UP) {
-        const int p = t >> 1, q = min(max(p + ((t & 1) ? 1 : -1), 0), L.gcp.n[1] - 1);
-        r.ca = crow(p);
-        r.cb = crow(q);
-        r.ea = cedge(p);
-        r.eb = cedge(q);
+        leg2::cprow(&S.x[MODE == LEG_UP ? PH : 0][lane], on ? L.xi + fo + t * sy : L.xi, on);
+        if (t & 1) request_coarse((t >> 1) + 1);
       }
     }
-    return r;
+    const int k = t - 6;
+    if (MODE != LEG_UP && cols && k >= y0 && k < y1) {
+      if (MODE == LEG_POST) leg2::cprow(&S.x[MODE == LEG_POST ? PH : 0][lane], L.xo + fo + k * sy, true);
+      if (L.x2 != nullptr) leg2::cprow(&S.y[MODE == LEG_UP ? 0 : PH][lane], L.x2 + fo + k * sy, true);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  __device__ __forceinline__ void request_coarse(int q) {
+    if (q < 0 || q >= L.gcp.n[1]) return;
+    const int sl = MODE == LEG_UP ? q & (LEG_CRING - 1) : 0;
+    const float* r = L.xc + (q + NG) * (int)L.gcp.sy + NG;
+    leg2::cpone(&S.c[sl][lane], act ? r + (c0 >> 1) : r, act);
+    if (lane == 0) leg2::cpone(&S.e[sl][0], r + max((c0 >> 1) - 1, 0), true);
+    if (lane == 31) leg2::cpone(&S.e[sl][1], act ? r + min((c0 >> 1) + 2, L.gcp.n[0] - 1) : r, act);
   }
 
   // One step: push row t, then every stage.  PH: physical slot of the windows' newest row.
   // FACE: some row of this step lies at a y edge of the patch.
   template <int PH, bool FACE>
-  __device__ __forceinline__ void step(int t, const Row& in) {
+  __device__ __forceinline__ void step(int t) {
+    request<(PH + LEG_AHEAD) % 5>(t + LEG_AHEAD);
+    asm volatile("cp.async.wait_group %0;" ::"n"(LEG_AHEAD) : "memory");
     if (!FACE || t < n1) {
-      ring[(t & (LEG_RING - 1)) * 32] = in.f;
-      W[0][PH] = first(t, in.f, in.x, in.ca, in.cb, in.ea, in.eb, FACE);
+      const float4 f = fring(t);
+      if (MODE == LEG_UP) {
+        const int p = t >> 1, q = min(max(p + ((t & 1) ? 1 : -1), 0), L.gcp.n[1] - 1), m = LEG_CRING - 1;
+        const bool end = lane == 0 || lane == 31;
+        const int e = lane >> 4;
+        const int sp = MODE == LEG_UP ? p & m : 0, sq = MODE == LEG_UP ? q & m : 0;
+        W[0][PH] = first(t, f, S.x[MODE == LEG_UP ? PH : 0][lane], S.c[sp][lane], S.c[sq][lane], end ? S.e[sp][e] : 0.f,
+                         end ? S.e[sq][e] : 0.f, FACE);
+      } else {
+        const float2 z = make_float2(0.f, 0.f);
+        W[0][PH] = first(t, f, f, z, z, 0.f, 0.f, FACE);
+      }
     } else {
       push_ghost<PH>(W[0], t);
     }
@@ -302,26 +339,26 @@ struct LegRun {
       const float4 g2 = leg2::lin4(L.g[2][1], V[C], V[B], V[A], V[N]);
       V[D] = g1;
       const float4 r = resid(g2, g1, V[C], V[B], V[A], fring(0));
-      emit<PH, true>(s, last, 0, r, V[C], A);
+      emit<PH, true>(s, last, 0, r, V[C], A, -1);  // its slot is taken again by now
     }
     const float4 r = resid(V[D], V[C], V[B], V[A], V[N], fring(k));
-    emit<PH, FACE>(s, last, k, r, V[B], N);
+    emit<PH, FACE>(s, last, k, r, V[B], N, PH);
   }
   // the residual r of centre row k of stage s (iterate c): restricted, or swept into the next window's slot
   template <int PH, bool FACE>
-  __device__ __forceinline__ void emit(int s, bool last, int k, float4 r, float4 c, int slot) {
+  __device__ __forceinline__ void emit(int s, bool last, int k, float4 r, float4 c, int slot, int sl) {
     if (MODE == LEG_DOWN && last) {
       restrict_row(k, r);
       return;
     }
     const float4 v = fma4(FACE ? factors(k) : wI, r, c);
     if (last) {
-      store(k, v);
+      store(k, v, sl);
       return;
     }
     // slot is a constant after inlining
     if (s + 1 < 4) W[s + 1 < 4 ? s + 1 : 3][slot] = v;
-    if (MODE == LEG_DOWN && s == 2) store(k, v);  // x after four sweeps
+    if (MODE == LEG_DOWN && s == 2) store(k, v, sl);  // x after four sweeps
   }
 
   __device__ __forceinline__ void run(int strip, int chunk) {
@@ -331,6 +368,7 @@ struct LegRun {
     const int xs = strip == 0 ? 0 : min(u0 - HX, n0 - LEG_W);
     y0 = chunk * L.ch;
     y1 = min(n1, y0 + L.ch);
+    tend = y1 + LAG;
     c0 = xs + 4 * lane;
     act = c0 < n0;
     cols = act && c0 >= u0 && c0 < u1;
@@ -352,51 +390,60 @@ struct LegRun {
 #pragma unroll
       for (int q = 0; q < 5; ++q) W[s][q] = make_float4(0.f, 0.f, 0.f, 0.f);
     hg = rp = make_float4(0.f, 0.f, 0.f, 0.f);
-    const int r0 = max(0, y0 - HY), tend = y1 + LAG;  // steps r0 .. tend - 1
-    Row in = read(r0);
+    const int r0 = max(0, y0 - HY);  // steps r0 .. tend - 1
+    if (MODE == LEG_UP) {
+      const int p = r0 >> 1;
+      request_coarse(p - 1);
+      request_coarse(p);
+    }
+    static_assert(LEG_AHEAD == 4, "four rows are requested before the first step");
+    request<0>(r0);
+    request<1>(r0 + 1);
+    request<2>(r0 + 2);
+    request<3>(r0 + 3);
     // groups of five steps (the windows' slots are then constants); the last group may run past
     // tend: its extra rows are not stored
     for (int t = r0; t < tend; t += 5) {
       // rows t + 4 - LAG .. t + 4: none within two rows of a y edge that this region contains
       const bool face = (r0 == 0 && t - LAG <= 1) || t + 5 > n1 - 3;
       if (!face) {
-        group<false>(t, in);
+        group<false>(t);
       } else {
-        group<true>(t, in);
+        group<true>(t);
       }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
   }
   template <bool FACE>
-  __device__ __forceinline__ void group(int t, Row& in) {
-    Row nx = read(t + 1);
-    step<0, FACE>(t, in);
-    in = read(t + 2);
-    step<1, FACE>(t + 1, nx);
-    nx = read(t + 3);
-    step<2, FACE>(t + 2, in);
-    in = read(t + 4);
-    step<3, FACE>(t + 3, nx);
-    nx = read(t + 5);
-    step<4, FACE>(t + 4, in);
-    in = nx;
+  __device__ __forceinline__ void group(int t) {
+    step<0, FACE>(t);
+    step<1, FACE>(t + 1);
+    step<2, FACE>(t + 2);
+    step<3, FACE>(t + 3);
+    step<4, FACE>(t + 4);
   }
 };
 
 template <int MODE>
+constexpr size_t leg_smem_bytes() { return LEG_WARPS * sizeof(typename LegRun<MODE>::Smem); }
+
+template <int MODE>
 __global__ void __launch_bounds__(32 * LEG_WARPS, 3) k_leg2d(const __grid_constant__ Leg2D d) {
-  __shared__ float4 ring[LEG_WARPS][LEG_RING][32];
+  extern __shared__ float4 leg_smem[];
+  auto* ring = reinterpret_cast<typename LegRun<MODE>::Smem*>(leg_smem);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int w = blockIdx.x * LEG_WARPS + warp;
   pdl_wait();
   if (w >= d.ns * d.nch) return;
-  LegRun<MODE> r{d, &ring[warp][0][lane], lane};
+  LegRun<MODE> r{d, ring[warp], lane};
   r.run(w % d.ns, w / d.ns);
 }
 
 // batches: entry blockIdx.y of a descriptor list, skipped once its problem has converged
 template <int MODE>
 __global__ void __launch_bounds__(32 * LEG_WARPS, 3) k_leg2d_b(const Leg2D* __restrict__ list, const int* __restrict__ active) {
-  __shared__ float4 ring[LEG_WARPS][LEG_RING][32];
+  extern __shared__ float4 leg_smem[];
+  auto* ring = reinterpret_cast<typename LegRun<MODE>::Smem*>(leg_smem);
   __shared__ Leg2D d;
   pdl_wait();
   const Leg2D* e = list + blockIdx.y;
@@ -407,7 +454,7 @@ __global__ void __launch_bounds__(32 * LEG_WARPS, 3) k_leg2d_b(const Leg2D* __re
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int w = blockIdx.x * LEG_WARPS + warp;
   if (w >= d.ns * d.nch) return;
-  LegRun<MODE> r{d, &ring[warp][0][lane], lane};
+  LegRun<MODE> r{d, ring[warp], lane};
   r.run(w % d.ns, w / d.ns);
 }
 
