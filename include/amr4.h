@@ -153,13 +153,14 @@ typedef struct {
   int zero_initial;  /* 1: start from phi = 0; 0: use phi as the initial guess            */
   int use_graph;     /* 1: capture the whole solve as one CUDA graph (device-side loop over
                         V-cycles, no host round trip per V-cycle) and replay it              */
-  int fuse_coarse;   /* coarse end of the level-0 V-cycle.  0 (default): per-grid launches (in
-                        2-D the one-block square coarse kernel where it applies).  1: one
-                        shared-memory block from the largest grid that fits (generic per-cell
+  int fuse_coarse;   /* coarse end of the level-0 V-cycle.  0 (default): in one launch where it
+                        pays (2-D FP32 forward V-cycles: one block; otherwise the distributed
+                        shared memory of one thread-block cluster), per-grid launches else.  1:
+                        one shared-memory block from the largest grid that fits (generic per-cell
                         code).  2 (3-D): the grids of at most 32^3 cells as one launch of one
-                        thread-block cluster, phases separated by cluster barriers, same
-                        per-cell arithmetic as the per-grid kernels.  On GB300 both fused
-                        forms are slower than captured per-grid launches.                   */
+                        thread-block cluster working in global memory, phases separated by
+                        cluster barriers, same per-cell arithmetic as the per-grid kernels.
+                        On GB300 forms 1 and 2 are slower than the default.                 */
   int temporal_blocking; /* 1 (default): in forward FP32 V-cycles on 2-D level-0 multigrid grids,
                         each down leg (nu1 sweeps, residual, restriction) and each up leg
                         (prolongation, nu2 sweeps) is one launch over shared-memory tiles
@@ -537,7 +538,8 @@ amr_status amr_set_tile_rows(int rows);
  * the largest interior |phi| rounded down to a power of two (at most half a unit in the last
  * place of that value, the size of one FP64 rounding of it); the sum 16 s1 - s2 - 90 phi of
  * Eq. (discreteOps) is then exact in int64, and r = f - alpha phi - beta/(12 h^2) * sum is
- * formed in FP64.  Physical ghost values are fixed combinations of interior values and
+ * formed in FP64.  The same switch covers 2-D levels that are the whole domain, of at least
+ * 2^21 cells, with a unit three bits finer.  Physical ghost values are fixed combinations of interior values and
  * always fit; a stored ghost value (coarse-fine, copy) of 4 * 2^53 units or more, or a
  * non-finite value, makes the plain FP64 kernel recompute the level.  Not in the paper: on
  * this GPU FP64 arithmetic runs at a small fraction of the integer rate.  on = 0: the plain

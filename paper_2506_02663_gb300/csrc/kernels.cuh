@@ -837,7 +837,7 @@ __device__ __forceinline__ double fx_to_double(long long t) {
   return __longlong_as_double((long long)(sg | ((((unsigned long long)(1085 - lz)) << 52) + mant)));
 }
 
-// largest |x| over the interior cells of a single-patch level, as IEEE bits (non-negative
+// largest |x| over the interior cells of a single-patch level, as IEEE bits cut to the upper word (non-negative
 // doubles order like their bit patterns), into *acc; block size 256
 __global__ void __launch_bounds__(256) k_absmax_patch(LevelView lv, const double* __restrict__ x,
                                                       unsigned long long* __restrict__ acc) {
@@ -847,22 +847,19 @@ __global__ void __launch_bounds__(256) k_absmax_patch(LevelView lv, const double
   const PatchDesc p = lv.patches[blockIdx.y];
   acc += 2 * blockIdx.y;
   const int n0 = p.n[0], n1 = p.n[1], rows = p.n[1] * p.n[2];
-  unsigned long long v = 0ull;
+  // the frame is set by the exponent alone, so the upper words are compared
+  unsigned v = 0u;
   // one warp per row, eight loads of a lane in flight
   const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
   for (int r = blockIdx.x * wpb + (threadIdx.x >> 5); r < rows; r += gridDim.x * wpb) {
     const double* __restrict__ row = x + p.off + (long long)(r / n1 + NG) * p.sz + (long long)(r % n1 + NG) * p.sy + NG;
 #pragma unroll 8
     for (int i = lane; i < n0; i += 32) {
-      const unsigned long long b = (unsigned long long)__double_as_longlong(__ldg(row + i)) & 0x7fffffffffffffffull;
-      v = b > v ? b : v;
+      v = max(v, (unsigned)__double2hiint(__ldg(row + i)) & 0x7fffffffu);
     }
   }
-  for (int s = 16; s > 0; s >>= 1) {
-    const unsigned long long u = __shfl_xor_sync(0xffffffffu, v, s);
-    v = u > v ? u : v;
-  }
-  if ((threadIdx.x & 31) == 0 && v != 0ull) atomicMax(acc, v);
+  v = __reduce_max_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0 && v != 0u) atomicMax(acc, (unsigned long long)v << 32);
 }
 
 // The residual f - (alpha x + beta L x) of a z-chunked single-patch 3-D level (same tiles,
