@@ -3230,57 +3230,147 @@ __device__ __forceinline__ void dd_add(double& s, double& c, double a, double ac
   two_sum(t, e, s, c);
 }
 
-// Compensated, deterministic partial sums of w * x over the valid interior cells of one
-// level, with a fixed number of blocks per level (the rows each warp visits depend only on the
-// launch shape): one double-double partial part[2*(base+block)].  A warp sums whole rows; each
-// lane adds its cells with TwoSum and collects the errors (seven FP64 operations a cell, which
-// bound the pass: the renormalising double-double sum of w x took sixteen and 370 us for 17 M
-// cells), the lanes' and warps' sums combine in double-double, and w multiplies the block's sum
-// exactly (TwoProd).
+// A warp's sum of doubles in 128-bit fixed point: a double enters as its 53-bit significand
+// shifted to the warp's common frame (exponent E), so additions are exact integer ones in any
+// order.  Below the sign the frame keeps 26 bits of headroom (2^24 terms at least) and 47 bits
+// under the last bit of the largest term: terms within a factor 2^47 of it enter exactly.  An
+// addition costs about 30 integer instructions, where TwoSum costs seven FP64 ones at a fiftieth
+// of their rate.
+struct WarpSum {
+  unsigned l0 = 0, l1 = 0, l2 = 0, l3 = 0;
+  int E = 0;                // frame; 0: nothing added yet
+  double s = 0.0, c = 0.0;  // what earlier frames collected
+  bool bad = false;         // a non-finite term
+
+  __device__ __forceinline__ static int exponent(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+  // v, of an exponent <= E - 2
+  __device__ __forceinline__ void add(double v) {
+    const unsigned bh = (unsigned)__double2hiint(v), bl = (unsigned)__double2loint(v);
+    const int e = (int)((bh >> 20) & 0x7ffu);
+    const unsigned mh = (bh & 0xfffffu) | (e != 0 ? 0x100000u : 0u);
+    const unsigned sh = (unsigned)(E - max(e, 1) + 14), bs = sh & 31u, ws = sh >> 5;
+    const unsigned t2 = mh >> bs, t1 = __funnelshift_r(bl, mh, bs), t0 = __funnelshift_r(0u, bl, bs);
+    const unsigned m = (unsigned)((int)bh >> 31);  // negative: complement, plus one through the carry
+    const unsigned x3 = m ^ (ws == 0 ? t2 : 0u);
+    const unsigned x2 = m ^ (ws == 0 ? t1 : ws == 1 ? t2 : 0u);
+    const unsigned x1 = m ^ (ws == 0 ? t0 : ws == 1 ? t1 : ws == 2 ? t2 : 0u);
+    const unsigned x0 = m ^ (ws == 1 ? t0 : ws == 2 ? t1 : ws == 3 ? t2 : 0u);
+    asm("{\n\t.reg .u32 t;\n\t"
+        "add.cc.u32 t, %4, 1;\n\t"
+        "addc.cc.u32 %0, %0, %5;\n\t"
+        "addc.cc.u32 %1, %1, %6;\n\t"
+        "addc.cc.u32 %2, %2, %7;\n\t"
+        "addc.u32 %3, %3, %8;\n\t}"
+        : "+&r"(l0), "+&r"(l1), "+&r"(l2), "+&r"(l3)
+        : "r"(m), "r"(x0), "r"(x1), "r"(x2), "r"(x3));
+  }
+  __device__ __forceinline__ void join(unsigned a0, unsigned a1, unsigned a2, unsigned a3) {
+    asm("add.cc.u32 %0, %0, %4;\n\t"
+        "addc.cc.u32 %1, %1, %5;\n\t"
+        "addc.cc.u32 %2, %2, %6;\n\t"
+        "addc.u32 %3, %3, %7;"
+        : "+&r"(l0), "+&r"(l1), "+&r"(l2), "+&r"(l3)
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3));
+  }
+  // the lanes' integers summed into every lane
+  __device__ __forceinline__ void reduce() {
+#pragma unroll 1
+    for (int st = 16; st > 0; st >>= 1) {
+      const unsigned a0 = __shfl_xor_sync(0xffffffffu, l0, st), a1 = __shfl_xor_sync(0xffffffffu, l1, st);
+      const unsigned a2 = __shfl_xor_sync(0xffffffffu, l2, st), a3 = __shfl_xor_sync(0xffffffffu, l3, st);
+      join(a0, a1, a2, a3);
+    }
+  }
+  // the integers as a double-double added to (s, c); the frame is free again
+  __device__ __forceinline__ void collect() {
+    double h, e1, e2, e3;
+    two_sum(79228162514264337593543950336.0 * (double)(int)l3, 18446744073709551616.0 * (double)l2, h, e1);
+    two_sum(h, 4294967296.0 * (double)l1, h, e2);
+    two_sum(h, (double)l0, h, e3);
+    const double lo = e1 + (e2 + e3);
+    // l3's unit is 2^(E - 1075 + 32 + 14)
+    if (E != 0) dd_add(s, c, scalbn(h, E - 1125), scalbn(lo, E - 1125));
+    l0 = l1 = l2 = l3 = 0;
+    E = 0;
+  }
+  // the warp's frame for terms of exponents up to e (warp-uniform)
+  __device__ __forceinline__ void frame(int e) {
+    if (e + 2 <= E) return;
+    if (E != 0) {
+      reduce();
+      collect();
+    }
+    E = max(e, 1) + 2;
+  }
+};
+
+// Deterministic partial sums of w * x over the valid interior cells of one level, with a fixed
+// number of blocks per level (the rows each warp visits depend only on the launch shape): one
+// double-double partial part[2*(base+block)].  A warp sums whole rows in fixed point (WarpSum),
+// the warps' sums combine in double-double, and w multiplies the block's sum exactly (TwoProd).
 template <int D>
 __global__ void __launch_bounds__(256) k_wsum_gs(LevelView lv, const double* __restrict__ x,
                                                  const unsigned char* __restrict__ vmask, double w,
                                                  double* __restrict__ part, long long base) {
   pdl_wait();
-  __shared__ double ss[256], sc[256];
-  double s = 0.0, c = 0.0;
-  const int lane = threadIdx.x & 31;
+  constexpr int K = 8;  // cells of a lane in flight
+  __shared__ double ss[8], sc[8];
+  WarpSum a;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nw = gridDim.x * 8;
   for (int pi = 0; pi < lv.npatch; ++pi) {
     const PatchDesc p = lv.patches[pi];
     const int nr = p.n[1] * p.n[2];
-    for (int row = blockIdx.x * 8 + (threadIdx.x >> 5); row < nr; row += nw) {
+    for (int row = blockIdx.x * 8 + warp; row < nr; row += nw) {
       const long long o = poff(p, 0, row % p.n[1], row / p.n[1]);
-#pragma unroll 4
-      for (int i = lane; i < p.n[0]; i += 32) {
-        const double v = (vmask == nullptr || vmask[o + i]) ? x[o + i] : 0.0;
-        double t, e;
-        two_sum(s, v, t, e);
-        s = t;
-        c += e;
+      for (int i0 = 0; i0 < p.n[0]; i0 += 32 * K) {
+        double v[K];
+        unsigned char m[K];
+        int e = 0;
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+          const int i = i0 + 32 * q + lane;
+          v[q] = i < p.n[0] ? x[o + i] : 0.0;
+          m[q] = vmask == nullptr || (i < p.n[0] && vmask[o + i]);
+        }
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+          if (!m[q]) v[q] = 0.0;
+          e = max(e, WarpSum::exponent(v[q]));
+        }
+        e = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+        if (e == 0x7ff) {
+          a.bad = true;
+          continue;
+        }
+        a.frame(e);
+#pragma unroll
+        for (int q = 0; q < K; ++q)
+          if (i0 + 32 * q < p.n[0]) a.add(v[q]);
       }
     }
   }
-  {
+  a.reduce();
+  a.collect();
+  if (a.bad) a.s = __longlong_as_double(0x7ff8000000000000ll);
+  if (lane == 0) {
+    ss[warp] = a.s;
+    sc[warp] = a.c;
+  }
+  __syncthreads();
+  if (warp != 0) return;
+  double s = lane < 8 ? ss[lane & 7] : 0.0, c = lane < 8 ? sc[lane & 7] : 0.0;
+#pragma unroll 1
+  for (int st = 4; st > 0; st >>= 1) {
+    const double t = __shfl_down_sync(0xffffffffu, s, st), tc = __shfl_down_sync(0xffffffffu, c, st);
+    dd_add(s, c, t, tc);
+  }
+  if (lane == 0) {
     const double hi = w * s, lo = fma(w, s, -hi);
     const double e = fma(w, c, lo);
     two_sum(hi, e, s, c);
-  }
-  ss[threadIdx.x] = s;
-  sc[threadIdx.x] = c;
-  __syncthreads();
-  for (int st = 128; st > 0; st >>= 1) {
-    if ((int)threadIdx.x < st) {
-      double a = ss[threadIdx.x], ac = sc[threadIdx.x];
-      dd_add(a, ac, ss[threadIdx.x + st], sc[threadIdx.x + st]);
-      ss[threadIdx.x] = a;
-      sc[threadIdx.x] = ac;
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    part[2 * (base + blockIdx.x)] = ss[0];
-    part[2 * (base + blockIdx.x) + 1] = sc[0];
+    part[2 * (base + blockIdx.x)] = s;
+    part[2 * (base + blockIdx.x) + 1] = c;
   }
 }
 
@@ -3334,26 +3424,33 @@ __global__ void k_bsum(LevelView lv, const double* __restrict__ bc, const unsign
   }
 }
 
-// Final fixed-order reduction of n double-double partials (one block of 256 threads):
-// out[0] = (sum_a - sum_b_scaled ... ) handled by the caller; here out[slot] = sum.
-__global__ void k_dd_final(const double* __restrict__ part, long long n, double* __restrict__ out) {
+// Sum of n double-double partials (one block of 256 threads), in the same fixed point with one
+// frame for all: the tree of double-double additions it replaces took 12 us.
+__global__ void __launch_bounds__(256) k_dd_final(const double* __restrict__ part, long long n, double* __restrict__ out) {
   pdl_wait();
-  __shared__ double ss[256], sc[256];
-  double s = 0.0, c = 0.0;
-  for (long long t = threadIdx.x; t < n; t += blockDim.x) dd_add(s, c, part[2 * t], part[2 * t + 1]);
-  ss[threadIdx.x] = s;
-  sc[threadIdx.x] = c;
+  __shared__ int se[8];
+  __shared__ uint4 sl[8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int e = 0;
+  for (long long t = threadIdx.x; t < 2 * n; t += 256) e = max(e, WarpSum::exponent(part[t]));
+  e = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+  if (lane == 0) se[warp] = e;
   __syncthreads();
-  for (int st = 128; st > 0; st >>= 1) {
-    if ((int)threadIdx.x < st) {
-      double a = ss[threadIdx.x], ac = sc[threadIdx.x];
-      dd_add(a, ac, ss[threadIdx.x + st], sc[threadIdx.x + st]);
-      ss[threadIdx.x] = a;
-      sc[threadIdx.x] = ac;
-    }
-    __syncthreads();
+  for (int q = 0; q < 8; ++q) e = max(e, se[q]);
+  if (e == 0x7ff) {
+    if (threadIdx.x == 0) out[0] = __longlong_as_double(0x7ff8000000000000ll);
+    return;
   }
-  if (threadIdx.x == 0) out[0] = ss[0] + sc[0];
+  WarpSum a;
+  a.frame(e);
+  for (long long t = threadIdx.x; t < 2 * n; t += 256) a.add(part[t]);
+  a.reduce();
+  if (lane == 0) sl[warp] = make_uint4(a.l0, a.l1, a.l2, a.l3);
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int q = 1; q < 8; ++q) a.join(sl[q].x, sl[q].y, sl[q].z, sl[q].w);
+  a.collect();
+  out[0] = a.s + a.c;
 }
 
 // m = (S_f - beta * S_b) / V ; used by the solvability fix and mean-zero
