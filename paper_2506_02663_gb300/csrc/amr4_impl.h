@@ -79,7 +79,9 @@ struct CfiGroup {
   long long dst[8];  // fine ghost cells
   int cpatch;
   signed char pos[3];
-  signed char pad;
+  signed char face;  // 2 dir + (1 above the fine patch's high side)
+  int fpatch;        // fine patch
+  int pad;
 };
 
 // A rectangle of up to 8 x 8 coarse parents on one face of a fine patch (3-D, ratio 2) whose

@@ -309,6 +309,8 @@ static std::vector<CfiGroup> cfi_groups(const std::vector<CfiEntry>& cfi, const 
     CfiGroup g{};
     g.src = e0.src;
     g.cpatch = e0.cpatch;
+    g.face = (signed char)(2 * e0.dir + (e0.layer > 0 ? 1 : 0));
+    g.fpatch = e0.fpatch;
     for (int e = 0; e < 3; ++e) g.pos[e] = e0.pos[e];
     for (int c = 0; c < 8; ++c) g.dst[c] = -1;
     size_t j = i;

@@ -2744,52 +2744,42 @@ __device__ __forceinline__ void scatter_read(T* __restrict__ W, const PatchDesc&
 // Transposed refluxing (COH-3).  kind 0: Laplacian fluxes (face derivative, one field, all
 // W.p[] equal); kind 1: divergence fluxes (face values of component d into W.p[d]).  The
 // forward correction is out[c] += coef/hc * sum_faces s (Fbar/hf' - Fc/hc') with hf' = hf,
-// hc' = hc for derivatives and 1 for values.
+// hc' = hc for derivatives and 1 for values.  A thread per (cell, face, cell of the face's line):
+// as one thread per cell the lists of a 2-D level, a few hundred cells, took 10 us of serial
+// atomics and FP64 divisions on five SMs.
+constexpr int REFLUX_T_LANES = 4;
 template <typename T, int D>
-__global__ void k_reflux_T(LevelView crs, LevelView fine, const RefluxEntry* __restrict__ list, long long n,
-                           const T* __restrict__ z, Out3<T> W, T coef, int kind) {
+__global__ void __launch_bounds__(128) k_reflux_T(LevelView crs, LevelView fine, const RefluxEntry* __restrict__ list,
+                                                  long long n, const T* __restrict__ z, Out3<T> W, T coef, int kind) {
   pdl_wait();
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const RefluxEntry e = list[t];
+  const long long t = (long long)blockIdx.x * 128 + threadIdx.x;
+  const int q = (int)(t & 3), f = (int)((t >> 2) % (2 * D)), d = f >> 1, side = f & 1;
+  if (t >= n * (8 * D)) return;
+  const RefluxEntry& e = list[t / (8 * D)];
+  if (!(e.faces & (1 << f))) return;
   const T zc = z[e.coff];
   if (zc == T(0)) return;
-  const PatchDesc cp = crs.patches[e.cpatch];
-  const T fd[4] = {T(1.0 / 12.0), T(-15.0 / 12.0), T(15.0 / 12.0), T(-1.0 / 12.0)};
-  const T fv[4] = {T(-1.0 / 12.0), T(7.0 / 12.0), T(7.0 / 12.0), T(-1.0 / 12.0)};
-  const T* fc = kind == 0 ? fd : fv;
-  const T hc = pick<T>(crs.hd, crs.hf), hf = pick<T>(fine.hd, fine.hf);
-  const T a = coef * zc / hc;
-  const T hck = kind == 0 ? hc : T(1), hfk = kind == 0 ? hf : T(1);
-  for (int d = 0; d < D; ++d)
-    for (int side = 0; side < 2; ++side) {
-      if (!(e.faces & (1 << (2 * d + side)))) continue;
-      T* Wd = W.p[kind == 0 ? 0 : d];
-      const T s = T(side == 1 ? 1 : -1);
-      int own[3] = {e.g[0] - cp.lo[0], e.g[1] - cp.lo[1], e.g[2] - cp.lo[2]};
-      if (side == 0) own[d] -= 1;
-      for (int q = 0; q < 4; ++q) {
-        int cc[3] = {own[0], own[1], own[2]};
-        cc[d] += q - 1;
-        scatter_read<T, D>(Wd, cp, crs, cc, d, -a * s * fc[q] / hck);
-      }
-      const PatchDesc fp = fine.patches[e.fpatch[2 * d + side]];
-      const int e1 = (d == 0) ? 1 : 0;
-      const int e2 = (d == 2) ? 1 : 2;
-      const T fw = a * s / (T(D == 3 ? 4 : 2) * hfk);
-      for (int t2 = 0; t2 < (D == 3 ? 2 : 1); ++t2)
-        for (int t1 = 0; t1 < 2; ++t1) {
-          int gf[3] = {0, 0, 0};
-          gf[d] = side == 1 ? 2 * (e.g[d] + 1) - 1 : 2 * e.g[d] - 1;
-          gf[e1] = 2 * e.g[e1] + t1;
-          if (D == 3) gf[e2] = 2 * e.g[e2] + t2;
-          for (int q = 0; q < 4; ++q) {
-            int cc[3] = {gf[0] - fp.lo[0], gf[1] - fp.lo[1], gf[2] - fp.lo[2]};
-            cc[d] += q - 1;
-            atomicAdd(&Wd[poff(fp, cc[0], cc[1], cc[2])], fc[q] * fw);
-          }
-        }
-    }
+  const PatchDesc cp = crs.patches[e.cpatch], fp = fine.patches[e.fpatch[f]];
+  const T fq = kind == 0 ? (q == 0 ? T(1.0 / 12.0) : q == 1 ? T(-15.0 / 12.0) : q == 2 ? T(15.0 / 12.0) : T(-1.0 / 12.0))
+                         : (q == 0 || q == 3 ? T(-1.0 / 12.0) : T(7.0 / 12.0));
+  const T ihc = pick<T>(crs.invh, crs.invh_f), ihf = pick<T>(fine.invh, fine.invh_f);
+  const T a = coef * zc * ihc * T(side == 1 ? 1 : -1) * fq;
+  T* __restrict__ Wd = kind == 0 || d == 0 ? W.p[0] : d == 1 ? W.p[1] : W.p[2];
+  const int g0 = e.g[0], g1 = e.g[1], g2 = D == 3 ? e.g[2] : 0;
+  const int sc = side - 2 + q;  // coarse cells gd - 2 + side ..
+  int cc[3] = {g0 - cp.lo[0] + (d == 0 ? sc : 0), g1 - cp.lo[1] + (d == 1 ? sc : 0),
+               D == 3 ? g2 - cp.lo[2] + (d == 2 ? sc : 0) : 0};
+  scatter_read<T, D>(Wd, cp, crs, cc, d, kind == 0 ? -a * ihc : -a);
+  const T fw = (kind == 0 ? a * ihf : a) * T(D == 3 ? 0.25 : 0.5);
+  const int fd = q + 2 * side - 2;  // fine cells 2 gd - 2 + 2 side ..
+  const int b0 = 2 * g0 + (d == 0 ? fd : 0) - fp.lo[0], b1 = 2 * g1 + (d == 1 ? fd : 0) - fp.lo[1];
+  const int b2 = D == 3 ? 2 * g2 + (d == 2 ? fd : 0) - fp.lo[2] : 0;
+  const long long s1 = d == 0 ? (long long)fp.sy : 1, s2 = d == 2 ? (long long)fp.sy : (long long)fp.sz;
+  T* w = Wd + poff(fp, b0, b1, b2);
+#pragma unroll
+  for (int t2 = 0; t2 < (D == 3 ? 2 : 1); ++t2)
+#pragma unroll
+    for (int t1 = 0; t1 < 2; ++t1) atomicAdd(w + t1 * s1 + t2 * s2, fw);
 }
 
 // Transposed G^comp stencil (Eq. discreteOps a): each valid cell o hands z_d[o]/(12h) times
@@ -2878,6 +2868,64 @@ __global__ void k_cfi_T(const CfiEntry* __restrict__ list, long long n, const lo
       for (int c1 = 0; c1 < CFI_W; ++c1)
         for (int c0 = 0; c0 < CFI_W; ++c0, ++q)
           atomicAdd(&W[sd[q]], cfiw<T>(b0 + c0) * cfiw<T>(b1 + c1) * (D == 3 ? cfiw<T>(b2 + c2) : T(1)) * wg);
+  }
+}
+
+// The same by groups of the 2^D ghosts that share a window (ratio 2): a warp per group forms their
+// weights, folds them dimension by dimension -- a lane per (x, y) of the window, its cells along z
+// in turn -- and adds every window cell once, where a thread per ghost made 2^D times as many
+// atomic additions (64^3 box: 33 us per pass in FP32).
+template <typename T, int D>
+__global__ void __launch_bounds__(128) k_cfi_T_grp(const CfiGroup* __restrict__ list, long long n,
+                                                   const long long* __restrict__ side,
+                                                   const PatchDesc* __restrict__ cpatches,
+                                                   const PatchDesc* __restrict__ fpatches, const T* __restrict__ z,
+                                                   const T* wghost, T* W, T beta_inv12h2, T sign) {
+  pdl_wait();
+  constexpr int NC = D == 3 ? 8 : 4;
+  const long long t = (long long)blockIdx.x * 4 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (t >= n) return;
+  const CfiGroup& g = list[t];
+  T wg = T(0);
+  const int dir = g.face >> 1;
+  if (lane < NC && g.dst[lane] >= 0) {
+    const PatchDesc fp = fpatches[g.fpatch];
+    const int hi = g.face & 1, sub = (lane >> dir) & 1;  // layer 1 next to the interior
+    const long long st = dir == 0 ? 1 : dir == 1 ? (long long)fp.sy : (long long)fp.sz, step = hi ? -st : st;
+    const long long dst = g.dst[lane];
+    const T* zi = z + dst + step;
+    wg = sub != hi ? T(16) * zi[0] - zi[step] : -zi[step];
+    wg = sign * (wg * beta_inv12h2 + (wghost != nullptr ? wghost[dst] : T(0)));
+  }
+  if (!__any_sync(0xffffffffu, wg != T(0))) return;
+  T w[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) w[c] = __shfl_sync(0xffffffffu, wg, c);
+  if (lane >= CFI_W * CFI_W) return;
+  const int c0 = lane % CFI_W, c1 = lane / CFI_W;
+  const int i0 = 2 * g.pos[0] * CFI_W + c0, i1 = 2 * g.pos[1] * CFI_W + c1, i2 = 2 * g.pos[2] * CFI_W;
+  const T u00 = cfiw<T>(i0), u01 = cfiw<T>(i0 + CFI_W), u10 = cfiw<T>(i1), u11 = cfiw<T>(i1 + CFI_W);
+  T f[2];
+#pragma unroll
+  for (int c = 0; c < (D == 3 ? 2 : 1); ++c)
+    f[c] = fma(u11, fma(u01, w[4 * c + 3], u00 * w[4 * c + 2]), u10 * fma(u01, w[4 * c + 1], u00 * w[4 * c]));
+  if (g.src >= 0) {
+    const PatchDesc& cp = cpatches[g.cpatch];
+    T* p = W + g.src + c0 + (long long)c1 * cp.sy;
+    if (D == 3) {
+      const long long sz = cp.sz;
+      for (int c2 = 0; c2 < CFI_W; ++c2) atomicAdd(p + c2 * sz, fma(cfiw<T>(i2 + CFI_W + c2), f[1], cfiw<T>(i2 + c2) * f[0]));
+    } else {
+      atomicAdd(p, f[0]);
+    }
+  } else {
+    const long long* sd = side + (-1 - g.src) * (D == 3 ? 125 : 25) + lane;
+    if (D == 3)
+      for (int c2 = 0; c2 < CFI_W; ++c2)
+        atomicAdd(W + sd[c2 * CFI_W * CFI_W], fma(cfiw<T>(i2 + CFI_W + c2), f[1], cfiw<T>(i2 + c2) * f[0]));
+    else
+      atomicAdd(W + sd[0], f[0]);
   }
 }
 

@@ -12,6 +12,47 @@
 
 namespace amr4 {
 
+// One dimension of the transposed operator (trans_sums) with what does not depend on the plane
+// formed once per column: which neighbours exist, and the weights of the two cells next to the
+// near face that the cell's rows of the ghost formulas put on it.  Domains of eight cells and
+// more, so that a cell is near one face only.
+template <typename T>
+struct TransLine {
+  T a, b;          // ex += a x[f] + b x[f + s]
+  int f, s;        // offset of the face cell from the cell; step into the domain
+  bool near, m1, p1, m2, p2;
+  __device__ __forceinline__ TransLine(int g, int n, int plo, int pn, int st, int tlo, int thi) {
+    m1 = g >= 1;
+    p1 = g + 1 < n;
+    m2 = g >= 2;
+    p2 = g + 2 < n;
+    const bool low = g <= 3 && plo == 0, high = n - 1 - g <= 3 && plo + pn == n;
+    near = g < 4 || n - 1 - g < 4;
+    a = b = T(0);
+    f = s = 0;
+    if (low || high) {
+      const int m = low ? g : n - 1 - g, t = low ? tlo : thi;
+      const T c0 = gcoef<T>(t, 0, m), c1 = gcoef<T>(t, 1, m);
+      a = T(16) * c0 - c1;
+      b = -c0;
+      s = low ? st : -st;
+      f = -m * s;
+    }
+  }
+  __device__ __forceinline__ void sums(const T* __restrict__ xb, int o, int st, T& s1, T& s2, T& ex) const {
+    if (!near) {
+      s1 = xb[o - st] + xb[o + st];
+      s2 = xb[o - 2 * st] + xb[o + 2 * st];
+      return;
+    }
+    const T v1 = m1 ? xb[o - st] : T(0), w1 = p1 ? xb[o + st] : T(0), v2 = m2 ? xb[o - 2 * st] : T(0),
+            w2 = p2 ? xb[o + 2 * st] : T(0);
+    s1 = v1 + w1;
+    s2 = v2 + w2;
+    ex = fma(a, xb[o + f], fma(b, xb[o + f + s], ex));
+  }
+};
+
 // Level operator (OP_APPLY, OP_RESID, OP_JACOBI, OP_JACOBI0; homogeneous data; TR: its transpose).  A thread owns
 // one (x, y) column of a patch -- columns numbered linearly, so narrow grids fill their warps --
 // and kz planes of it, its z neighbours in a register queue.  The host sizes kz so that small
@@ -38,7 +79,10 @@ __global__ void __launch_bounds__(128) k_level_op3d_col(LevelView lv, int kz, co
   const int sy = (int)p.sy, sz = (int)p.sz;
   const int gx = p.lo[0] + i, gy = p.lo[1] + j, lz = p.lo[2], nzd = lv.ndom[2];
   const int cx = face_class(gx, lv.ndom[0]), cy = face_class(gy, lv.ndom[1]);
-  const bool inx = gx >= 4 && gx <= lv.ndom[0] - 5, iny = gy >= 4 && gy <= lv.ndom[1] - 5;  // transposed: no ghost rows
+  // transposed: small domains take trans_sums plane by plane
+  const bool wide = TR && lv.ndom[0] >= 8 && lv.ndom[1] >= 8;
+  const TransLine<T> tx(gx, lv.ndom[0], p.lo[0], p.n[0], 1, lv.bc[0], lv.bc[1]);
+  const TransLine<T> ty(gy, lv.ndom[1], p.lo[1], p.n[1], sy, lv.bc[2], lv.bc[3]);
   const T* __restrict__ xb = x + p.off;
   const T* fb = f + p.off;  // may be out (in-place residual)
   T* ob = out + p.off;
@@ -65,16 +109,11 @@ __global__ void __launch_bounds__(128) k_level_op3d_col(LevelView lv, int kz, co
     if (MODE != OP_APPLY) fk = fb[o];
     T x1, x2, y1, y2, z1, z2, ex = T(0);
     if (TR) {
-      if (inx) {
-        x1 = xb[o - 1] + xb[o + 1];
-        x2 = xb[o - 2] + xb[o + 2];
+      if (wide) {
+        tx.sums(xb, o, 1, x1, x2, ex);
+        ty.sums(xb, o, sy, y1, y2, ex);
       } else {
         trans_sums<T>(xb, o, 1, i, lv.ndom[0], p.lo[0], p.n[0], lv.bc[0], lv.bc[1], x1, x2, ex);
-      }
-      if (iny) {
-        y1 = xb[o - sy] + xb[o + sy];
-        y2 = xb[o - 2 * sy] + xb[o + 2 * sy];
-      } else {
         trans_sums<T>(xb, o, sy, j, lv.ndom[1], p.lo[1], p.n[1], lv.bc[2], lv.bc[3], y1, y2, ex);
       }
       if (gz >= 4 && gz <= nzd - 5) {
@@ -254,7 +293,7 @@ __global__ void __launch_bounds__(256) k_restrict3d_resid(LevelView fine, LevelV
 // Prolongation by coarse parent on any grid: one thread per coarse cell gathers the 27 coarse
 // values around it, with the homogeneous layer-1 extension where the neighbourhood leaves the
 // domain (dimension after dimension, Fig. 1(c); four inward cells per dimension instead of
-// three), and updates its eight children, whose sums are k_prolong3d's in order and weights.
+// three), and updates its eight children.
 // Replaces one thread per fine cell with the face cells' 64-term products inline: 143 us for
 // an FP64 72^3 grid, 45 us for 36^3.
 template <typename T>

@@ -763,8 +763,8 @@ amr_status level_op(int mode, const LevelView& lv, const T* x, const T* f, T* ou
   if constexpr (D == 3) {
     if (bc == nullptr && (!TR || vmask == nullptr) && small_offsets(lv)) {
       // any other homogeneous 3-D level: one thread per column and run of kz planes, as many runs
-      // as give every SM 16 warps (a quarter of its slots: enough loads in flight for L2, and long
-      // runs where the grid allows them)
+      // as give every SM 32 warps (half of its slots: enough loads in flight for L2, and long runs
+      // where the grid allows them)
       const long long warps = (long long)lv.npatch * ((lv.maxn[0] * (long long)lv.maxn[1] + 31) / 32);
       const long long want = 32LL * sm_count();
       const int nz = lv.maxn[2];
@@ -900,6 +900,9 @@ struct P3 {
   const T* p[3];
 };
 
+// lanes per coarse cell of the reflux kernels: its faces, rounded up to a power of two
+template <int D>
+__host__ __device__ constexpr int reflux_lanes() { return D == 3 ? 8 : 4; }
 template <typename T, int D>
 __global__ void k_reflux_p3(LevelView crs, LevelView fine, const RefluxEntry* __restrict__ list, long long n,
                             P3<T> xcs, P3<T> xfs, P3<T> bcs, T* __restrict__ out, T coef, int kind);
@@ -909,8 +912,8 @@ amr_status reflux(const amr_hierarchy* h, int l, const LevelView& crs, const Lev
                   P3<T> bcs, T* out, double coef, int kind, cudaStream_t st) {
   const DeviceLists& dl = h->lev[l].dev;
   if (dl.nreflux == 0) return AMR_OK;
-  const int nt = 32;  // as above
-  launch(k_reflux_p3<T, D>, (unsigned)((dl.nreflux + nt - 1) / nt), nt, 0, st, crs, fine, dl.reflux, dl.nreflux, xc, xf,
+  const int nt = 128;
+  launch(k_reflux_p3<T, D>, (unsigned)((dl.nreflux * reflux_lanes<D>() + nt - 1) / nt), nt, 0, st, crs, fine, dl.reflux, dl.nreflux, xc, xf,
                                                                          bcs, out, T(coef), kind);
   return launch_check();
 }
@@ -935,72 +938,82 @@ amr_status convert(const LevelView& lv, const S* x, T* y, cudaStream_t st) {
 // reflux kernel with by-value pointer triples (defined outside the anonymous namespace
 // declaration above so that it can be instantiated)
 namespace {
-// Refluxing (COH-3) of one coarse cell: its flux through every coarse-fine face replaced by
-// the mean of the fine fluxes.  KIND 0: the derivative flux of L (1/12, -15/12, 15/12, -1/12
-// divided by h); KIND 1: the face value of D (-1/12, 7/12, 7/12, -1/12).  Reciprocals of h
-// instead of divisions: FP64 division is slow on this part.
-template <typename T, int D, int KIND>
-__device__ __forceinline__ void reflux_cell(const LevelView& crs, const LevelView& fine, const RefluxEntry& e,
-                                            const P3<T>& xcs, const P3<T>& xfs, const P3<T>& bcs, T* __restrict__ out,
-                                            T coef) {
-  constexpr double FC[2][4] = {{1.0 / 12.0, -15.0 / 12.0, 15.0 / 12.0, -1.0 / 12.0},
-                               {-1.0 / 12.0, 7.0 / 12.0, 7.0 / 12.0, -1.0 / 12.0}};
-  const PatchDesc cp = crs.patches[e.cpatch];
-  const T ihc = KIND == 0 ? pick<T>(crs.invh, crs.invh_f) : T(1);
-  const T ihf = KIND == 0 ? pick<T>(fine.invh, fine.invh_f) : T(1);
+// Refluxing (COH-3): a coarse cell's flux through every coarse-fine face replaced by the mean of
+// the fine fluxes.  kind 0: the derivative flux of L (1/12, -15/12, 15/12, -1/12 divided by h);
+// kind 1: the face value of D (-1/12, 7/12, 7/12, -1/12).  Reciprocals of h instead of
+// divisions: FP64 division is slow on this part.  A lane per (cell, face), the faces of a cell
+// summed by shuffle: a cell has one such face, rarely two or three, and the thread per cell with
+// its six faces in turn spent its time fetching six copies of the code.
+template <typename T, int D>
+__global__ void __launch_bounds__(128) k_reflux_p3(LevelView crs, LevelView fine, const RefluxEntry* __restrict__ list,
+                                                   long long n, P3<T> xcs, P3<T> xfs, P3<T> bcs, T* __restrict__ out, T coef,
+                                                   int kind) {
+  constexpr int FL = reflux_lanes<D>();
+  pdl_wait();
+  const long long t = ((long long)blockIdx.x * 128 + threadIdx.x) / FL;
+  const int f = threadIdx.x % FL, d = f >> 1, side = f & 1;
   T corr = T(0);
-#pragma unroll
-  for (int d = 0; d < D; ++d)
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {
-      if (!(e.faces & (1 << (2 * d + side)))) continue;
-      const int comp = KIND == 0 ? 0 : d;
-      const T* xc = xcs.p[comp];
-      const T* xf = xfs.p[comp];
-      int own[3] = {e.g[0] - cp.lo[0], e.g[1] - cp.lo[1], e.g[2] - cp.lo[2]};
-      if (side == 0) own[d] -= 1;
-      T Fc = T(0);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        int cc[3] = {own[0], own[1], own[2]};
-        cc[d] += q - 1;
-        Fc += T(FC[KIND][q]) * read_nb<T, D>(xc, cp, crs, bcs.p[comp], cc[0], cc[1], cc[2], d);
+  long long coff = 0;
+  if (t < n) {
+    const RefluxEntry& e = list[t];
+    coff = e.coff;
+    if (f < 2 * D && (e.faces & (1 << f))) {
+      const PatchDesc cp = crs.patches[e.cpatch];
+      const PatchDesc fp = fine.patches[e.fpatch[f]];
+      const T* __restrict__ xc = kind == 0 ? xcs.p[0] : d == 0 ? xcs.p[0] : d == 1 ? xcs.p[1] : xcs.p[2];
+      const T* __restrict__ xf = kind == 0 ? xfs.p[0] : d == 0 ? xfs.p[0] : d == 1 ? xfs.p[1] : xfs.p[2];
+      const T* bc = kind == 0 ? bcs.p[0] : d == 0 ? bcs.p[0] : d == 1 ? bcs.p[1] : bcs.p[2];
+      const T c0 = kind == 0 ? T(1.0 / 12.0) : T(-1.0 / 12.0), c1 = kind == 0 ? T(-15.0 / 12.0) : T(7.0 / 12.0);
+      const T c2 = kind == 0 ? T(15.0 / 12.0) : T(7.0 / 12.0), c3 = -T(1.0 / 12.0);
+      const T ihc = kind == 0 ? pick<T>(crs.invh, crs.invh_f) : T(1);
+      const T ihf = kind == 0 ? pick<T>(fine.invh, fine.invh_f) : T(1);
+      const int g0 = e.g[0], g1 = e.g[1], g2 = D == 3 ? e.g[2] : 0;
+      const int gd = d == 0 ? g0 : d == 1 ? g1 : g2, nd = d == 0 ? crs.ndom[0] : d == 1 ? crs.ndom[1] : crs.ndom[2];
+      // coarse cells gd - 2 + side .. gd + 1 + side of the line along d
+      const int first = gd - 2 + side;
+      const int a0 = g0 - cp.lo[0], a1 = g1 - cp.lo[1], a2 = D == 3 ? g2 - cp.lo[2] : 0;
+      T Fc;
+      if (first >= 0 && first + 3 < nd) {
+        const long long st = d == 0 ? 1 : d == 1 ? (long long)cp.sy : (long long)cp.sz;
+        const T* q = xc + poff(cp, a0, a1, a2) + (long long)(side - 2) * st;
+        Fc = T(0) + c0 * q[0];
+        Fc += c1 * q[st];
+        Fc += c2 * q[2 * st];
+        Fc += c3 * q[3 * st];
+      } else {
+        Fc = T(0);
+#pragma unroll 1
+        for (int q = 0; q < 4; ++q) {
+          const int s = side - 2 + q;
+          const T v = read_nb<T, D>(xc, cp, crs, bc, a0 + (d == 0 ? s : 0), a1 + (d == 1 ? s : 0), a2 + (d == 2 ? s : 0), d);
+          Fc += (q == 0 ? c0 : q == 1 ? c1 : q == 2 ? c2 : c3) * v;
+        }
       }
-      const PatchDesc fp = fine.patches[e.fpatch[2 * d + side]];
+      // fine cells: along d the face's two on each side, across it the 2 (4) fine faces
+      const int fd = side == 1 ? 2 * gd : 2 * gd - 2;  // first cell of the line
+      const int b0 = (d == 0 ? fd : 2 * g0) - fp.lo[0], b1 = (d == 1 ? fd : 2 * g1) - fp.lo[1];
+      const int b2 = D == 3 ? (d == 2 ? fd : 2 * g2) - fp.lo[2] : 0;
+      const long long sd = d == 0 ? 1 : d == 1 ? (long long)fp.sy : (long long)fp.sz;
+      const long long s1 = d == 0 ? (long long)fp.sy : 1, s2 = d == 2 ? (long long)fp.sy : (long long)fp.sz;
+      const T* q = xf + poff(fp, b0, b1, b2);
       T Fs = T(0);
-      const int t1d = (d == 0) ? 1 : 0;
-      const int t2d = (d == 2) ? 1 : 2;
 #pragma unroll
       for (int t2 = 0; t2 < (D == 3 ? 2 : 1); ++t2)
 #pragma unroll
         for (int t1 = 0; t1 < 2; ++t1) {
-          int gf[3] = {0, 0, 0};
-          gf[d] = side == 1 ? 2 * (e.g[d] + 1) - 1 : 2 * e.g[d] - 1;
-          gf[t1d] = 2 * e.g[t1d] + t1;
-          if (D == 3) gf[t2d] = 2 * e.g[t2d] + t2;
-          const int cf[3] = {gf[0] - fp.lo[0], gf[1] - fp.lo[1], gf[2] - fp.lo[2]};
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            int cc[3] = {cf[0], cf[1], cf[2]};
-            cc[d] += q - 1;
-            Fs += T(FC[KIND][q]) * xf[poff(fp, cc[0], cc[1], cc[2])];
-          }
+          const T* r = q + t1 * s1 + t2 * s2;
+          Fs += c0 * r[0];
+          Fs += c1 * r[sd];
+          Fs += c2 * r[2 * sd];
+          Fs += c3 * r[3 * sd];
         }
       const T Fbar = Fs * T(D == 3 ? 0.25 : 0.5);
-      corr += T(side == 1 ? 1 : -1) * (Fbar * ihf - Fc * ihc);
+      corr = T(side == 1 ? 1 : -1) * (Fbar * ihf - Fc * ihc);
     }
-  out[e.coff] += coef * corr * pick<T>(crs.invh, crs.invh_f);
-}
-
-template <typename T, int D>
-__global__ void k_reflux_p3(LevelView crs, LevelView fine, const RefluxEntry* __restrict__ list, long long n,
-                            P3<T> xcs, P3<T> xfs, P3<T> bcs, T* __restrict__ out, T coef, int kind) {
-  pdl_wait();
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const RefluxEntry e = list[t];
-  if (kind == 0) reflux_cell<T, D, 0>(crs, fine, e, xcs, xfs, bcs, out, coef);
-  else reflux_cell<T, D, 1>(crs, fine, e, xcs, xfs, bcs, out, coef);
+  }
+#pragma unroll
+  for (int st = 1; st < FL; st <<= 1) corr += __shfl_xor_sync(0xffffffffu, corr, st);
+  if (t < n && f == 0) out[coff] += coef * corr * pick<T>(crs.invh, crs.invh_f);
 }
 
 // ---------------------------------------------------------------- scratch management
@@ -1861,6 +1874,21 @@ amr_status mg_level0(amr_operator* op, const amr_solver_params& p, int m, const 
   return AMR_OK;
 }
 
+// Transposed AMRCFI of level l: the ghosts' weights to their coarse windows (k_cfi_T)
+template <typename T, int D>
+amr_status cfi_transpose(amr_hierarchy* h, int l, const T* z, const T* wghost, T* W, T beta_inv12h2, T sign,
+                         cudaStream_t st) {
+  const DeviceLists& dl = h->lev[l].dev;
+  const int nt = 128;
+  if (dl.ncfig > 0)
+    launch(k_cfi_T_grp<T, D>, (unsigned)((dl.ncfig + 3) / 4), nt, 0, st, dl.cfig, dl.ncfig, dl.cfi_side,
+           h->lev[l - 1].d_patches, h->lev[l].d_patches, z, wghost, W, beta_inv12h2, sign);
+  else
+    launch(k_cfi_T<T, D>, (unsigned)((dl.ncfi + nt - 1) / nt), nt, 0, st, dl.cfi, dl.ncfi, dl.cfi_side,
+           h->lev[l - 1].d_patches, h->lev[l].d_patches, h->r, z, wghost, W, beta_inv12h2, sign);
+  return launch_check();
+}
+
 // ---------------------------------------------------------------- composite transpose
 // S.W <- (A^comp)^T x over every covered cell (valid entries are the result; the rest is
 // scratch): z = x on valid cells (0 elsewhere, copies of siblings in the copy ghosts),
@@ -1889,7 +1917,7 @@ amr_status composite_AT(amr_operator* op, const T* x, cudaStream_t st, int only_
   for (int l = 0; l + 1 < h->L; ++l) {
     const DeviceLists& dl = h->lev[l].dev;
     if (dl.nreflux == 0) continue;
-    launch(k_reflux_T<T, D>, (unsigned)((dl.nreflux + nt - 1) / nt), nt, 0, st, 
+    launch(k_reflux_T<T, D>, (unsigned)((dl.nreflux * REFLUX_T_LANES * 2 * D + nt - 1) / nt), nt, 0, st,
         level_view(h, l, op->bc), level_view(h, l + 1, op->bc), dl.reflux, dl.nreflux, S.Z, Out3<T>{{S.W, S.W, S.W}},
         T(op->beta), 0);
     TRY(launch_check());
@@ -1904,10 +1932,8 @@ amr_status composite_AT(amr_operator* op, const T* x, cudaStream_t st, int only_
     const DeviceLists& dl = h->lev[l].dev;
     if (dl.ncfi == 0) continue;
     const LevelView fv = level_view(h, l, op->bc);
-    launch(k_cfi_T<T, D>, (unsigned)((dl.ncfi + nt - 1) / nt), nt, 0, st, 
-        dl.cfi, dl.ncfi, dl.cfi_side, h->lev[l - 1].d_patches, h->lev[l].d_patches, h->r, S.Z, S.W, S.W,
-        T(op->beta * fv.inv12h2), T(1));
-    TRY(launch_check());
+    TRY((cfi_transpose<T, D>(h, l, S.Z, S.W, S.W,
+        T(op->beta * fv.inv12h2), T(1), st)));
   }
   for (int l = 0; l + 1 < h->L; ++l) {
     const DeviceLists& dl = h->lev[l].dev;
@@ -2005,10 +2031,8 @@ amr_status vcycle_corr_T(amr_operator* op, const amr_solver_params& p, const T* 
     {
       const DeviceLists& dl = h->lev[l].dev;
       if (dl.ncfi) {
-        launch(k_cfi_T<T, D>, (unsigned)((dl.ncfi + nt - 1) / nt), nt, 0, st, 
-            dl.cfi, dl.ncfi, dl.cfi_side, h->lev[l - 1].d_patches, h->lev[l].d_patches, h->r, Rb, (const T*)nullptr,
-            Eb, T(b_ * lv[l].inv12h2), T(-1));
-        TRY(launch_check());
+        TRY((cfi_transpose<T, D>(h, l, Rb, (const T*)nullptr,
+            Eb, T(b_ * lv[l].inv12h2), T(-1), st)));
       }
     }
     // U1^T: Eb_{l-1} += P^T (Eb_l + Xb_l)
@@ -3050,9 +3074,7 @@ amr_status ghost_fill_T(amr_hierarchy* h, double* W, cudaStream_t st) {
   for (int l = h->L - 1; l >= 1; --l) {
     const DeviceLists& dl = h->lev[l].dev;
     if (dl.ncfi == 0) continue;
-    launch(k_cfi_T<double, D>, (unsigned)((dl.ncfi + nt - 1) / nt), nt, 0, st, 
-        dl.cfi, dl.ncfi, dl.cfi_side, h->lev[l - 1].d_patches, h->lev[l].d_patches, h->r, W, W, W, 0.0, 1.0);
-    TRY(launch_check());
+    TRY((cfi_transpose<double, D>(h, l, W, W, W, 0.0, 1.0, st)));
   }
   TRY(avgdown_T_all<D>(h, W, st));
   for (int l = 0; l < h->L; ++l) {
@@ -3105,7 +3127,7 @@ amr_status divergence_T_impl(amr_hierarchy* h, const int* bct, const double* y, 
   for (int l = 0; l + 1 < h->L; ++l) {
     const DeviceLists& dl = h->lev[l].dev;
     if (dl.nreflux == 0) continue;
-    launch(k_reflux_T<double, D>, (unsigned)((dl.nreflux + nt - 1) / nt), nt, 0, st, 
+    launch(k_reflux_T<double, D>, (unsigned)((dl.nreflux * REFLUX_T_LANES * 2 * D + nt - 1) / nt), nt, 0, st,
         level_view(h, l, bct), level_view(h, l + 1, bct), dl.reflux, dl.nreflux, Z, W, 1.0, 1);
     TRY(launch_check());
   }
