@@ -2961,19 +2961,6 @@ __global__ void k_copy_T(const CopyEntry* __restrict__ list, long long n, T* __r
   }
 }
 
-// out = vmask ? (f ? f - w : w) : 0 on interior cells (composite transpose epilogue; also
-// used to copy the valid part of a field)
-template <typename T, int D>
-__global__ void k_valid_out(LevelView lv, int nby, const T* __restrict__ w, const T* __restrict__ f, T* __restrict__ out,
-                            const unsigned char* __restrict__ vmask) {
-  pdl_wait();
-  const PatchDesc p = lv.patches[blockIdx.z];
-  int i, j, k;
-  if (!thread_cell<D>(p, nby, i, j, k)) return;
-  const long long o = poff(p, i, j, k);
-  out[o] = vmask[o] ? (f != nullptr ? f[o] - w[o] : w[o]) : T(0);
-}
-
 // Transposed prolongation (Sec. 6.5 linear interpolation): every fine cell hands
 // w * (y1 + y2) to each coarse cell its interpolation reads (atomic adds); coarse positions
 // outside the domain pass their weight on through the homogeneous extension.
@@ -3038,18 +3025,6 @@ __global__ void k_prolong_T(LevelView fine, LevelView crs, const XferBlock* __re
       }
 }
 
-// y += a * x on valid interior cells (x is read as 0 elsewhere)
-template <typename T, int D>
-__global__ void k_axpy_valid(LevelView lv, int nby, const T* __restrict__ x, T* __restrict__ y, T a,
-                             const unsigned char* __restrict__ vmask) {
-  pdl_wait();
-  const PatchDesc p = lv.patches[blockIdx.z];
-  int i, j, k;
-  if (!thread_cell<D>(p, nby, i, j, k)) return;
-  const long long o = poff(p, i, j, k);
-  if (vmask[o]) y[o] += a * x[o];
-}
-
 // Transposed average-down from one coarse buffer into a fine buffer: y_f += y_c / 2^D for
 // every fine cell of the transfer blocks (the coarse cells are the invalid ones).
 template <typename T, int D>
@@ -3069,32 +3044,102 @@ __global__ void k_avgdown_T2(LevelView fine, LevelView crs, const XferBlock* __r
   yf[poff(fp, gf[0] - fp.lo[0], gf[1] - fp.lo[1], gf[2] - fp.lo[2])] += wc * T(D == 3 ? 0.125 : 0.25);
 }
 
-// out = f - w on valid interior cells only (other cells untouched)
-template <typename T, int D>
-__global__ void k_level_op_masked_copy(LevelView lv, int nby, const T* __restrict__ w, const T* __restrict__ f,
-                                       T* __restrict__ out, const unsigned char* __restrict__ vmask) {
+// ------------------------------------------------------------------------ elementwise
+// A pass over the interior cells of a level: a warp takes rows, a lane up to ROW_K of its cells at
+// once, their loads issued together (F::load), then their stores (F::store).  Bound by memory: as
+// one thread per cell in 65,536 blocks, X += E on 256^3 took 60 us where its bytes take 30.
+constexpr int ROW_K = 4;
+template <int D, typename F>
+__global__ void __launch_bounds__(256) k_rows(LevelView lv, F f) {
   pdl_wait();
-  const PatchDesc p = lv.patches[blockIdx.z];
-  int i, j, k;
-  if (!thread_cell<D>(p, nby, i, j, k)) return;
-  const long long o = poff(p, i, j, k);
-  if (vmask[o]) out[o] = f[o] - w[o];
+  const PatchDesc p = lv.npatch == 1 ? lv.p0 : lv.patches[blockIdx.y];
+  const int lane = threadIdx.x & 31, rows = p.n[1] * (D == 3 ? p.n[2] : 1), nw = gridDim.x * 8;
+  f.begin();
+  for (int row = blockIdx.x * 8 + (threadIdx.x >> 5); row < rows; row += nw) {
+    const long long o0 = poff(p, 0, row % p.n[1], D == 3 ? row / p.n[1] : 0);
+    for (int i0 = lane; i0 < p.n[0]; i0 += 32 * ROW_K) {
+      typename F::V v[ROW_K];
+#pragma unroll
+      for (int q = 0; q < ROW_K; ++q)
+        if (i0 + 32 * q < p.n[0]) v[q] = f.load(o0 + i0 + 32 * q);
+#pragma unroll
+      for (int q = 0; q < ROW_K; ++q)
+        if (i0 + 32 * q < p.n[0]) f.store(o0 + i0 + 32 * q, v[q]);
+    }
+  }
 }
 
-// ------------------------------------------------------------------------ elementwise
-// y[o] += a * x[o] on the interior cells of a level (optionally also y2[o] += a * x[o]);
-// source type S, destination type T.
-template <typename S, typename T, int D>
-__global__ void k_axpy(LevelView lv, int nby, const S* __restrict__ x, T* __restrict__ y, T* __restrict__ y2, T a) {
-  pdl_wait();
-  const PatchDesc p = lv.patches[blockIdx.z];
-  int i, j, k;
-  if (!thread_cell<D>(p, nby, i, j, k)) return;
-  const long long o = poff(p, i, j, k);
-  const T v = a * cvt<T, S>(x[o]);
-  y[o] += v;
-  if (y2 != nullptr) y2[o] += v;
-}
+// y += a x (optionally also y2 += a x); source type S, destination type T
+template <typename S, typename T>
+struct RowAxpy {
+  const S* x;
+  T *y, *y2;
+  T a;
+  struct V {
+    T d, y, y2;
+  };
+  __device__ __forceinline__ void begin() {}
+  __device__ __forceinline__ V load(long long o) const { return V{a * cvt<T, S>(x[o]), y[o], y2 != nullptr ? y2[o] : T(0)}; }
+  __device__ __forceinline__ void store(long long o, const V& v) const {
+    y[o] = v.y + v.d;
+    if (y2 != nullptr) y2[o] = v.y2 + v.d;
+  }
+};
+
+// y += a x on valid cells (x is read as 0 elsewhere)
+template <typename T>
+struct RowAxpyValid {
+  const T* x;
+  T* y;
+  T a;
+  const unsigned char* vmask;
+  struct V {
+    T x, y;
+    unsigned char m;
+  };
+  __device__ __forceinline__ void begin() {}
+  __device__ __forceinline__ V load(long long o) const { return V{x[o], y[o], vmask[o]}; }
+  __device__ __forceinline__ void store(long long o, const V& v) const {
+    if (v.m) y[o] = v.y + a * v.x;
+  }
+};
+
+// out = f - w (f null: w) on valid cells, zero on invalid ones (used to copy the valid part of a
+// field); keep: invalid cells untouched
+template <typename T>
+struct RowValidOut {
+  const T *w, *f;
+  T* out;
+  const unsigned char* vmask;
+  bool keep;
+  struct V {
+    T w, f;
+    unsigned char m;
+  };
+  __device__ __forceinline__ void begin() {}
+  __device__ __forceinline__ V load(long long o) const { return V{w[o], f != nullptr ? f[o] : T(0), vmask[o]}; }
+  __device__ __forceinline__ void store(long long o, const V& v) const {
+    if (v.m) out[o] = f != nullptr ? v.f - v.w : v.w;
+    else if (!keep) out[o] = T(0);
+  }
+};
+
+// y += sign * a[0] (vmask non-null: on valid cells)
+struct RowShift {
+  double* y;
+  const double* a;
+  const unsigned char* vmask;
+  double sign, s;
+  struct V {
+    double y;
+    unsigned char m;
+  };
+  __device__ __forceinline__ void begin() { s = a[0]; }
+  __device__ __forceinline__ V load(long long o) const { return V{y[o], vmask != nullptr ? vmask[o] : (unsigned char)1}; }
+  __device__ __forceinline__ void store(long long o, const V& v) const {
+    if (v.m) y[o] = v.y + sign * s;
+  }
+};
 
 template <typename S, typename T, int D>
 __global__ void k_convert(LevelView lv, int nby, const S* __restrict__ x, T* __restrict__ y) {
@@ -3104,19 +3149,6 @@ __global__ void k_convert(LevelView lv, int nby, const S* __restrict__ x, T* __r
   if (!thread_cell<D>(p, nby, i, j, k)) return;
   const long long o = poff(p, i, j, k);
   y[o] = cvt<T, S>(x[o]);
-}
-
-// y[o] += a on interior cells (mask: only valid cells when vmask != null)
-template <int D>
-__global__ void k_shift(LevelView lv, int nby, double* __restrict__ y, const double* __restrict__ a,
-                        const unsigned char* __restrict__ vmask, double sign) {
-  pdl_wait();
-  const PatchDesc p = lv.patches[blockIdx.z];
-  int i, j, k;
-  if (!thread_cell<D>(p, nby, i, j, k)) return;
-  const long long o = poff(p, i, j, k);
-  if (vmask != nullptr && vmask[o] == 0) return;
-  y[o] += sign * a[0];
 }
 
 // out = w - g on interior cells

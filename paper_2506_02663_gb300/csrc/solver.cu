@@ -918,11 +918,17 @@ amr_status reflux(const amr_hierarchy* h, int l, const LevelView& crs, const Lev
   return launch_check();
 }
 
+// an elementwise pass over a level's rows: enough blocks to fill the chip, the rest by stride
+template <int D, typename F>
+amr_status row_pass(const LevelView& lv, const F& f, cudaStream_t st) {
+  const long long rows = (long long)lv.maxn[1] * (D == 3 ? lv.maxn[2] : 1);
+  launch(k_rows<D, F>, dim3((unsigned)std::min<long long>((rows + 7) / 8, 16LL * sm_count()), lv.npatch, 1), 256, 0, st, lv, f);
+  return launch_check();
+}
+
 template <typename S, typename T, int D>
 amr_status axpy(const LevelView& lv, const S* x, T* y, T* y2, double a, cudaStream_t st) {
-  Geo g = geo_of(lv);
-  launch(k_axpy<S, T, D>, g.grid, g.block, 0, st, lv, g.nby, x, y, y2, T(a));
-  return launch_check();
+  return row_pass<D>(lv, RowAxpy<S, T>{x, y, y2, T(a)}, st);
 }
 
 template <typename S, typename T, int D>
@@ -1904,9 +1910,7 @@ amr_status composite_AT(amr_operator* op, const T* x, cudaStream_t st, int only_
   for (int l = 0; l < h->L; ++l) {
     if (only_level >= 0 && l != only_level) continue;
     LevelView lv = level_view(h, l, op->bc);
-    Geo g = geo_of(lv);
-    launch(k_valid_out<T, D>, g.grid, g.block, 0, st, lv, g.nby, x, (const T*)nullptr, S.Z, h->d_valid);
-    TRY(launch_check());
+    TRY((row_pass<D>(lv, RowValidOut<T>{x, (const T*)nullptr, S.Z, h->d_valid, false}, st)));
     TRY(copy_fill<T>(h, l, S.Z, st));
   }
   for (int l = 0; l < h->L; ++l) {
@@ -1957,14 +1961,12 @@ amr_status transpose_residual(amr_operator* op, int l, const T* f, T* out, cudaS
   for (int m = 0; m < h->L; ++m) {
     if (l >= 0 && m != l) continue;
     LevelView lv = level_view(h, m, nullptr);
-    Geo g = geo_of(lv);
     if (l < 0) {
-      launch(k_valid_out<T, D>, g.grid, g.block, 0, st, lv, g.nby, S.W, f, out, h->d_valid);
+      TRY((row_pass<D>(lv, RowValidOut<T>{S.W, f, out, h->d_valid, false}, st)));
     } else {
       // valid cells only: residual, invalid cells untouched
-      launch(k_level_op_masked_copy<T, D>, g.grid, g.block, 0, st, lv, g.nby, S.W, f, out, h->d_valid);
+      TRY((row_pass<D>(lv, RowValidOut<T>{S.W, f, out, h->d_valid, true}, st)));
     }
-    TRY(launch_check());
   }
   return AMR_OK;
 }
@@ -2003,11 +2005,7 @@ amr_status vcycle_corr_T(amr_operator* op, const amr_solver_params& p, const T* 
   CK(cudaMemsetAsync(Xb, 0, bytes, st));
   std::vector<LevelView> lv(h->L);
   for (int l = 0; l <= L; ++l) lv[l] = level_view(h, l, op->bc);
-  for (int l = 0; l <= L; ++l) {
-    Geo g = geo_of(lv[l]);
-    launch(k_axpy_valid<T, D>, g.grid, g.block, 0, st, lv[l], g.nby, r, Xb, T(1), h->d_valid);
-    TRY(launch_check());
-  }
+  for (int l = 0; l <= L; ++l) TRY((row_pass<D>(lv[l], RowAxpyValid<T>{r, Xb, T(1), h->d_valid}, st)));
   CK(cudaMemsetAsync(Eb, 0, bytes, st));
   CK(cudaMemsetAsync(Rb, 0, bytes, st));
   CK(cudaMemsetAsync(rb, 0, bytes, st));
@@ -2057,17 +2055,9 @@ amr_status vcycle_corr_T(amr_operator* op, const amr_solver_params& p, const T* 
   for (int l = 1; l <= L; ++l) {
     const DeviceLists& cl = h->lev[l - 1].dev;
     // D4^T: rb_{l-1} += Rb_{l-1} (valid) ; Xb -= valid part of A^T (Rb_{l-1} on level l-1 valid cells)
-    {
-      Geo g = geo_of(lv[l - 1]);
-      launch(k_axpy_valid<T, D>, g.grid, g.block, 0, st, lv[l - 1], g.nby, Rb, rb, T(1), h->d_valid);
-      TRY(launch_check());
-    }
+    TRY((row_pass<D>(lv[l - 1], RowAxpyValid<T>{Rb, rb, T(1), h->d_valid}, st)));
     TRY((composite_AT<T, D>(op, Rb, st, l - 1)));
-    for (int m = l; m <= L; ++m) {
-      Geo g = geo_of(lv[m]);
-      launch(k_axpy_valid<T, D>, g.grid, g.block, 0, st, lv[m], g.nby, S.W, Xb, T(-1), h->d_valid);
-      TRY(launch_check());
-    }
+    for (int m = l; m <= L; ++m) TRY((row_pass<D>(lv[m], RowAxpyValid<T>{S.W, Xb, T(-1), h->d_valid}, st)));
     // D3^T: tmp_l = Avg^T (Rb_{l-1} on invalid cells) ; Rb_l += tmp_l ; Eb_l -= A_l^T tmp_l
     CK(cudaMemsetAsync(tmp, 0, bytes, st));
     if (cl.nxfer) {
@@ -2086,11 +2076,7 @@ amr_status vcycle_corr_T(amr_operator* op, const amr_solver_params& p, const T* 
     TRY((axpy<T, T, D>(lv[l], S.T1, Rb, (T*)nullptr, 1.0, st)));
   }
   // R_L = r_L: rb_L += Rb_L (valid cells)
-  {
-    Geo g = geo_of(lv[L]);
-    launch(k_axpy_valid<T, D>, g.grid, g.block, 0, st, lv[L], g.nby, Rb, rb, T(1), h->d_valid);
-    TRY(launch_check());
-  }
+  TRY((row_pass<D>(lv[L], RowAxpyValid<T>{Rb, rb, T(1), h->d_valid}, st)));
   CK(cudaMemcpyAsync(S.X, rb, bytes, cudaMemcpyDeviceToDevice, st));
   return AMR_OK;
 }
@@ -2473,9 +2459,7 @@ template <int D>
 amr_status shift_all(amr_hierarchy* h, double* x, const double* d_m, bool valid_only, double sign, cudaStream_t st) {
   for (int l = 0; l < h->L; ++l) {
     LevelView lv = level_view(h, l, nullptr);
-    Geo g = geo_of(lv);
-    launch(k_shift<D>, g.grid, g.block, 0, st, lv, g.nby, x, d_m, valid_only ? h->d_valid : nullptr, sign);
-    TRY(launch_check());
+    TRY((row_pass<D>(lv, RowShift{x, d_m, valid_only ? h->d_valid : nullptr, sign, 0.0}, st)));
   }
   return AMR_OK;
 }
@@ -2523,9 +2507,7 @@ amr_status neumann_fix_T(amr_hierarchy* h, double* x, double* m_host, cudaStream
   TRY(launch_check());
   for (int l = 0; l < h->L; ++l) {
     LevelView lv = level_view(h, l, nullptr);
-    Geo g = geo_of(lv);
-    launch(k_shift<D>, g.grid, g.block, 0, st, lv, g.nby, x, h->d_scalar + 4, h->d_valid, -std::pow(lv.h, D));
-    TRY(launch_check());
+    TRY((row_pass<D>(lv, RowShift{x, h->d_scalar + 4, h->d_valid, -std::pow(lv.h, D), 0.0}, st)));
   }
   if (m_host) {
     CK(cudaMemcpyAsync(h->h_scalar + 4, h->d_scalar + 4, sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -2940,9 +2922,7 @@ amr_status solve_transpose_impl(amr_operator* op, const amr_solver_params& p, do
   // the adjoint unknowns live on valid cells: zero the invalid ones
   for (int l = 0; l < h->L; ++l) {
     LevelView lv = level_view(h, l, nullptr);
-    Geo gg = geo_of(lv);
-    launch(k_valid_out<double, D>, gg.grid, gg.block, 0, st, lv, gg.nby, lam, (const double*)nullptr, lam, h->d_valid);
-    TRY(launch_check());
+    TRY((row_pass<D>(lv, RowValidOut<double>{lam, (const double*)nullptr, lam, h->d_valid, false}, st)));
   }
   loc.vcycles = it;
   loc.final_res = res;
@@ -3079,9 +3059,7 @@ amr_status ghost_fill_T(amr_hierarchy* h, double* W, cudaStream_t st) {
   TRY(avgdown_T_all<D>(h, W, st));
   for (int l = 0; l < h->L; ++l) {
     LevelView lv = level_view(h, l, nullptr);
-    Geo g = geo_of(lv);
-    launch(k_valid_out<double, D>, g.grid, g.block, 0, st, lv, g.nby, W, (const double*)nullptr, W, h->d_valid);
-    TRY(launch_check());
+    TRY((row_pass<D>(lv, RowValidOut<double>{W, (const double*)nullptr, W, h->d_valid, false}, st)));
   }
   return AMR_OK;
 }
