@@ -1329,10 +1329,10 @@ __global__ void k_restrict(LevelView fine, LevelView crs, const XferBlock* __res
   cell_restrict<T, D, RESID, TR>(fine, fine.patches[b.fpatch], crs.patches[b.cpatch], g, xf, ff, outc, alpha, beta);
 }
 
-// 2-D residual restriction, one thread per coarse cell: the four children's residuals
-// f - A x from one plus-shaped load of the fine neighbourhood (32-bit offsets) when the
-// block's children and their two-cell reach lie inside the domain; generic code otherwise.
-// Same summation order as cell_restrict / cell_Lx.
+// 2-D residual restriction, one lane per fine cell: a warp takes 16 columns of two fine rows, each
+// lane the residual of its cell (the sums of edge_op2d next to the faces), and the four children
+// of a coarse cell are added by shuffle in cell_restrict's order.  A thread per coarse cell, its
+// block in generic code wherever it touched a face, took 11 us per FP64 pass at 128^2.
 template <typename T, bool TR>
 __global__ void __launch_bounds__(BX* BY) k_restrict2d_resid(LevelView fine, LevelView crs,
                                                              const XferBlock* __restrict__ blocks,
@@ -1340,57 +1340,46 @@ __global__ void __launch_bounds__(BX* BY) k_restrict2d_resid(LevelView fine, Lev
                                                              T* __restrict__ outc, T alpha, T beta) {
   pdl_wait();
   const XferBlock b = blocks[blockIdx.z];
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * BY + threadIdx.y;
+  const int lane = threadIdx.x;
+  const int f0 = 2 * b.clo[0] + blockIdx.x * 16 + (lane & 15);
+  const int f1 = 2 * (b.clo[1] + (int)(blockIdx.y * BY + threadIdx.y)) + (lane >> 4);
+  const int g0 = f0 >> 1, g1 = f1 >> 1;
+  const bool on = g0 <= b.chi[0] && g1 <= b.chi[1];
   const PatchDesc cp = crs.patches[b.cpatch];
   const PatchDesc fp = fine.patches[b.fpatch];
-  const int g[3] = {b.clo[0] + i, b.clo[1] + j, 0};
-  constexpr int M = TR ? 4 : 2;
-  const int c0 = b.clo[0] + blockIdx.x * BX, c1 = b.clo[1] + blockIdx.y * BY;
-  const bool full = c0 + BX - 1 <= b.chi[0] && c1 + BY - 1 <= b.chi[1];
-  const bool inside = 2 * c0 >= M && 2 * (c0 + BX) - 1 <= fine.ndom[0] - 1 - M && 2 * c1 >= M &&
-                      2 * (c1 + BY) - 1 <= fine.ndom[1] - 1 - M;
-  if (!(full && inside)) {
-    if (g[0] > b.chi[0] || g[1] > b.chi[1]) return;
-    cell_restrict<T, 2, true, TR>(fine, fp, cp, g, xf, ff, outc, alpha, beta);
-    return;
-  }
-  const T inv = pick<T>(fine.inv12h2, fine.inv12h2_f);
-  const T* __restrict__ xb = xf + fp.off;
-  const T* __restrict__ fb = ff + fp.off;
-  const int sy = (int)fp.sy;
-  const int o = (2 * g[1] - fp.lo[1] + NG) * sy + (2 * g[0] - fp.lo[0] + NG);
-  // rows 0 and 1 of the 2x2 block: columns -2..3 ; columns 0 and 1: rows -2, -1, 2, 3
-  T r0[6], r1[6], cu[2][2], cd[2][2];
-#pragma unroll
-  for (int q = 0; q < 6; ++q) {
-    r0[q] = xb[o + q - 2];
-    r1[q] = xb[o + sy + q - 2];
-  }
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    cd[0][q] = xb[o - 2 * sy + q];
-    cd[1][q] = xb[o - sy + q];
-    cu[0][q] = xb[o + 2 * sy + q];
-    cu[1][q] = xb[o + 3 * sy + q];
-  }
-  T acc = T(0);
-#pragma unroll
-  for (int q1 = 0; q1 < 2; ++q1)
-#pragma unroll
-    for (int q0 = 0; q0 < 2; ++q0) {
-      const T* row = q1 == 0 ? r0 : r1;
-      const T xc = row[q0 + 2];
-      const T ym1 = q1 == 0 ? cd[1][q0] : r0[q0 + 2];
-      const T yp1 = q1 == 0 ? r1[q0 + 2] : cu[0][q0];
-      const T ym2 = q1 == 0 ? cd[0][q0] : cd[1][q0];
-      const T yp2 = q1 == 0 ? cu[0][q0] : cu[1][q0];
-      const T s1 = (row[q0 + 1] + row[q0 + 3]) + (ym1 + yp1);
-      const T s2 = (row[q0] + row[q0 + 4]) + (ym2 + yp2);
-      const T lap = (T(16) * s1 - s2 - T(60) * xc) + T(0);
-      acc += fb[o + q1 * sy + q0] - (alpha * xc + beta * (lap * inv));
+  T r = T(0);
+  if (on) {
+    const int sy = (int)fp.sy, i = f0 - fp.lo[0], j = f1 - fp.lo[1], o = (j + NG) * sy + i + NG;
+    const T* __restrict__ xb = xf + fp.off;
+    const T xc = xb[o], fk = ff[fp.off + o];
+    T x1, x2, y1, y2, ex = T(0);
+    if (TR) {
+      if (f0 >= 4 && f0 <= fine.ndom[0] - 5) {
+        x1 = xb[o - 1] + xb[o + 1];
+        x2 = xb[o - 2] + xb[o + 2];
+      } else {
+        trans_sums<T>(xb, o, 1, i, fine.ndom[0], fp.lo[0], fp.n[0], fine.bc[0], fine.bc[1], x1, x2, ex);
+      }
+      if (f1 >= 4 && f1 <= fine.ndom[1] - 5) {
+        y1 = xb[o - sy] + xb[o + sy];
+        y2 = xb[o - 2 * sy] + xb[o + 2 * sy];
+      } else {
+        trans_sums<T>(xb, o, sy, j, fine.ndom[1], fp.lo[1], fp.n[1], fine.bc[2], fine.bc[3], y1, y2, ex);
+      }
+    } else {
+      line_sums<T>(xb, o, 1, face_class(f0, fine.ndom[0]) == 0, f0, fine.ndom[0], fine.bc[0], fine.bc[1], x1, x2);
+      line_sums<T>(xb, o, sy, face_class(f1, fine.ndom[1]) == 0, f1, fine.ndom[1], fine.bc[2], fine.bc[3], y1, y2);
     }
-  outc[poff(cp, g[0] - cp.lo[0], g[1] - cp.lo[1], 0)] = acc * T(0.25);
+    const T s1 = x1 + y1, s2 = x2 + y2;
+    const T inv = pick<T>(fine.inv12h2, fine.inv12h2_f);
+    r = fk - (alpha * xc + beta * (((T(16) * s1 - s2 - T(60) * xc) + ex) * inv));
+  }
+  const int q = lane & 14;
+  T acc = __shfl_sync(0xffffffffu, r, q);
+  acc += __shfl_sync(0xffffffffu, r, q + 1);
+  acc += __shfl_sync(0xffffffffu, r, q + 16);
+  acc += __shfl_sync(0xffffffffu, r, q + 17);
+  if (on && lane == q) outc[poff(cp, g0 - cp.lo[0], g1 - cp.lo[1], 0)] = acc * T(0.25);
 }
 
 // Fine cell gf += cell-centred tensor linear interpolation of the coarse correction
@@ -1446,55 +1435,38 @@ __global__ void k_prolong(LevelView fine, LevelView crs, const XferBlock* __rest
   cell_prolong<T, D>(crs, fine.patches[b.fpatch], crs.patches[b.cpatch], gf, xc, xf, xf2);
 }
 
-// 2-D prolongation, one thread per coarse cell: its four children += linear interpolation
-// from the 3x3 coarse neighbourhood (32-bit offsets) when the neighbourhood lies inside the
-// domain and the patch; generic per-fine-cell code otherwise (same arithmetic).
+// 2-D prolongation, one thread per fine cell: linear interpolation from its four coarse corners
+// (32-bit offsets) when they lie inside the domain and the patch, generic code otherwise (same
+// arithmetic).  The grids are small, so the pass lasts as long as one thread next to a face: with
+// a thread per coarse cell, four generic children in turn, an FP64 pass took 14 us at 128^2.
 template <typename T>
 __global__ void __launch_bounds__(BX* BY) k_prolong2d(LevelView fine, LevelView crs, const XferBlock* __restrict__ blocks,
                                                       const T* __restrict__ xc, T* __restrict__ xf, T* __restrict__ xf2) {
   pdl_wait();
   const XferBlock b = blocks[blockIdx.z];
-  const int i = blockIdx.x * BX + threadIdx.x;
-  const int j = blockIdx.y * BY + threadIdx.y;
-  const int g0 = b.clo[0] + i, g1 = b.clo[1] + j;
+  const int f0 = 2 * b.clo[0] + blockIdx.x * BX + threadIdx.x, f1 = 2 * b.clo[1] + blockIdx.y * BY + threadIdx.y;
+  const int g0 = f0 >> 1, g1 = f1 >> 1;
   if (g0 > b.chi[0] || g1 > b.chi[1]) return;
   const PatchDesc cp = crs.patches[b.cpatch];
   const PatchDesc fp = fine.patches[b.fpatch];
-  const bool inside = g0 - 1 >= cp.lo[0] && g0 + 1 <= cp.lo[0] + cp.n[0] - 1 && g1 - 1 >= cp.lo[1] &&
-                      g1 + 1 <= cp.lo[1] + cp.n[1] - 1;
-  if (!inside) {
-    for (int q1 = 0; q1 < 2; ++q1)
-      for (int q0 = 0; q0 < 2; ++q0) {
-        const int gf[3] = {2 * g0 + q0, 2 * g1 + q1, 0};
-        cell_prolong<T, 2>(crs, fp, cp, gf, xc, xf, xf2);
-      }
+  const int s0 = (f0 & 1) ? 1 : -1, s1 = (f1 & 1) ? 1 : -1;
+  const int e0 = g0 + s0 - cp.lo[0], e1 = g1 + s1 - cp.lo[1];
+  if (e0 < 0 || e0 >= cp.n[0] || e1 < 0 || e1 >= cp.n[1]) {
+    const int gf[3] = {f0, f1, 0};
+    cell_prolong<T, 2>(crs, fp, cp, gf, xc, xf, xf2);
     return;
   }
-  const T* __restrict__ cb = xc + cp.off;
   const int csy = (int)cp.sy;
-  const int oc = (g1 - cp.lo[1] + NG) * csy + (g0 - cp.lo[0] + NG);
-  T c[3][3];
-#pragma unroll
-  for (int a1 = 0; a1 < 3; ++a1)
-#pragma unroll
-    for (int a0 = 0; a0 < 3; ++a0) c[a1][a0] = cb[oc + (a1 - 1) * csy + (a0 - 1)];
-  const int fsy = (int)fp.sy;
-  const long long of = fp.off + (long long)((2 * g1 - fp.lo[1] + NG) * fsy + (2 * g0 - fp.lo[0] + NG));
-#pragma unroll
-  for (int q1 = 0; q1 < 2; ++q1)
-#pragma unroll
-    for (int q0 = 0; q0 < 2; ++q0) {
-      const int s0 = q0 == 0 ? -1 : 1, s1 = q1 == 0 ? -1 : 1;
-      // corners in the generic order: (q0, q1) = (0,0), (1,0), (0,1), (1,1) over the parent
-      T v = T(0);
-      v += (T(0.75) * T(0.75)) * c[1][1];
-      v += (T(0.25) * T(0.75)) * c[1][1 + s0];
-      v += (T(0.75) * T(0.25)) * c[1 + s1][1];
-      v += (T(0.25) * T(0.25)) * c[1 + s1][1 + s0];
-      const long long o = of + q1 * fsy + q0;
-      xf[o] += v;
-      if (xf2 != nullptr) xf2[o] += v;
-    }
+  const T* __restrict__ c = xc + cp.off + (g1 - cp.lo[1] + NG) * csy + (g0 - cp.lo[0] + NG);
+  // corners in the generic order: (q0, q1) = (0,0), (1,0), (0,1), (1,1) over the parent
+  T v = T(0);
+  v += (T(0.75) * T(0.75)) * c[0];
+  v += (T(0.25) * T(0.75)) * c[s0];
+  v += (T(0.75) * T(0.25)) * c[s1 * csy];
+  v += (T(0.25) * T(0.25)) * c[s1 * csy + s0];
+  const long long o = fp.off + (long long)((f1 - fp.lo[1] + NG) * (int)fp.sy + (f0 - fp.lo[0] + NG));
+  xf[o] += v;
+  if (xf2 != nullptr) xf2[o] += v;
 }
 
 // ------------------------------------------------------------------------ temporally blocked 2-D smoothing

@@ -817,7 +817,7 @@ amr_status restrict_blocks(const LevelView& fine, const LevelView& crs, const Xf
   cudaEvent_t ev;
   prof_begin(st, &ev);
   if (resid && D == 2)
-    launch(k_restrict2d_resid<T, TR>, grid, block, 0, st, fine, crs, blocks, xf, ff, outc, T(alpha), T(beta));
+    launch(k_restrict2d_resid<T, TR>, dim3((2 * xmax[0] + 15) / 16, (xmax[1] + BY - 1) / BY, nblocks), block, 0, st, fine, crs, blocks, xf, ff, outc, T(alpha), T(beta));
   else if (D == 3 && resid && !TR && small_offsets(fine)) {
     const long long groups = (long long)((xmax[0] + 3) / 4) * xmax[1] * xmax[2];  // warps of four coarse cells
     launch(k_restrict3d_resid<T>, dim3((unsigned)((groups + 7) / 8), 1, nblocks), 256, 0, st, fine, crs, blocks, xf, ff,
@@ -838,7 +838,7 @@ amr_status prolong_blocks(const LevelView& fine, const LevelView& crs, const Xfe
   cudaEvent_t ev;
   prof_begin(st, &ev);
   if (D == 2) {
-    dim3 grid((xmax[0] + BX - 1) / BX, (xmax[1] + BY - 1) / BY, nblocks);
+    dim3 grid((2 * xmax[0] + BX - 1) / BX, (2 * xmax[1] + BY - 1) / BY, nblocks);
     launch(k_prolong2d<T>, grid, dim3(BX, BY, 1), 0, st, fine, crs, blocks, xc, xf, xf2);
   } else {
     // a 3-D patch beyond 2^31 elements takes the generic kernel
