@@ -3141,7 +3141,7 @@ __global__ void k_sub(LevelView lv, int nby, const double* __restrict__ w, const
 //                   for non-negative doubles, a NaN wins) and, when rin is given, r rounded to
 //                   FP32 over the whole array (the next FP32 V-cycle's right-hand side; ghost
 //                   entries are never read);
-//   k_update_valid  phi += X on the valid cells (invalid cells are recomputed by the
+//   k_update_valid  phi += X (x2 given: X + X2) on the valid cells (invalid cells are recomputed by the
 //                   average-down that starts the next composite residual), and clears the
 //                   norm accumulator for that residual.
 //   V elements per thread and step: 4 (16-byte loads of FP64 pairs, 4-byte masks; arrays
@@ -3235,7 +3235,8 @@ __global__ void __launch_bounds__(256) k_norm_convert(long long n, const double*
 }
 
 template <typename S, int V>
-__global__ void __launch_bounds__(256) k_update_valid(long long n, const S* __restrict__ x, double* __restrict__ phi,
+__global__ void __launch_bounds__(256) k_update_valid(long long n, const S* __restrict__ x, const S* __restrict__ x2,
+                                                      double* __restrict__ phi,
                                                       const unsigned char* __restrict__ vmask,
                                                       unsigned long long* __restrict__ acc_clear,
                                                       const int* __restrict__ active) {
@@ -3251,6 +3252,12 @@ __global__ void __launch_bounds__(256) k_update_valid(long long n, const S* __re
     FlatVec<V>::ld(vmask + e, m);
     FlatVec<V>::ld(x + e, c);
     FlatVec<V>::ld(phi + e, y);
+    if (x2 != nullptr) {
+      S d[V];
+      FlatVec<V>::ld(x2 + e, d);
+#pragma unroll
+      for (int q = 0; q < V; ++q) c[q] += d[q];
+    }
     unsigned any = 0, all = 1;
 #pragma unroll
     for (int q = 0; q < V; ++q) {

@@ -2361,16 +2361,16 @@ inline amr_status norm_flat(const amr_hierarchy* h, long long n, int nc, const d
   return launch_check();
 }
 
-// phi += x on the valid cells
+// phi += x (x2 given: x + x2, added in S) on the valid cells
 template <typename S>
-amr_status update_flat(const amr_hierarchy* h, const S* x, double* phi, unsigned long long* acc_clear, const int* active,
+amr_status update_flat(const amr_hierarchy* h, const S* x, const S* x2, double* phi, unsigned long long* acc_clear, const int* active,
                        cudaStream_t st) {
   const long long n = rep_elems(h);
   const unsigned char* m = h->d_valid;
-  if (flat_vec(n, x, phi))
-    launch(k_update_valid<S, 4>, dim3(flat_blocks(n / 4), h->ncomp, 1), 256, 0, st, n, x, phi, m, acc_clear, active);
+  if (flat_vec(n, x, phi) && flat_vec(n, x2))
+    launch(k_update_valid<S, 4>, dim3(flat_blocks(n / 4), h->ncomp, 1), 256, 0, st, n, x, x2, phi, m, acc_clear, active);
   else
-    launch(k_update_valid<S, 1>, dim3(flat_blocks(n), h->ncomp, 1), 256, 0, st, n, x, phi, m, acc_clear, active);
+    launch(k_update_valid<S, 1>, dim3(flat_blocks(n), h->ncomp, 1), 256, 0, st, n, x, x2, phi, m, acc_clear, active);
   return launch_check();
 }
 
@@ -2585,7 +2585,11 @@ amr_status ensure_inner(amr_operator* op) {
 // one composite V-cycle, then (cycles_per_refinement > 1) further cycles on the FP32
 // composite residual rin - A X of the correction so far (homogeneous boundary data), each
 // added to it.  The correction so far moves to inner_x and the next cycle writes the other
-// buffer, so no copy is made.
+// buffer, so no copy is made.  The last cycle's result is left in X beside inner_x: the update
+// of phi adds the two (inner_sum) in one pass instead of two.
+inline const float* inner_sum(const amr_operator* op, const amr_solver_params& p) {
+  return cpr_of(p) > 1 ? op->inner_x : nullptr;
+}
 template <int D>
 amr_status mixed_correction(amr_operator* op, const amr_solver_params& p, cudaStream_t st) {
   Scratch<float>& S = op->s32;
@@ -2600,7 +2604,7 @@ amr_status mixed_correction(amr_operator* op, const amr_solver_params& p, cudaSt
     std::swap(S.X, op->inner_x);
     TRY(composite_op<D>(op, OP_RESID, op->inner_x, (const float*)S.rin, op->inner_r, (const float*)nullptr, st));
     TRY((vcycle_corr<float, D>(op, p, op->inner_r, st, VC_SCRATCH_R)));
-    for (int l = 0; l < h->L; ++l)
+    for (int l = 0; l < h->L && c + 1 < cpr_of(p); ++l)
       TRY((axpy<float, float, D>(level_view(h, l, nullptr), op->inner_x, S.X, (float*)nullptr, 1.0, st)));
   }
   return AMR_OK;
@@ -2648,10 +2652,10 @@ amr_status solve_impl(amr_operator* op, const amr_solver_params& p, double* phi,
     }
     if (p.precision == AMR_MIXED) {
       TRY(mixed_correction<D>(op, p, st));
-      TRY(update_flat<float>(h, op->s32.X, phi, nullptr, nullptr, st));
+      TRY(update_flat<float>(h, op->s32.X, inner_sum(op, p), phi, nullptr, nullptr, st));
     } else {
       TRY(vcycle_corr<double, D>(op, p, op->Res, st, VC_SCRATCH_R));
-      TRY(update_flat<double>(h, op->s64.X, phi, nullptr, nullptr, st));
+      TRY(update_flat<double>(h, op->s64.X, (const double*)nullptr, phi, nullptr, nullptr, st));
     }
   }
   loc.vcycles = it * (p.precision == AMR_MIXED ? cpr_of(p) : 1);
@@ -2687,10 +2691,10 @@ amr_status iteration_body(amr_operator* op, int prec, const amr_solver_params& p
   const int* active = h->ncomp > 1 ? op->d_active : nullptr;  // converged replicas keep their phi
   if (prec == AMR_MIXED) {
     TRY(mixed_correction<D>(op, p, st));
-    TRY(update_flat<float>(h, op->s32.X, phi, rbits, active, st));
+    TRY(update_flat<float>(h, op->s32.X, inner_sum(op, p), phi, rbits, active, st));
   } else {
     TRY(vcycle_corr<double, D>(op, p, op->Res, st, VC_SCRATCH_R));
-    TRY(update_flat<double>(h, op->s64.X, phi, rbits, active, st));
+    TRY(update_flat<double>(h, op->s64.X, (const double*)nullptr, phi, rbits, active, st));
   }
   TRY(composite_op<D>(op, OP_RESID, phi, op->F, op->Res, bc, st));
   return norm_convert(op, prec, rbits, st);
@@ -2912,10 +2916,10 @@ amr_status solve_transpose_impl(amr_operator* op, const amr_solver_params& p, do
     if (it >= p.max_vcycles) { set_error("max_vcycles reached"); break; }
     if (p.precision == AMR_MIXED) {
       TRY((vcycle_corr_T<float, D>(op, p, op->s32.rin, st)));
-      TRY(update_flat<float>(h, op->s32.X, lam, nullptr, nullptr, st));
+      TRY(update_flat<float>(h, op->s32.X, (const float*)nullptr, lam, nullptr, nullptr, st));
     } else {
       TRY((vcycle_corr_T<double, D>(op, p, op->Res, st)));
-      TRY(update_flat<double>(h, op->s64.X, lam, nullptr, nullptr, st));
+      TRY(update_flat<double>(h, op->s64.X, (const double*)nullptr, lam, nullptr, nullptr, st));
     }
   }
   if (op->neumann) TRY(neumann_fix_T<D>(h, lam, nullptr, st));
