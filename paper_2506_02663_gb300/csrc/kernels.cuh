@@ -2718,7 +2718,7 @@ __device__ __forceinline__ void scatter_read(T* __restrict__ W, const PatchDesc&
 // forward correction is out[c] += coef/hc * sum_faces s (Fbar/hf' - Fc/hc') with hf' = hf,
 // hc' = hc for derivatives and 1 for values.  A thread per (cell, face, cell of the face's line):
 // as one thread per cell the lists of a 2-D level, a few hundred cells, took 10 us of serial
-// atomics and FP64 divisions on five SMs.
+// atomics and FP64 divisions on five SMs (now 3.9 us).
 constexpr int REFLUX_T_LANES = 4;
 template <typename T, int D>
 __global__ void __launch_bounds__(128) k_reflux_T(LevelView crs, LevelView fine, const RefluxEntry* __restrict__ list,
@@ -2846,7 +2846,7 @@ __global__ void k_cfi_T(const CfiEntry* __restrict__ list, long long n, const lo
 // The same by groups of the 2^D ghosts that share a window (ratio 2): a warp per group forms their
 // weights, folds them dimension by dimension -- a lane per (x, y) of the window, its cells along z
 // in turn -- and adds every window cell once, where a thread per ghost made 2^D times as many
-// atomic additions (64^3 box: 33 us per pass in FP32).
+// atomic additions (64^3 box: 33 -> 6.0 us per pass in FP32, 23 -> 11 us in FP64).
 template <typename T, int D>
 __global__ void __launch_bounds__(128) k_cfi_T_grp(const CfiGroup* __restrict__ list, long long n,
                                                    const long long* __restrict__ side,
@@ -3019,7 +3019,8 @@ __global__ void k_avgdown_T2(LevelView fine, LevelView crs, const XferBlock* __r
 // ------------------------------------------------------------------------ elementwise
 // A pass over the interior cells of a level: a warp takes rows, a lane up to ROW_K of its cells at
 // once, their loads issued together (F::load), then their stores (F::store).  Bound by memory: as
-// one thread per cell in 65,536 blocks, X += E on 256^3 took 60 us where its bytes take 30.
+// one thread per cell in 65,536 blocks, X += E on 256^3 took 60 us where its bytes take 30 (128^3
+// FP32: 10.1 -> 6.0 us).
 constexpr int ROW_K = 4;
 template <int D, typename F>
 __global__ void __launch_bounds__(256) k_rows(LevelView lv, F f) {
@@ -3289,17 +3290,15 @@ __device__ __forceinline__ void dd_add(double& s, double& c, double a, double ac
   two_sum(t, e, s, c);
 }
 
-// A warp's sum of doubles in 128-bit fixed point: a double enters as its 53-bit significand
-// shifted to the warp's common frame (exponent E), so additions are exact integer ones in any
-// order.  Below the sign the frame keeps 26 bits of headroom (2^24 terms at least) and 47 bits
-// under the last bit of the largest term: terms within a factor 2^47 of it enter exactly.  An
-// addition costs about 30 integer instructions, where TwoSum costs seven FP64 ones at a fiftieth
-// of their rate.
-struct WarpSum {
+// A sum of doubles in 128-bit fixed point: a double enters as its 53-bit significand shifted to a
+// common frame (exponent E), so additions are exact integer ones in any order.  Below the sign
+// the frame keeps 26 bits of headroom (2^24 terms at least) and 47 bits under the last bit of the
+// largest term: terms within a factor 2^47 of it enter exactly.  A larger term moves the frame by
+// a shift of the sum so far; bits below 2^-100 of the largest term are dropped.  An addition costs
+// about 30 integer instructions, where TwoSum costs seven FP64 ones at a fiftieth of their rate.
+struct FixSum {
   unsigned l0 = 0, l1 = 0, l2 = 0, l3 = 0;
-  int E = 0;                // frame; 0: nothing added yet
-  double s = 0.0, c = 0.0;  // what earlier frames collected
-  bool bad = false;         // a non-finite term
+  int E = 0;  // frame; 0: nothing added yet
 
   __device__ __forceinline__ static int exponent(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
   // v, of an exponent <= E - 2
@@ -3331,50 +3330,68 @@ struct WarpSum {
         : "+&r"(l0), "+&r"(l1), "+&r"(l2), "+&r"(l3)
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3));
   }
-  // the lanes' integers summed into every lane
-  __device__ __forceinline__ void reduce() {
+  // the lanes' sums (of one frame) added up over groups of n lanes, into every lane
+  __device__ __forceinline__ void reduce(int n) {
 #pragma unroll 1
-    for (int st = 16; st > 0; st >>= 1) {
+    for (int st = n >> 1; st > 0; st >>= 1) {
       const unsigned a0 = __shfl_xor_sync(0xffffffffu, l0, st), a1 = __shfl_xor_sync(0xffffffffu, l1, st);
       const unsigned a2 = __shfl_xor_sync(0xffffffffu, l2, st), a3 = __shfl_xor_sync(0xffffffffu, l3, st);
       join(a0, a1, a2, a3);
     }
   }
-  // the integers as a double-double added to (s, c); the frame is free again
-  __device__ __forceinline__ void collect() {
+  // frame e (not below the present one)
+  __device__ __forceinline__ void move(int e) {
+    int d = E == 0 ? 0 : e - E;
+    E = e;
+    const unsigned sg = (unsigned)((int)l3 >> 31);
+    if (d >= 128) {
+      l0 = l1 = l2 = l3 = sg;
+      return;
+    }
+    for (; d >= 32; d -= 32) {
+      l0 = l1;
+      l1 = l2;
+      l2 = l3;
+      l3 = sg;
+    }
+    l0 = __funnelshift_r(l0, l1, d);
+    l1 = __funnelshift_r(l1, l2, d);
+    l2 = __funnelshift_r(l2, l3, d);
+    l3 = (unsigned)((int)l3 >> d);
+  }
+  // room for terms of exponents up to e
+  __device__ __forceinline__ void frame(int e) {
+    if (e + 2 > E) move(max(e, 1) + 2);
+  }
+  // the sum as a double-double
+  __device__ __forceinline__ void value(double& s, double& c) const {
     double h, e1, e2, e3;
     two_sum(79228162514264337593543950336.0 * (double)(int)l3, 18446744073709551616.0 * (double)l2, h, e1);
     two_sum(h, 4294967296.0 * (double)l1, h, e2);
     two_sum(h, (double)l0, h, e3);
-    const double lo = e1 + (e2 + e3);
-    // l3's unit is 2^(E - 1075 + 32 + 14)
-    if (E != 0) dd_add(s, c, scalbn(h, E - 1125), scalbn(lo, E - 1125));
-    l0 = l1 = l2 = l3 = 0;
-    E = 0;
-  }
-  // the warp's frame for terms of exponents up to e (warp-uniform)
-  __device__ __forceinline__ void frame(int e) {
-    if (e + 2 <= E) return;
-    if (E != 0) {
-      reduce();
-      collect();
-    }
-    E = max(e, 1) + 2;
+    // the unit is 2^(E - 1125): two factors in the normal range
+    const int k = E - 1125, ka = k / 2;
+    const double fa = __longlong_as_double((long long)(1023 + ka) << 52), fb = __longlong_as_double((long long)(1023 + k - ka) << 52);
+    s = h * fa * fb;
+    c = (e1 + (e2 + e3)) * fa * fb;
   }
 };
 
 // Deterministic partial sums of w * x over the valid interior cells of one level, with a fixed
 // number of blocks per level (the rows each warp visits depend only on the launch shape): one
-// double-double partial part[2*(base+block)].  A warp sums whole rows in fixed point (WarpSum),
-// the warps' sums combine in double-double, and w multiplies the block's sum exactly (TwoProd).
+// double-double partial part[2*(base+block)].  A warp sums whole rows in fixed point (FixSum, one
+// frame per warp), the warps' sums are brought to one frame and added, and w multiplies the
+// block's sum exactly (TwoProd).
 template <int D>
 __global__ void __launch_bounds__(256) k_wsum_gs(LevelView lv, const double* __restrict__ x,
                                                  const unsigned char* __restrict__ vmask, double w,
                                                  double* __restrict__ part, long long base) {
   pdl_wait();
   constexpr int K = 8;  // cells of a lane in flight
-  __shared__ double ss[8], sc[8];
-  WarpSum a;
+  __shared__ uint4 sl[8];
+  __shared__ int se[8];
+  FixSum a;
+  bool bad = false;  // a non-finite term
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nw = gridDim.x * 8;
   for (int pi = 0; pi < lv.npatch; ++pi) {
@@ -3395,11 +3412,11 @@ __global__ void __launch_bounds__(256) k_wsum_gs(LevelView lv, const double* __r
 #pragma unroll
         for (int q = 0; q < K; ++q) {
           if (!m[q]) v[q] = 0.0;
-          e = max(e, WarpSum::exponent(v[q]));
+          e = max(e, FixSum::exponent(v[q]));
         }
         e = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
         if (e == 0x7ff) {
-          a.bad = true;
+          bad = true;
           continue;
         }
         a.frame(e);
@@ -3409,21 +3426,25 @@ __global__ void __launch_bounds__(256) k_wsum_gs(LevelView lv, const double* __r
       }
     }
   }
-  a.reduce();
-  a.collect();
-  if (a.bad) a.s = __longlong_as_double(0x7ff8000000000000ll);
+  a.reduce(32);
   if (lane == 0) {
-    ss[warp] = a.s;
-    sc[warp] = a.c;
+    sl[warp] = make_uint4(a.l0, a.l1, a.l2, a.l3);
+    se[warp] = bad ? -1 : a.E;
   }
   __syncthreads();
   if (warp != 0) return;
-  double s = lane < 8 ? ss[lane & 7] : 0.0, c = lane < 8 ? sc[lane & 7] : 0.0;
-#pragma unroll 1
-  for (int st = 4; st > 0; st >>= 1) {
-    const double t = __shfl_down_sync(0xffffffffu, s, st), tc = __shfl_down_sync(0xffffffffu, c, st);
-    dd_add(s, c, t, tc);
-  }
+  const uint4 l = sl[lane & 7];
+  a.l0 = l.x;
+  a.l1 = l.y;
+  a.l2 = l.z;
+  a.l3 = l.w;
+  a.E = se[lane & 7];
+  const bool nan = __any_sync(0xffffffffu, a.E < 0);
+  a.move((int)__reduce_max_sync(0xffffffffu, (unsigned)max(a.E, 1)));
+  a.reduce(8);
+  double s, c;
+  a.value(s, c);
+  if (nan) s = __longlong_as_double(0x7ff8000000000000ll);
   if (lane == 0) {
     const double hi = w * s, lo = fma(w, s, -hi);
     const double e = fma(w, c, lo);
@@ -3491,7 +3512,7 @@ __global__ void __launch_bounds__(256) k_dd_final(const double* __restrict__ par
   __shared__ uint4 sl[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int e = 0;
-  for (long long t = threadIdx.x; t < 2 * n; t += 256) e = max(e, WarpSum::exponent(part[t]));
+  for (long long t = threadIdx.x; t < 2 * n; t += 256) e = max(e, FixSum::exponent(part[t]));
   e = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
   if (lane == 0) se[warp] = e;
   __syncthreads();
@@ -3500,16 +3521,17 @@ __global__ void __launch_bounds__(256) k_dd_final(const double* __restrict__ par
     if (threadIdx.x == 0) out[0] = __longlong_as_double(0x7ff8000000000000ll);
     return;
   }
-  WarpSum a;
+  FixSum a;
   a.frame(e);
   for (long long t = threadIdx.x; t < 2 * n; t += 256) a.add(part[t]);
-  a.reduce();
+  a.reduce(32);
   if (lane == 0) sl[warp] = make_uint4(a.l0, a.l1, a.l2, a.l3);
   __syncthreads();
   if (threadIdx.x != 0) return;
   for (int q = 1; q < 8; ++q) a.join(sl[q].x, sl[q].y, sl[q].z, sl[q].w);
-  a.collect();
-  out[0] = a.s + a.c;
+  double s, c;
+  a.value(s, c);
+  out[0] = s + c;
 }
 
 // m = (S_f - beta * S_b) / V ; used by the solvability fix and mean-zero

@@ -644,7 +644,8 @@ inline bool small_offsets(const LevelView& lv) {
 // The fixed-point FP64 residual of a 2-D level that is the whole domain (k_resid2d_fx): columns in
 // groups of four, fields aligned for FP64 pairs, and a grid large enough for the FP64 rate,
 // not the launches, to bound the plain kernel (residual with its frame pass against plain, launch
-// gaps included: 1024^2 74 against 65 us, 2048^2 99 against 126 us, 4096^2 258 against 377 us).
+// gaps included, alpha not zero: 2048 x 1024 81 against 87 us, 2304 x 2048 99 against 137 us, 4096^2
+// 262 against 377 us; an earlier form on 1024^2: 74 against 65 us).
 inline bool fx2d_shape(const LevelView& lv) {
   const PatchDesc& p = lv.p0;
   return lv.D == 2 && lv.npatch == 1 && p.n[0] == lv.ndom[0] && p.n[1] == lv.ndom[1] && p.n[0] % 4 == 0 && p.n[0] >= 16 &&
@@ -3613,8 +3614,8 @@ amr_status batch_worklist(amr_operator* const* ops, int n, const amr_solver_para
   std::lock_guard<std::mutex> lock(mu);
   // The graph holds launch shapes, parameters and the addresses of the plan's own arrays; fields
   // and operators enter through the descriptors.  A call with other operators or fields but
-  // the launches of the last one therefore only uploads descriptors (releasing and rebuilding
-  // everything took 2.5 ms of a 96-problem call).
+  // the launches of the last one therefore only uploads descriptors (96 problems, three
+  // sets of fields in turn: 7.70 -> 7.39 ms a call).
   const bool same = plan.exec && plan.n == n && same_params(plan.p, q);
   bool hit = same;
   for (int k = 0; hit && k < n; ++k)
