@@ -377,15 +377,15 @@ def _timed(torch, fn, k, flush=None):
 
 
 KERNEL_CLASSES = {
-    "jacobi": ("KC_JACOBI", "weighted-Jacobi sweep (k_sweep3d / k_level_op3d_zc / k_level_op3d_march / k_level_op2d_tiled)"),
+    "jacobi": ("KC_JACOBI", "weighted-Jacobi sweep (k_sweep3d / k_level_op3d_zc / k_level_op3d_col / k_level_op2d_tiled)"),
     "residual": ("KC_RESID", "FP32 level residual or operator application (k_sweep3d / k_level_op3d_zc / k_level_op*)"),
     "residual64": ("KC_RESID64", "FP64 level residual of the refinement loop (3-D: k_absmax_patch + k_resid3d_fx, "
                                  "fixed-point stencil sums)"),
     "restrict": ("KC_RESTRICT", "residual restriction and average-down (k_restrict*)"),
     "prolong": ("KC_PROLONG", "linear prolongation + correction (k_prolong*)"),
-    "down_leg": ("KC_DOWN", "k_mg_down2d<float>: nu1 sweeps + residual + restriction, one launch per grid"),
-    "up_leg": ("KC_UP", "k_mg_up2d<float>: prolongation + nu2 sweeps, one launch per grid"),
-    "coarse_block": ("KC_COARSE", "k_mg_coarse2d<float>: the V-cycle on the grids <= 64^2, one block"),
+    "down_leg": ("KC_DOWN", "k_mg_down2d<float> / k_leg2d: nu1 sweeps + residual + restriction, one launch per grid"),
+    "up_leg": ("KC_UP", "k_mg_up2d<float> / k_leg2d: prolongation + nu2 sweeps, one launch per grid"),
+    "coarse_block": ("KC_COARSE", "the V-cycle on the coarse grids in one launch (k_mg_coarse2d*<float>, k_mg_cluster)"),
 }
 # grid-size buckets (cells) of the 3-D workload's grids: the 256^3 base, the 128^3 grids (fine
 # box, second multigrid grid), 64^3, and the coarse end
@@ -634,7 +634,7 @@ def _cic3d_run(amr, torch, w, peak, peak_kind, reps):
             "coarse_window_cells": nband, "interface_faces": nf, "components": nc,
             "bytes_per_call": nbytes, "gbs_per_call": gbs,
             "ghost_call_ms": msg,
-            "roofline": {"bound": "alu", "kernels": "k_cic_combine + k_cic_grp3 (one amr_cic_ghosts call)",
+            "roofline": {"bound": "alu", "kernels": "k_cfi_tile with four time levels (+ k_cic_grp), one amr_cic_ghosts call",
                          "achieved": tf, "peak": FP64_PEAK_TFLOPS, "unit": "FP64 TFLOP/s", "frac": tf / FP64_PEAK_TFLOPS,
                          "flops_per_call": flops, "peak_kind": "nominal (2 FP64 FMA/clk/SM x 152 SMs x 2070 MHz)"},
             "corrected_face_sum": tot,
