@@ -159,23 +159,23 @@ __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.p
 // cell_restrict, times 1/8, into the coarse grid's right-hand side.
 constexpr int OP_RESTRICT = 4;
 
-// FP32 sweeps and residuals keep their z neighbours in registers (zqueue_march).
+// FP32 sweeps keep their z neighbours in registers (zqueue_march).  Not the residual: with its mask
+// and without the factors it spilled, 63 us on 256^3 in a solve against 55 from the ring.
 template <typename T, int MODE>
 __host__ __device__ constexpr bool sw3_zqueue() {
-  return sizeof(T) == 4 && (MODE == OP_JACOBI || MODE == OP_RESID);
+  return sizeof(T) == 4 && MODE == OP_JACOBI;
 }
 
-// The consumer loop of the FP32 sweep and residual: a thread's four rows (RW) of planes k-2 ..
+// The consumer loop of the FP32 sweep: a thread's four rows (RW) of planes k-2 ..
 // k+1 sit in registers, so a step reads from the ring only the new plane's own cells, the x
 // neighbours and the four rows around the thread's own -- 16 shared loads for eight cells
 // instead of 44 -- and a plane's slot is free once its own step is done, two planes earlier.
-// One sweep of 256^3: 44.5 -> 42.8 us (bound by the plane traffic, 1.33 halo included); of 128^3,
-// where few planes are in flight: 12.0 -> 8.6 us.
+// One sweep repeated by itself: 256^3 44.5 -> 42.8 us (bound by the plane traffic, 1.33 halo
+// included); 128^3, where few planes are in flight, 12.0 -> 8.6 us.
 // Same sums in the same order as the loop that reads every neighbour from the ring.
-template <typename T, int MODE, int RW, int S, int SLOT>
+template <typename T, int RW, int S, int SLOT>
 __device__ __forceinline__ void zqueue_march(T* ring, unsigned long long* gbar, unsigned long long* empty, int rbase,
-                                             const T* __restrict__ f, T* __restrict__ orow,
-                                             const unsigned char* __restrict__ vrow, const PatchDesc& p, int ka, int kb,
+                                             const T* __restrict__ f, T* __restrict__ orow, const PatchDesc& p, int ka, int kb,
                                              int lz, int nzd, int row, int col, const T* wt, const int (&wxy)[RW][2],
                                              T kc0, T kc1, T kc2, int lane, unsigned* err) {
   using namespace sw3;
@@ -193,12 +193,10 @@ __device__ __forceinline__ void zqueue_march(T* ring, unsigned long long* gbar, 
   }
   const T* __restrict__ frow = f + p.off + (long long)(ka + NG) * p.sz + (long long)(row + NG) * p.sy + col;
   V fq[2][RW];
-  uchar2 mq[RW];
 #pragma unroll
   for (int r = 0; r < RW; ++r) {
     fq[0][r] = __ldg(reinterpret_cast<const V*>(frow + r * sy));
     fq[1][r] = ka + 1 < kb ? __ldg(reinterpret_cast<const V*>(frow + sz + r * sy)) : V{T(0), T(0)};
-    mq[r] = (MODE == OP_RESID && vrow != nullptr) ? *reinterpret_cast<const uchar2*>(vrow + r * sy) : make_uchar2(1, 1);
   }
   int s2 = 2, s4 = 4, par4 = 0;  // slots of planes k and k+2, phase of the latter
   auto step = [&](int k, auto slotc) -> bool {
@@ -228,23 +226,7 @@ __device__ __forceinline__ void zqueue_march(T* ring, unsigned long long* gbar, 
       if (k + 2 < kb) fq[FS][r] = __ldg(reinterpret_cast<const V*>(frow + 2 * sz + r * sy));
       const T ra = fma(kc2, s2a, fma(-kc1, s1a, fma(-kc0, xc.x, fk.x)));
       const T rb = fma(kc2, s2b, fma(-kc1, s1b, fma(-kc0, xc.y, fk.y)));
-      T o0 = ra, o1 = rb;
-      if (MODE == OP_JACOBI) {
-        o0 = fma(wt[wxy[r][0] + kz25], ra, xc.x);
-        o1 = fma(wt[wxy[r][1] + kz25], rb, xc.y);
-      }
-      if (MODE == OP_RESID && vrow != nullptr) {
-        const uchar2 vm = mq[r];
-        if (k + 1 < kb) mq[r] = *reinterpret_cast<const uchar2*>(vrow + sz + r * sy);
-        if (vm.x && vm.y) {
-          st2<T>(orow + r * sy, V{o0, o1});
-        } else {
-          if (vm.x) orow[r * sy] = o0;
-          if (vm.y) orow[r * sy + 1] = o1;
-        }
-      } else {
-        st2<T>(orow + r * sy, V{o0, o1});
-      }
+      st2<T>(orow + r * sy, V{fma(wt[wxy[r][0] + kz25], ra, xc.x), fma(wt[wxy[r][1] + kz25], rb, xc.y)});
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[s2]);  // plane k
@@ -261,7 +243,6 @@ __device__ __forceinline__ void zqueue_march(T* ring, unsigned long long* gbar, 
       par4 ^= 1;
     }
     orow += sz;
-    if (MODE == OP_RESID && vrow) vrow += sz;
     frow += sz;
     return true;
   };
@@ -507,7 +488,7 @@ __global__ void __launch_bounds__(32 * (TY / RW + 2), sizeof(T) == 4 ? 3 : 2)  /
     for (int q = 0; q < 4; ++q)
       if (!mbar_wait(&gbar[q], 0u)) { fail(); return; }
     if constexpr (sw3_zqueue<T, MODE>()) {
-      zqueue_march<T, MODE, RW, S, SLOT>(ring, gbar, empty, (warp * RW + 2) * XW + c0, f, orow, vrow, p, ka, kb, lz, nzd,
+      zqueue_march<T, RW, S, SLOT>(ring, gbar, empty, (warp * RW + 2) * XW + c0, f, orow, p, ka, kb, lz, nzd,
                                          j0 + warp * RW, i0 + c0, wt, wxy, kc0, kc1, kc2, lane, err);
       return;
     }
