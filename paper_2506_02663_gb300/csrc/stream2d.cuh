@@ -10,7 +10,9 @@
 // the down form, whose first sweep is a product), each from a five-row register window of the
 // previous iterate; x neighbours come by shuffle from the two adjacent lanes.  A sweep costs ten
 // arithmetic instructions a cell plus one shuffle, and the halo is 2 x 12 of 128 columns
-// (1.2) and 18 rows per chunk: the 4096^2 Helmholtz solve went from 29.8 to 17.5 ms.  Rows of f wait in shared memory (thread-private: no barrier).
+// (1.2) and 18 rows per chunk: the 4096^2 Helmholtz solve went from 29.8 to 17.5 ms.  Rows are
+// requested four steps ahead by cp.async into slots private to their lane (no barrier): a step
+// waited for the row asked for one step earlier.
 //
 // Physical faces: the first and last lane of a face strip evaluate the two ghost cells of
 // Eqs. (velBCHomoDiri5th)/(Neumann5) from their own four cells; at the low y face row 0 is
