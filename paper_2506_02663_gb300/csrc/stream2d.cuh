@@ -170,7 +170,9 @@ struct LegRun {
       leg2::strow(L.x2 + o, make_float4(e.x + v.x, e.y + v.y, e.z + v.z, e.w + v.w));
     }
   }
-  // a residual row (down): rows pair up into coarse rows
+  // A residual row (down): rows pair up into coarse rows.  The lane's two coarse cells are stored in one
+  // access where they start on an even column of the coarse patch: always on level 0, and on a refined
+  // level where the box starts on an even coarse cell (boxes start on even fine cells).
   __device__ __forceinline__ void restrict_row(int k, float4 r) {
     if ((k & 1) == 0) {
       rp = r;
@@ -180,7 +182,13 @@ struct LegRun {
     const float2 v = make_float2((((rp.x + rp.y) + r.x) + r.y) * 0.25f, (((rp.z + rp.w) + r.z) + r.w) * 0.25f);
     const PatchDesc& q = L.gcp;
     const int gy = (L.gp.lo[1] + k) >> 1, gx = (L.gp.lo[0] + c0) >> 1;
-    *reinterpret_cast<float2*>(L.bcn + (gy - q.lo[1] + NG) * (int)q.sy + gx - q.lo[0] + NG) = v;
+    float* o = L.bcn + (gy - q.lo[1] + NG) * (int)q.sy + gx - q.lo[0] + NG;
+    if (((gx - q.lo[0]) & 1) == 0) {
+      *reinterpret_cast<float2*>(o) = v;
+    } else {
+      o[0] = v.x;
+      o[1] = v.y;
+    }
   }
   // row t of the first window: down / post w f, up xi + prolongation
   __device__ __forceinline__ float4 first(int t, float4 f, float4 xrow, float2 ca, float2 cb, float ea, float eb,
