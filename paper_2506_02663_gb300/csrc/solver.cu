@@ -3210,6 +3210,8 @@ struct BatchPlan {
   DevStats* d_stats = nullptr;
   DevStats* h_stats = nullptr;  // pinned
   unsigned long long* h_bits = nullptr;  // pinned copy of rbits, fbits
+  unsigned char* h_stage = nullptr;      // pinned: the descriptors of one call on their way to the device
+  size_t cap_stage = 0;
   cudaStream_t cs = nullptr, bs = nullptr;
   cudaGraphExec_t exec = nullptr;
   long long launches_pre = 0, launches_body = 0;
@@ -3219,6 +3221,7 @@ struct BatchPlan {
     cudaFree(d_active); cudaFree(d_bits); cudaFree(d_stats);
     if (h_stats) cudaFreeHost(h_stats);
     if (h_bits) cudaFreeHost(h_bits);
+    if (h_stage) cudaFreeHost(h_stage);
     if (cs) cudaStreamDestroy(cs);
     if (bs) cudaStreamDestroy(bs);
     *this = BatchPlan();
@@ -3241,10 +3244,13 @@ inline int batch_levels(const amr_operator* op, const amr_solver_params& p) {
 }
 
 // Descriptors into a plan's array, kept from call to call and grown when needed (``moved``: the
-// graph holds the old address).  The caller's last use of the array has completed: every
-// batch call ends with a synchronisation.
+// graph holds the old address).  They go through the plan's pinned block, from offset ``at`` on, by a
+// copy on the caller's stream, which the graph launch that follows there waits for: a copy on the
+// default stream may still be on its way when a non-blocking stream reads the array.  The last
+// use of the array and of the block has completed: every batch call ends with a synchronisation
+// of its stream.
 template <typename D>
-amr_status upload(D** dst, size_t& cap, const std::vector<D>& v, bool& moved) {
+amr_status upload(BatchPlan& B, D** dst, size_t& cap, const std::vector<D>& v, size_t& at, bool& moved, cudaStream_t st) {
   const size_t bytes = v.size() * sizeof(D);
   if (bytes > cap) {
     cudaFree(*dst);
@@ -3254,7 +3260,10 @@ amr_status upload(D** dst, size_t& cap, const std::vector<D>& v, bool& moved) {
     cap = bytes;
     moved = true;
   }
-  if (bytes > 0) CK(cudaMemcpy(*dst, v.data(), bytes, cudaMemcpyHostToDevice));
+  if (bytes == 0) return AMR_OK;
+  std::memcpy(B.h_stage + at, v.data(), bytes);
+  CK(cudaMemcpyAsync(*dst, B.h_stage + at, bytes, cudaMemcpyHostToDevice, st));
+  at += bytes;
   return AMR_OK;
 }
 
@@ -3268,7 +3277,7 @@ inline int batch_tile(const int*) { return 32; }
 constexpr int LEG_BATCH_MIN = 300;
 
 // descriptors of every phase, grouped into launches
-amr_status build_batch_lists(BatchPlan& B, bool& moved) {
+amr_status build_batch_lists(BatchPlan& B, bool& moved, cudaStream_t st) {
   const amr_solver_params& p = B.p;
   B.down.clear();
   B.up.clear();
@@ -3445,12 +3454,22 @@ amr_status build_batch_lists(BatchPlan& B, bool& moved) {
   B.coarse = BatchGroup{0, B.n, 0, 0, 0};
   B.resid = BatchGroup{0, B.n, rtx, rty, 0};
   B.flat = BatchGroup{0, B.n, (int)std::min<long long>((nmax + 255) / 256, 64), 0, 0};
-  TRY(upload(&B.d_leg, B.cap[0], leg, moved));
-  TRY(upload(&B.d_down, B.cap[1], down, moved));
-  TRY(upload(&B.d_up, B.cap[2], up, moved));
-  TRY(upload(&B.d_coarse, B.cap[3], coarse, moved));
-  TRY(upload(&B.d_resid, B.cap[4], resid, moved));
-  TRY(upload(&B.d_flat, B.cap[5], flat, moved));
+  const size_t stage = leg.size() * sizeof(Leg2D) + down.size() * sizeof(BDown) + up.size() * sizeof(BUp) +
+                       coarse.size() * sizeof(BCoarse) + resid.size() * sizeof(BResid) + flat.size() * sizeof(BFlat);
+  if (stage > B.cap_stage) {
+    cudaFreeHost(B.h_stage);
+    B.h_stage = nullptr;
+    B.cap_stage = 0;
+    CK(cudaMallocHost(&B.h_stage, stage));
+    B.cap_stage = stage;
+  }
+  size_t at = 0;
+  TRY(upload(B, &B.d_leg, B.cap[0], leg, at, moved, st));
+  TRY(upload(B, &B.d_down, B.cap[1], down, at, moved, st));
+  TRY(upload(B, &B.d_up, B.cap[2], up, at, moved, st));
+  TRY(upload(B, &B.d_coarse, B.cap[3], coarse, at, moved, st));
+  TRY(upload(B, &B.d_resid, B.cap[4], resid, at, moved, st));
+  TRY(upload(B, &B.d_flat, B.cap[5], flat, at, moved, st));
   if (B.n > B.cap_n) {
     moved = true;
     B.cap_n = 0;
@@ -3607,6 +3626,15 @@ bool same_params(const amr_solver_params& a, const amr_solver_params& b) {
          a.temporal_blocking == b.temporal_blocking && a.fuse_coarse == b.fuse_coarse;
 }
 
+// one run of the plan's graph, its statistics and norms read back
+amr_status run_batch(BatchPlan& B, int n, cudaStream_t st) {
+  CK(cudaGraphLaunch(B.exec, st));
+  CK(cudaMemcpyAsync(B.h_stats, B.d_stats, n * sizeof(DevStats), cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(B.h_bits, B.d_bits, 2 * n * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
+  return AMR_OK;
+}
+
 // the batch through the work-list graph; AMR_OK / per-problem status as amr_batch_solve
 amr_status batch_worklist(amr_operator* const* ops, int n, const amr_solver_params& q, double* const* phi,
                           const double* const* f, amr_solve_stats* stats, int* status, cudaStream_t st) {
@@ -3618,6 +3646,13 @@ amr_status batch_worklist(amr_operator* const* ops, int n, const amr_solver_para
   // the launches of the last one therefore only uploads descriptors (96 problems, three
   // sets of fields in turn: 7.70 -> 7.39 ms a call).
   const bool same = plan.exec && plan.n == n && same_params(plan.p, q);
+  // no plan is kept whose descriptors may not have reached the device
+  auto fail = [&](amr_status s) {
+    cudaStreamSynchronize(st);
+    cudaGetLastError();
+    plan.release();
+    return s;
+  };
   bool hit = same;
   for (int k = 0; hit && k < n; ++k)
     hit = plan.serial[k] == ops[k]->serial && plan.phi[k] == phi[k] && plan.f[k] == f[k];
@@ -3639,16 +3674,13 @@ amr_status batch_worklist(amr_operator* const* ops, int n, const amr_solver_para
     const std::vector<BatchGroup> down = plan.down, up = plan.up;
     const BatchGroup parts[3] = {plan.coarse, plan.resid, plan.flat};
     bool moved = !same;
-    if (s == AMR_OK) s = build_batch_lists(plan, moved);
+    if (s == AMR_OK) s = build_batch_lists(plan, moved, st);
     moved = moved || down != plan.down || up != plan.up || !(parts[0] == plan.coarse) || !(parts[1] == plan.resid) ||
             !(parts[2] == plan.flat);
     if (s == AMR_OK && moved) s = build_batch_graph(plan);
-    if (s != AMR_OK) { plan.release(); return s; }
+    if (s != AMR_OK) return fail(s);
   }
-  CK(cudaGraphLaunch(plan.exec, st));
-  CK(cudaMemcpyAsync(plan.h_stats, plan.d_stats, n * sizeof(DevStats), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(plan.h_bits, plan.d_bits, 2 * n * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
+  if (const amr_status s = run_batch(plan, n, st); s != AMR_OK) return fail(s);
   amr_status worst = AMR_OK;
   long long iters = 0;
   for (int k = 0; k < n; ++k) {
