@@ -3271,10 +3271,19 @@ amr_status upload(BatchPlan& B, D** dst, size_t& cap, const std::vector<D>& v, s
 // where the halo recomputation of a tile (a 36^2 region for 16^2 cells, 52^2 for 32^2) is
 // the cost, so the batch takes 32^2 tiles
 inline int batch_tile(const int*) { return 32; }
-// smallest extent of a streamed leg in a batch: a leg of a smaller grid is bound by one warp's
-// 50 dependent row steps (96 problems of 64^2 .. 512^2: 7.4 ms with 300, 7.7 ms without
-// streaming, 8.4 ms with 200, 9.3 ms with 96)
+// Streamed legs in a batch.  LEG_BATCH_MIN: smallest extent; a leg of a smaller grid is bound by one
+// warp's 50 dependent row steps (96 problems of 64^2 .. 512^2: 7.4 ms with 300, 7.7 ms without
+// streaming, 8.4 ms with 200, 9.3 ms with 96).  The problems are squares of 64 2^k or 48 2^k cells, so
+// the line lies between 256 and 384.  LEG_BATCH_ROWS: strip rows a depth of the batch needs, so
+// that every resident warp gets about eleven; with fewer the chip stays idle behind the same 50 steps,
+// and tiles, a block per 32^2 cells, are faster.  Batches of k problems of n^2 cells, us, streamed at
+// any number of rows / with the line at 12000, 16000, 20000, 28000:
+//   1 x 512 (2,560 rows)    1710 / 1256 1254 1253 1254    12 x 384 (18,432 rows)   1743 / 1779 1783 1729 1721
+//   8 x 384 (12,288 rows)   1476 / 1478 1326 1327 1326    16 x 384 (24,576 rows)   2044 / 2035 2040 2040 2121
+//   2 x 1024 (20,480 rows)  4988 / 4634 4599 4692 4558     3 x 1024 (30,720 rows)  5922 / 5457 5409 5458 5700
+//   8 x 512 (20,480 rows)   2511 / 2490 2437 2435 2449    16 x 768 (98,304 rows)   7841 / 7833 7837 7833 8065
 constexpr int LEG_BATCH_MIN = 300;
+constexpr long long LEG_BATCH_ROWS = 20000;
 
 // descriptors of every phase, grouped into launches
 amr_status build_batch_lists(BatchPlan& B, bool& moved, cudaStream_t st) {
@@ -3297,28 +3306,37 @@ amr_status build_batch_lists(BatchPlan& B, bool& moved, cudaStream_t st) {
   };
   // streamed legs of depth m: one entry per problem, rows split so that the launch fills the chip
   std::vector<Leg2D> leg;
-  auto streamed = [&](int k, int m, int nu) {
+  auto leg_fits = [&](int k, int m, int mode) {
     const int* n = B.ops[k]->h->mg[m].n;
-    return nu == LEG_NU && leg_shape(n) && n[0] >= LEG_BATCH_MIN && n[1] >= LEG_BATCH_MIN;
+    return (mode == LEG_DOWN ? p.nu1 : p.nu2) == LEG_NU && leg_shape(n) && n[0] >= LEG_BATCH_MIN && n[1] >= LEG_BATCH_MIN;
   };
-  auto leg_group = [&](int m, int mode) {
-    const int off = (int)leg.size(), nu = mode == LEG_DOWN ? p.nu1 : p.nu2;
-    long long rows = 0;  // strip rows of the launch
+  // strip rows of depth m's launch; 0 where they are too few to fill the chip
+  auto leg_rows = [&](int m, int mode) {
+    long long rows = 0;
     for (int k = 0; k < B.n; ++k)
-      if (K[k] > m && streamed(k, m, nu)) {
+      if (K[k] > m && leg_fits(k, m, mode)) {
         const int* n = B.ops[k]->h->mg[m].n;
         rows += (long long)leg_strips(n[0], mode == LEG_DOWN ? leg_hx<LEG_DOWN>() : leg_hx<LEG_UP>()) * n[1];
       }
+    return rows >= LEG_BATCH_ROWS ? rows : 0ll;
+  };
+  std::vector<long long> strip_rows[2];  // per direction and depth
+  for (int m = 0; m < B.kmax; ++m)
+    for (int mode : {LEG_DOWN, LEG_UP}) strip_rows[mode].push_back(leg_rows(m, mode));
+  auto streamed = [&](int k, int m, int mode) { return strip_rows[mode][m] > 0 && leg_fits(k, m, mode); };
+  auto leg_group = [&](int m, int mode) {
+    const int off = (int)leg.size();
+    const long long rows = strip_rows[mode][m];
     int blocks = 0;
     for (int k = 0; k < B.n; ++k) {
-      if (K[k] <= m || !streamed(k, m, nu)) continue;
+      if (K[k] <= m || !streamed(k, m, mode)) continue;
       amr_operator* op = B.ops[k];
       amr_hierarchy* h = op->h;
       Scratch<float>& S = op->s32;
       const LevelView lv = mg_view(h, m, op->bc), cv = mg_view(h, m + 1, op->bc);
       const PatchDesc &gp = h->mg[m].patch, &gcp = h->mg[m + 1].patch;
       const int ns = leg_strips(gp.n[0], mode == LEG_DOWN ? leg_hx<LEG_DOWN>() : leg_hx<LEG_UP>());
-      const long long share = std::max<long long>(1, leg_share() * ns * gp.n[1] / std::max<long long>(1, rows));
+      const long long share = std::max<long long>(1, leg_share() * ns * gp.n[1] / rows);
       Leg2D d = make_leg(mode, lv, &cv, gp, gcp, op->alpha, op->beta, p.omega, share);
       d.p = k;
       d.b = (m == 0 ? S.rin : S.mb[m]) + gp.off;
@@ -3342,7 +3360,7 @@ amr_status build_batch_lists(BatchPlan& B, bool& moved, cudaStream_t st) {
       const int off = (int)down.size();
       int tx = 0, ty = 0;
       for (int k = 0; k < B.n; ++k) {
-        if (K[k] <= m || streamed(k, m, p.nu1)) continue;
+        if (K[k] <= m || streamed(k, m, LEG_DOWN)) continue;
         amr_operator* op = B.ops[k];
         amr_hierarchy* h = op->h;
         if (batch_tile(h->mg[m].n) != tt) continue;
@@ -3377,7 +3395,7 @@ amr_status build_batch_lists(BatchPlan& B, bool& moved, cudaStream_t st) {
       const int off = (int)up.size();
       int tx = 0, ty = 0;
       for (int k = 0; k < B.n; ++k) {
-        if (K[k] <= m || streamed(k, m, p.nu2)) continue;
+        if (K[k] <= m || streamed(k, m, LEG_UP)) continue;
         amr_operator* op = B.ops[k];
         amr_hierarchy* h = op->h;
         if (batch_tile(h->mg[m].n) != tt) continue;
