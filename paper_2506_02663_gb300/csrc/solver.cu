@@ -1313,14 +1313,21 @@ size_t blk_smem_fx(const int* n, int nu, bool down) {
 }
 
 // Streamed legs (k_leg2d): FP32, four sweeps, columns in groups of four, whole coarse rows.
-// Below LEG_MIN_CELLS a leg has too few strips and rows to fill the chip and the tiled form,
-// with a block per 16^2 cells, is faster (4096^2 solve with the line at 768^2, 500^2, 250^2:
-// 14.3 to 15.2, 15.7, 16.5 ms).
-constexpr long long LEG_MIN_CELLS = 768ll * 768;
+// Below a number of cells a leg has too few strips and rows to fill the chip and the tiled form is
+// faster.  The line depends on the tile it competes with: 16^2 cells below 1024^2 (LEG_MIN_CELLS16), 32^2
+// with less halo from there on (LEG_MIN_CELLS32).  Single-level mixed solves, us, finest leg streamed /
+// in tiles:
+//   768^2 1752 / 1782, 832^2 2308 / 2422, 896^2 2439 / 2655, 960^2 2842 / 3224 (16^2 tiles)
+//   1024^2 2591 / 2430, 2048 x 512 3502 / 3295, 1152 x 1024 3214 / 3065, 1152^2 3418 / 3374,
+//   1280 x 1024 3448 / 3419, 1536 x 1024 3993 / 4113, 1280^2 3772 / 3868, 2048 x 768 4147 / 4291,
+//   2048 x 1024 5127 / 5255, 1536^2 4859 / 5095, 2048^2 5664 / 7185 (32^2 tiles)
+// (smaller than 768^2: 512^2 streamed 1593, in tiles 914).
+constexpr long long LEG_MIN_CELLS16 = 768ll * 768, LEG_MIN_CELLS32 = 1500000;
 inline bool leg_shape(const int* n) { return n[0] % 4 == 0 && n[1] % 2 == 0 && n[0] >= 16 && n[1] >= 16; }
 template <typename T>
 bool leg_ok(const int* n, int nu) {
-  return sizeof(T) == 4 && nu == LEG_NU && leg_shape(n) && (long long)n[0] * n[1] >= LEG_MIN_CELLS;
+  return sizeof(T) == 4 && nu == LEG_NU && leg_shape(n) &&
+         (long long)n[0] * n[1] >= (blk_tile(n) == 16 ? LEG_MIN_CELLS16 : LEG_MIN_CELLS32);
 }
 
 // Geometry and coefficients of one streamed leg; ``share``: warps it should split into.
