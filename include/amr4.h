@@ -538,8 +538,7 @@ amr_status amr_set_tile_rows(int rows);
  * the largest interior |phi| rounded down to a power of two (at most half a unit in the last
  * place of that value, the size of one FP64 rounding of it); the sum 16 s1 - s2 - 90 phi of
  * Eq. (discreteOps) is then exact in int64, and r = f - alpha phi - beta/(12 h^2) * sum is
- * formed in FP64.  The same switch covers 2-D levels that are the whole domain, of at least
- * 2^21 cells, with a unit three bits finer.  Physical ghost values are fixed combinations of interior values and
+ * formed in FP64.  Physical ghost values are fixed combinations of interior values and
  * always fit; a stored ghost value (coarse-fine, copy) of 4 * 2^53 units or more, or a
  * non-finite value, makes the plain FP64 kernel recompute the level.  Not in the paper: on
  * this GPU FP64 arithmetic runs at a small fraction of the integer rate.  on = 0: the plain

@@ -23,7 +23,6 @@
 #include "coarse3d.cuh"
 #include "mgcluster.cuh"
 #include "stream2d.cuh"
-#include "resid2d.cuh"
 #include "cic.cuh"
 #include "migrate.cuh"
 
@@ -641,53 +640,12 @@ inline bool small_offsets(const LevelView& lv) {
   return px * (lv.maxn[1] + 2 * NG) * (lv.D == 3 ? lv.maxn[2] + 2 * NG : 1) < (1LL << 31);
 }
 
-// The fixed-point FP64 residual of a 2-D level that is the whole domain (k_resid2d_fx): columns in
-// groups of four, fields aligned for FP64 pairs, and a grid large enough for the FP64 rate,
-// not the launches, to bound the plain kernel (residual with its frame pass against plain, launch
-// gaps included, alpha not zero: 2048 x 1024 81 against 87 us, 2304 x 2048 99 against 137 us, 4096^2
-// 262 against 377 us; an earlier form on 1024^2: 74 against 65 us).
-inline bool fx2d_shape(const LevelView& lv) {
-  const PatchDesc& p = lv.p0;
-  return lv.D == 2 && lv.npatch == 1 && p.n[0] == lv.ndom[0] && p.n[1] == lv.ndom[1] && p.n[0] % 4 == 0 && p.n[0] >= 16 &&
-         p.n[1] >= 8;
-}
-inline bool fx2d_aligned(const PatchDesc& p, const double* x, const double* f, const double* out) {
-  const uintptr_t o = (uintptr_t)p.off * sizeof(double);
-  return ((reinterpret_cast<uintptr_t>(x) + o) | (reinterpret_cast<uintptr_t>(f) + o) |
-          (reinterpret_cast<uintptr_t>(out) + o)) % 16 == 0 && p.sy % 2 == 0;
-}
-constexpr double FX2D_MIN_CELLS = 2097152.0;
-amr_status launch_resid2d_fx(const LevelView& lv, const double* x, const double* f, double* out, double alpha, double beta,
-                             cudaStream_t st) {
-  CK(cudaMemsetAsync(lv.fxs, 0, 2 * sizeof(unsigned long long), st));
-  const int n1 = lv.p0.n[1];
-  launch(k_absmax_patch, (unsigned)std::min((n1 + 7) / 8, 8 * sm_count()), 256, 0, st, lv, x, lv.fxs);
-  TRY(launch_check());
-  const int ns = (lv.p0.n[0] + RX_W - 1) / RX_W;
-  // rows per chunk: 16 warps per SM, at least 16 rows (four are read ahead of the first)
-  const int nch = (int)std::max<long long>(1, std::min<long long>(n1 / 16, 16LL * sm_count() / ns));
-  const int ch = (n1 + nch - 1) / nch;
-  const int chunks = (n1 + ch - 1) / ch;
-  launch(alpha != 0.0 ? k_resid2d_fx<true> : k_resid2d_fx<false>, (unsigned)((ns * chunks + RX_WARPS - 1) / RX_WARPS), 32 * RX_WARPS, 0, st, lv, ns, chunks, ch, x, f, out,
-         alpha, beta);
-  return launch_check();
-}
-
 template <typename T, int D, bool TR = false>
 amr_status level_op(int mode, const LevelView& lv, const T* x, const T* f, T* out, const T* bc, double alpha,
                     double beta, double omega, const unsigned char* vmask, cudaStream_t st) {
   Geo g = geo_of(lv);
   cudaEvent_t ev;
   prof_begin(st, &ev);
-  if constexpr (sizeof(T) == 8 && D == 2 && !TR) {
-    if (mode == OP_RESID && bc == nullptr && vmask == nullptr && lv.fxs != nullptr &&
-        g_fx_resid.load(std::memory_order_relaxed) != 0 && lv.ncells >= FX2D_MIN_CELLS && fx2d_shape(lv) &&
-        small_offsets(lv) && fx2d_aligned(lv.p0, x, f, out)) {
-      TRY(launch_resid2d_fx(lv, x, f, out, alpha, beta, st));
-      prof_end(st, ev, PC_RESID64, 3.0 * sizeof(T) * lv.ncells, lv.ncells);
-      return AMR_OK;
-    }
-  }
   if (D == 2) {
     // tiled 2-D path; omega / (interior diagonal) computed once here in the value type;
     // rows per thread from the autotuner's table (keyed by grid size), default by size
