@@ -732,11 +732,12 @@ amr_status level_op(int mode, const LevelView& lv, const T* x, const T* f, T* ou
       const dim3 grid((unsigned)((lv.maxn[0] * (long long)lv.maxn[1] + cb - 1) / cb), (nz + kz - 1) / kz, lv.npatch);
       const JFac<T, 3> jf = (mode == OP_JACOBI || mode == OP_JACOBI0) ? jacobi_factors<T, 3>(lv, alpha, beta, omega) : JFac<T, 3>{};
       const T A = T(alpha), B = T(beta);
+      const int lap = zc_eligible(lv, 2) ? 0 : 1;
       switch (mode) {
-        case OP_APPLY: launch(k_level_op3d_col<T, OP_APPLY, TR>, grid, cb, 0, st, lv, kz, x, f, out, A, B, jf, vmask); break;
-        case OP_RESID: launch(k_level_op3d_col<T, OP_RESID, TR>, grid, cb, 0, st, lv, kz, x, f, out, A, B, jf, vmask); break;
-        case OP_JACOBI: launch(k_level_op3d_col<T, OP_JACOBI, TR>, grid, cb, 0, st, lv, kz, x, f, out, A, B, jf, vmask); break;
-        default: launch(k_level_op3d_col<T, OP_JACOBI0, TR>, grid, cb, 0, st, lv, kz, x, f, out, A, B, jf, vmask);
+        case OP_APPLY: launch(k_level_op3d_col<T, OP_APPLY, TR>, grid, cb, 0, st, lv, kz, x, f, out, A, B, jf, vmask, lap); break;
+        case OP_RESID: launch(k_level_op3d_col<T, OP_RESID, TR>, grid, cb, 0, st, lv, kz, x, f, out, A, B, jf, vmask, lap); break;
+        case OP_JACOBI: launch(k_level_op3d_col<T, OP_JACOBI, TR>, grid, cb, 0, st, lv, kz, x, f, out, A, B, jf, vmask, lap); break;
+        default: launch(k_level_op3d_col<T, OP_JACOBI0, TR>, grid, cb, 0, st, lv, kz, x, f, out, A, B, jf, vmask, lap);
       }
       const double nb = mode == OP_JACOBI0 ? 2.0 : (mode == OP_APPLY ? 2.0 : 3.0);
       prof_end(st, ev, (mode == OP_JACOBI || mode == OP_JACOBI0) ? PC_JACOBI : (mode == OP_RESID && sizeof(T) == 8) ? PC_RESID64 : PC_RESID,
