@@ -3364,8 +3364,9 @@ struct FixSum {
   __device__ __forceinline__ void frame(int e) {
     if (e + 2 > E) move(max(e, 1) + 2);
   }
-  // the sum as a double-double
-  __device__ __forceinline__ void value(double& s, double& c) const {
+  // w times the sum as a double-double; w enters before the exponent, so that a sum beyond the double
+  // range whose weighted value is inside it does not overflow
+  __device__ __forceinline__ void value(double w, double& s, double& c) const {
     double h, e1, e2, e3;
     two_sum(79228162514264337593543950336.0 * (double)(int)l3, 18446744073709551616.0 * (double)l2, h, e1);
     two_sum(h, 4294967296.0 * (double)l1, h, e2);
@@ -3373,8 +3374,10 @@ struct FixSum {
     // the unit is 2^(E - 1125): two factors in the normal range
     const int k = E - 1125, ka = k / 2;
     const double fa = __longlong_as_double((long long)(1023 + ka) << 52), fb = __longlong_as_double((long long)(1023 + k - ka) << 52);
-    s = h * fa * fb;
-    c = (e1 + (e2 + e3)) * fa * fb;
+    const double hi = w * h;
+    two_sum(hi, fma(w, e1 + (e2 + e3), fma(w, h, -hi)), s, c);
+    s = s * fa * fb;
+    c = c * fa * fb;
   }
 };
 
@@ -3382,7 +3385,7 @@ struct FixSum {
 // number of blocks per level (the rows each warp visits depend only on the launch shape): one
 // double-double partial part[2*(base+block)].  A warp sums whole rows in fixed point (FixSum, one
 // frame per warp), the warps' sums are brought to one frame and added, and w multiplies the
-// block's sum exactly (TwoProd).
+// block's sum (TwoProd).
 template <int D>
 __global__ void __launch_bounds__(256) k_wsum_gs(LevelView lv, const double* __restrict__ x,
                                                  const unsigned char* __restrict__ vmask, double w,
@@ -3444,12 +3447,9 @@ __global__ void __launch_bounds__(256) k_wsum_gs(LevelView lv, const double* __r
   a.move((int)__reduce_max_sync(0xffffffffu, (unsigned)max(a.E, 1)));
   a.reduce(8);
   double s, c;
-  a.value(s, c);
+  a.value(w, s, c);
   if (nan) s = __longlong_as_double(0x7ff8000000000000ll);
   if (lane == 0) {
-    const double hi = w * s, lo = fma(w, s, -hi);
-    const double e = fma(w, c, lo);
-    two_sum(hi, e, s, c);
     part[2 * (base + blockIdx.x)] = s;
     part[2 * (base + blockIdx.x) + 1] = c;
   }
@@ -3531,7 +3531,7 @@ __global__ void __launch_bounds__(256) k_dd_final(const double* __restrict__ par
   if (threadIdx.x != 0) return;
   for (int q = 1; q < 8; ++q) a.join(sl[q].x, sl[q].y, sl[q].z, sl[q].w);
   double s, c;
-  a.value(s, c);
+  a.value(1.0, s, c);
   out[0] = s + c;
 }
 
