@@ -3292,14 +3292,18 @@ __device__ __forceinline__ void dd_add(double& s, double& c, double a, double ac
 
 // A sum of doubles in 128-bit fixed point: a double enters as its 53-bit significand shifted to a
 // common frame (exponent E), so additions are exact integer ones in any order.  Below the sign
-// the frame keeps 26 bits of headroom (2^24 terms at least) and 47 bits under the last bit of the
-// largest term: terms within a factor 2^47 of it enter exactly.  A larger term moves the frame by
-// a shift of the sum so far; bits below 2^-100 of the largest term are dropped.  An addition costs
+// the frame keeps 12 + room bits of headroom, for 2^(12 + room) terms (the host counts them, fixsum_room), and
+// 62 - room bits under the last bit of the largest term: terms within a factor 2^(62 - room) of it enter
+// exactly (2^59 with the 2^15 cells that a block takes of a 256^3 grid, 2^60 with 8192 partials).  A larger
+// term moves the frame by a shift of the sum so far; bits below 2^(room - 114) of the largest term are
+// dropped, where double-double sums drop those below 2^-106 of the sum so far.  An addition costs
 // about 30 integer instructions, where TwoSum costs seven FP64 ones at a fiftieth of their rate:
 // 128^3 + 64^3 33 -> 11 us, 256^2 14.3 -> 7.2 us.
 struct FixSum {
   unsigned l0 = 0, l1 = 0, l2 = 0, l3 = 0;
   int E = 0;  // frame; 0: nothing added yet
+  int room;   // bits of headroom beyond 12
+  __device__ __forceinline__ explicit FixSum(int room_) : room(room_) {}
 
   __device__ __forceinline__ static int exponent(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
   // v, of an exponent <= E - 2
@@ -3307,7 +3311,7 @@ struct FixSum {
     const unsigned bh = (unsigned)__double2hiint(v), bl = (unsigned)__double2loint(v);
     const int e = (int)((bh >> 20) & 0x7ffu);
     const unsigned mh = (bh & 0xfffffu) | (e != 0 ? 0x100000u : 0u);
-    const unsigned sh = (unsigned)(E - max(e, 1) + 14), bs = sh & 31u, ws = sh >> 5;
+    const unsigned sh = (unsigned)(E - max(e, 1) + room), bs = sh & 31u, ws = sh >> 5;
     const unsigned t2 = mh >> bs, t1 = __funnelshift_r(bl, mh, bs), t0 = __funnelshift_r(0u, bl, bs);
     const unsigned m = (unsigned)((int)bh >> 31);  // negative: complement, plus one through the carry
     const unsigned x3 = m ^ (ws == 0 ? t2 : 0u);
@@ -3371,8 +3375,8 @@ struct FixSum {
     two_sum(79228162514264337593543950336.0 * (double)(int)l3, 18446744073709551616.0 * (double)l2, h, e1);
     two_sum(h, 4294967296.0 * (double)l1, h, e2);
     two_sum(h, (double)l0, h, e3);
-    // the unit is 2^(E - 1125): two factors in the normal range
-    const int k = E - 1125, ka = k / 2;
+    // the unit is 2^(E - 1139 + room): two factors in the normal range
+    const int k = E - 1139 + room, ka = k / 2;
     const double fa = __longlong_as_double((long long)(1023 + ka) << 52), fb = __longlong_as_double((long long)(1023 + k - ka) << 52);
     const double hi = w * h;
     two_sum(hi, fma(w, e1 + (e2 + e3), fma(w, h, -hi)), s, c);
@@ -3389,12 +3393,12 @@ struct FixSum {
 template <int D>
 __global__ void __launch_bounds__(256) k_wsum_gs(LevelView lv, const double* __restrict__ x,
                                                  const unsigned char* __restrict__ vmask, double w,
-                                                 double* __restrict__ part, long long base) {
+                                                 double* __restrict__ part, long long base, int room) {
   pdl_wait();
   constexpr int K = 8;  // cells of a lane in flight
   __shared__ uint4 sl[8];
   __shared__ int se[8];
-  FixSum a;
+  FixSum a(room);
   bool bad = false;  // a non-finite term
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nw = gridDim.x * 8;
@@ -3507,7 +3511,8 @@ __global__ void k_bsum(LevelView lv, const double* __restrict__ bc, const unsign
 
 // Sum of n double-double partials (one block of 256 threads), in the same fixed point with one
 // frame for all: the tree of double-double additions it replaces took 12 us.
-__global__ void __launch_bounds__(256) k_dd_final(const double* __restrict__ part, long long n, double* __restrict__ out) {
+__global__ void __launch_bounds__(256) k_dd_final(const double* __restrict__ part, long long n, double* __restrict__ out,
+                                                  int room) {
   pdl_wait();
   __shared__ int se[8];
   __shared__ uint4 sl[8];
@@ -3522,7 +3527,7 @@ __global__ void __launch_bounds__(256) k_dd_final(const double* __restrict__ par
     if (threadIdx.x == 0) out[0] = __longlong_as_double(0x7ff8000000000000ll);
     return;
   }
-  FixSum a;
+  FixSum a(room);
   a.frame(e);
   for (long long t = threadIdx.x; t < 2 * n; t += 256) a.add(part[t]);
   a.reduce(32);

@@ -2360,6 +2360,20 @@ inline long long wsum_blocks(const LevelView& lv) {
   return std::min<long long>(512, std::max<long long>(1, ((long long)lv.ncells + 255) / 256));
 }
 
+// Headroom (FixSum::room) of a sum of ``terms`` terms: 2^(12 + room) of them fit.
+inline int fixsum_room(long long terms) {
+  int b = 0;
+  while ((1ll << b) < terms) ++b;
+  return std::max(0, b - 12);
+}
+// ... of a block of k_wsum_gs on nb blocks: eight warps, whole rows, every patch from the first warp on
+inline int wsum_room(const amr_hierarchy* h, int l, long long nb) {
+  long long t = 0;
+  for (const PatchDesc& p : h->lev[l].patches)
+    t += 8 * (((long long)p.n[1] * p.n[2] + 8 * nb - 1) / (8 * nb)) * p.n[0];
+  return fixsum_room(t);
+}
+
 // The weighted sums keep one partial per block in the hierarchy's 8192-slot scratch: a
 // hierarchy that needs more is rejected before anything is launched.
 inline amr_status wsum_fits(amr_hierarchy* h) {
@@ -2384,11 +2398,12 @@ amr_status wsum(amr_hierarchy* h, const double* x, const double* bc, const int* 
       set_error("reduction scratch too small");
       return AMR_ERR_INVALID_ARG;
     }
-    launch(k_wsum_gs<D>, (unsigned)nb, 256, 0, st, lv, x, h->d_valid, unweighted ? 1.0 : std::pow(lv.h, D), h->d_red, base);
+    launch(k_wsum_gs<D>, (unsigned)nb, 256, 0, st, lv, x, h->d_valid, unweighted ? 1.0 : std::pow(lv.h, D), h->d_red, base,
+           wsum_room(h, l, nb));
     TRY(launch_check());
     base += nb;
   }
-  launch(k_dd_final, 1, 256, 0, st, h->d_red, base, d_out);
+  launch(k_dd_final, 1, 256, 0, st, h->d_red, base, d_out, fixsum_room(2 * base));
   TRY(launch_check());
   if (bc != nullptr && bc_types != nullptr) {
     long long bb = 0;
@@ -2399,7 +2414,7 @@ amr_status wsum(amr_hierarchy* h, const double* x, const double* bc, const int* 
       TRY(launch_check());
       bb += nblk;
     }
-    launch(k_dd_final, 1, 256, 0, st, h->d_red, bb, d_out + 1);
+    launch(k_dd_final, 1, 256, 0, st, h->d_red, bb, d_out + 1, fixsum_room(2 * bb));
     TRY(launch_check());
   } else {
     CK(cudaMemsetAsync(d_out + 1, 0, sizeof(double), st));
@@ -3877,11 +3892,11 @@ amr_status mean_zero_noalloc_impl(amr_hierarchy* h, double* x, double* mean_host
     LevelView lv = level_view(h, l, nullptr);
     const long long nb = wsum_blocks(lv);
     // every block writes its own partial slot, so no slot needs clearing first
-    launch(k_wsum_gs<D>, (unsigned)nb, 256, 0, st, lv, x, h->d_valid, std::pow(lv.h, D), part, base);
+    launch(k_wsum_gs<D>, (unsigned)nb, 256, 0, st, lv, x, h->d_valid, std::pow(lv.h, D), part, base, wsum_room(h, l, nb));
     TRY(launch_check());
     base += nb;
   }
-  launch(k_dd_final, 1, 256, 0, st, part, base, sums);
+  launch(k_dd_final, 1, 256, 0, st, part, base, sums, fixsum_room(2 * base));
   TRY(launch_check());
   launch(k_mean_from_sums, 1, 1, 0, st, sums, nullptr, 0.0, valid_volume(h), sums + 2);
   TRY(launch_check());
