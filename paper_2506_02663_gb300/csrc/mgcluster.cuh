@@ -40,6 +40,7 @@ struct MgCluster {
   int ng, nu1, nu2, nbot, ldb;
   const double* minv;     // bottom inverse (transposed for adjoint cycles)
   PatchDesc gp;           // layout of grid 0's right-hand side and correction
+  long long cstride;      // stacked component batches: one cluster per replica, this many elements apart
   int n[MC_MAX][3];
   int R[MC_MAX];          // slabs per block
   int mul[MC_MAX];        // slab k belongs to block (k * mul) >> 16
@@ -325,8 +326,10 @@ __global__ void __launch_bounds__(MC_THREADS) k_mg_cluster(const __grid_constant
   __shared__ T swt[MC_MAX * MgCluster<T, D>::NWT];
   __shared__ T sgh[24];
   __shared__ double bot[MC_BOT];
-  unsigned rank;
+  unsigned rank, nranks;
   asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(nranks));
+  const long long rep = (blockIdx.x / nranks) * c.cstride;
   for (int q = threadIdx.x; q < 3 * 54; q += MC_THREADS) sband[q] = (&c.band[0][0][0])[q];
   for (int q = threadIdx.x; q < c.ng * MgCluster<T, D>::NWT; q += MC_THREADS) swt[q] = (&c.wt[0][0])[q];
   if (threadIdx.x < 24) sgh[threadIdx.x] = (&c.ghost[0][0])[threadIdx.x];
@@ -334,7 +337,7 @@ __global__ void __launch_bounds__(MC_THREADS) k_mg_cluster(const __grid_constant
   const MgClusterRun<T, D, TR> v{c, reinterpret_cast<T*>(smraw), sband, swt, sgh, (int)rank};
   mc_sync();  // every block's shared memory exists before it is read
   pdl_wait();
-  v.run(b, x, bot);
+  v.run(b + rep, x + rep, bot);
 }
 
 }  // namespace amr4

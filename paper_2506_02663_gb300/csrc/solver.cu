@@ -1669,7 +1669,7 @@ constexpr int MC_MIN = 64;  // cells a block takes at least (64: poisson 64^2 1.
 template <typename T, int D, bool TR>
 int mg_cluster_m0(const amr_operator* op) {
   const amr_hierarchy* h = op->h;
-  if (h->ncomp != 1 || op->nbot > MC_BOT) return -1;
+  if (op->nbot > MC_BOT) return -1;
   const int cs = mg_cluster_size<T, D, TR>();
   if (cs == 0) return -1;
   int m0 = -1;
@@ -1695,6 +1695,7 @@ amr_status mg_cluster(amr_operator* op, const amr_solver_params& p, int m0, cons
   c.ldb = op->ldb;
   c.minv = TR ? op->d_binvT : op->d_binv;
   c.gp = h->mg[m0].patch;
+  c.cstride = h->mg[m0].cstride;
   c.alpha = T(op->alpha);
   for (int q = 0; q < c.ng; ++q) {
     const LevelView lv = mg_view(h, m0 + q, op->bc);
@@ -1725,7 +1726,7 @@ amr_status mg_cluster(amr_operator* op, const amr_solver_params& p, int m0, cons
   cudaEvent_t ev;
   prof_begin(st, &ev);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(cs, 1, 1);
+  cfg.gridDim = dim3(cs * h->ncomp, 1, 1);
   cfg.blockDim = dim3(MC_THREADS, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
@@ -1742,7 +1743,7 @@ amr_status mg_cluster(amr_operator* op, const amr_solver_params& p, int m0, cons
   if (e != cudaSuccess && g_launch_err == cudaSuccess) g_launch_err = e;
   TRY(launch_check());
   const MgGrid& g = h->mg[m0];
-  const double cells = (double)g.n[0] * g.n[1] * g.n[2];
+  const double cells = (double)g.n[0] * g.n[1] * g.n[2] * h->ncomp;
   prof_end(st, ev, PC_COARSE, 2.0 * sizeof(T) * cells, cells);  // read f, write x of the top grid
   return AMR_OK;
 }
