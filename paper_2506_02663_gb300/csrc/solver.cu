@@ -3108,6 +3108,7 @@ struct BatchPlan {
   std::vector<const double*> f;
   amr_solver_params p{};
   int n = 0, kmax = 0;
+  int dev = -1;                        // device of the arrays and the graph
   size_t cap[6] = {0, 0, 0, 0, 0, 0};  // bytes of the descriptor arrays (upload)
   int cap_n = 0;                       // problems the per-problem state holds
   std::vector<BatchGroup> down, up;  // per (m, tile) group, down in increasing m, up in decreasing m
@@ -3576,6 +3577,12 @@ amr_status batch_worklist(amr_operator* const* ops, int n, const amr_solver_para
   // and operators enter through the descriptors.  A call with other operators or fields but
   // the launches of the last one therefore only uploads descriptors (96 problems, three
   // sets of fields in turn: 7.70 -> 7.39 ms a call).
+  int dev = 0;
+  CK(cudaGetDevice(&dev));
+  if (plan.dev != dev) {
+    plan.release();
+    plan.dev = dev;
+  }
   const bool same = plan.exec && plan.n == n && same_params(plan.p, q);
   // no plan is kept whose descriptors may not have reached the device
   auto fail = [&](amr_status s) {
