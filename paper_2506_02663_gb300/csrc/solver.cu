@@ -4027,6 +4027,9 @@ static amr_status ensure_device(amr_hierarchy* h) {
     CK(cudaMemcpyToSymbol(c_cfi, h->cfi_w.data(), h->cfi_w.size() * sizeof(double)));
     std::vector<float> wf(h->cfi_w.begin(), h->cfi_w.end());
     CK(cudaMemcpyToSymbol(c_cfi_f, wf.data(), wf.size() * sizeof(float)));
+    // the lists and weights went by copies from pageable memory on the default stream, which may
+    // still be on their way; the caller's stream need not wait for that stream
+    CK(cudaStreamSynchronize(0));
     h->cfi_const_ready = true;
   }
   return AMR_OK;
