@@ -3936,8 +3936,9 @@ struct MigrateDev {
   ~MigrateDev() {
     for (void* p : ptrs) cudaFree(p);
   }
+  // on the caller's stream, which the kernels that read the list run on
   template <typename T>
-  amr_status put(const std::vector<T>& v, T** out) {
+  amr_status put(const std::vector<T>& v, T** out, cudaStream_t st) {
     *out = nullptr;
     if (v.empty()) return AMR_OK;
     if (cudaMalloc(out, sizeof(T) * v.size()) != cudaSuccess) {
@@ -3946,7 +3947,7 @@ struct MigrateDev {
       return AMR_ERR_OOM;
     }
     ptrs.push_back(*out);
-    CK(cudaMemcpy(*out, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(*out, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice, st));
     return AMR_OK;
   }
 };
@@ -3960,17 +3961,18 @@ amr_status migrate_impl(amr_hierarchy* oh, const double* xo, amr_hierarchy* nh, 
     set_error(err);
     return ps;
   }
+  const std::vector<unsigned> zero(1, 0u);
   MigrateDev dev;
   unsigned* bad = nullptr;
-  TRY(dev.put(std::vector<unsigned>(1, 0u), &bad));
+  TRY(dev.put(zero, &bad, st));
   for (int l = 0; l < nh->L; ++l) {
     const MigrateLevel& M = plan[l];
     MigrateBlock* db = nullptr;
     CfiEntry* dc = nullptr;
     long long* ds = nullptr;
-    TRY(dev.put(M.blocks, &db));
-    TRY(dev.put(M.cfi, &dc));
-    TRY(dev.put(M.side, &ds));
+    TRY(dev.put(M.blocks, &db, st));
+    TRY(dev.put(M.cfi, &dc, st));
+    TRY(dev.put(M.side, &ds, st));
     if (!M.blocks.empty()) {
       long long most = 1;
       for (const MigrateBlock& b : M.blocks) {
