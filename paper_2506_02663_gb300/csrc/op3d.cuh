@@ -68,11 +68,12 @@ struct TransLine {
 // grids spread over every SM (kz = 1 on the coarsest) and large ones keep the queue.
 // Replaces a shared-memory marching kernel with a barrier and 64-bit ghost code per plane, which
 // took 10 us on every FP32 grid down to 6 x 5 x 4 cells and 34 us per FP64 sweep of 72^3.
-// OP_APPLY and OP_RESID, whose results leave the library, form L x from the neighbour sums first
-// (``lap``) and add alpha x to it: with the coefficients folded as in the sweeps, alpha - 90 kc2 is
-// rounded once for all cells and f - A x of a Helmholtz system (small beta) has twice the error (72^3,
-// N(0,1) fields: rms 8.9e-17 and 1.6e-16, largest 7.1e-16 and 1.5e-15).  Levels that the tile kernels
-// (k_level_op3d_zc, k_sweep3d) also serve keep their folded form, bit for bit (lap = 0).  With
+// Results that leave the library (OP_APPLY, OP_RESID, the sweeps of amr_smooth) form L x from the
+// neighbour sums first (``lap``) and add alpha x to it: with the coefficients folded as in the V-cycle's
+// sweeps, alpha - 90 kc2 is rounded once for all cells and f - A x of a Helmholtz system (small beta) has
+// twice the error (72^3, N(0,1) fields: rms 8.9e-17 and 1.6e-16, largest 7.1e-16 and 1.5e-15).  Levels
+// that the tile kernels (k_level_op3d_zc, k_sweep3d) also serve keep their folded form, bit for bit
+// (lap = 0), and so do the V-cycle's FP64 sweeps, whose FP64 rate it saves (144^3 solve 7.52 against 7.83 ms).  With
 // the restriction, prolongation and bottom solve below, the FP64 Helmholtz solve on 72^3 + a
 // 56 x 52 x 72 box went from 6.05 to 2.95 ms and the mixed pressure solve on 96 x 80 x 64 with two
 // ragged boxes from 10.1 to 5.8 ms.
@@ -149,11 +150,12 @@ __global__ void __launch_bounds__(128) k_level_op3d_col(LevelView lv, int kz, co
     const T s1 = (x1 + y1) + z1;
     const T s2 = (x2 + y2) + z2;
     if (vb == nullptr || vb[o]) {
-      if ((MODE == OP_APPLY || MODE == OP_RESID) && (TR || lap)) {
+      // FP32 and transposed sweeps belong to V-cycles only (the choice alone costs an FP32 sweep 12 %)
+      if (MODE == OP_JACOBI ? (sizeof(T) == 8 && !TR && lap) : (TR || lap)) {
         T l = fma(T(-90), q2, fma(T(16), s1, -s2));
         if (TR) l += ex;
         const T ax = fma(alpha, q2, kc2 * l);
-        ob[o] = MODE == OP_APPLY ? ax : fk - ax;
+        ob[o] = MODE == OP_APPLY ? ax : MODE == OP_RESID ? fk - ax : fma(jf.w[cx + 5 * cy + 25 * cz], fk - ax, q2);
       } else if (MODE == OP_APPLY) {
         ob[o] = kc0 * q2 + (kc1 * s1 - kc2 * s2);
       } else {

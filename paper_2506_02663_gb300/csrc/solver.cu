@@ -642,7 +642,7 @@ inline bool small_offsets(const LevelView& lv) {
 
 template <typename T, int D, bool TR = false>
 amr_status level_op(int mode, const LevelView& lv, const T* x, const T* f, T* out, const T* bc, double alpha,
-                    double beta, double omega, const unsigned char* vmask, cudaStream_t st) {
+                    double beta, double omega, const unsigned char* vmask, cudaStream_t st, bool lap_sweep = false) {
   Geo g = geo_of(lv);
   cudaEvent_t ev;
   prof_begin(st, &ev);
@@ -732,7 +732,7 @@ amr_status level_op(int mode, const LevelView& lv, const T* x, const T* f, T* ou
       const dim3 grid((unsigned)((lv.maxn[0] * (long long)lv.maxn[1] + cb - 1) / cb), (nz + kz - 1) / kz, lv.npatch);
       const JFac<T, 3> jf = (mode == OP_JACOBI || mode == OP_JACOBI0) ? jacobi_factors<T, 3>(lv, alpha, beta, omega) : JFac<T, 3>{};
       const T A = T(alpha), B = T(beta);
-      const int lap = zc_eligible(lv, 2) ? 0 : 1;
+      const int lap = (mode == OP_APPLY || mode == OP_RESID || lap_sweep) && !zc_eligible(lv, 2) ? 1 : 0;
       switch (mode) {
         case OP_APPLY: launch(k_level_op3d_col<T, OP_APPLY, TR>, grid, cb, 0, st, lv, kz, x, f, out, A, B, jf, vmask, lap); break;
         case OP_RESID: launch(k_level_op3d_col<T, OP_RESID, TR>, grid, cb, 0, st, lv, kz, x, f, out, A, B, jf, vmask, lap); break;
@@ -1144,7 +1144,7 @@ amr_status smooth_from(const amr_hierarchy* h, int l, const LevelView& lv, const
   T* oth = b;
   for (int s = 0; s < nsweeps; ++s) {
     if (amr_level) TRY(copy_fill<T>(h, l, cur, st));
-    TRY(level_op<T, D, TR>(OP_JACOBI, lv, cur, f, oth, nullptr, alpha, beta, omega, nullptr, st));
+    TRY(level_op<T, D, TR>(OP_JACOBI, lv, cur, f, oth, nullptr, alpha, beta, omega, nullptr, st, amr_level));
     std::swap(cur, oth);
   }
   if (cur != a) {
