@@ -170,7 +170,11 @@ inline bool sw_eligible(const LevelView& lv) {
 }
 constexpr int TILE_BULK = 8;  // tile-table code of the bulk-copy 3-D kernel
 constexpr int TILE_COL = 16;  // and of the one-thread-per-column kernel (k_level_op3d_col): FP32 sweeps of 64^3 take
-                              // 5.0 us against 6.0 z-chunked and 11.1 bulk-copy, of 128^3 12.2 / 10.6 / 8.6
+                              // 5.0 us against 6.0 z-chunked and 11.1 bulk-copy, of 128^3 12.2 / 10.6 / 8.6.  Offered up to
+                              // TILE_COL_CELLS: solves with it and without, us, 96 x 80 x 64 mixed 487 / 499, 128^3 mixed (its
+                              // coarser grids) 1338 / 1376, FP64 4354 / 4633, 160^3 1816 / 1807 and 7129 / 7138; on 192^3 and
+                              // 224^3 offering it changes nothing (2365 / 2361, 4127 / 4121) but the tuning's time
+constexpr double TILE_COL_CELLS = 4194304.0;
 
 void free_stack(amr_operator* op);  // stacked component batches (defined with amr_batch_solve)
 
@@ -624,12 +628,12 @@ inline int sm_count() {
   static std::atomic<int> nsm[64];
   int dev = 0;
   cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64) return 152;
-  int m = nsm[dev].load(std::memory_order_relaxed);
+  const bool keep = dev >= 0 && dev < 64;
+  int m = keep ? nsm[dev].load(std::memory_order_relaxed) : 0;
   if (m == 0) {
     cudaDeviceGetAttribute(&m, cudaDevAttrMultiProcessorCount, dev);
     m = std::max(1, m);
-    nsm[dev].store(m, std::memory_order_relaxed);
+    if (keep) nsm[dev].store(m, std::memory_order_relaxed);
   }
   return m;
 }
@@ -1075,7 +1079,7 @@ amr_status autotune_tiles(amr_operator* op, cudaStream_t st) {
     const LevelView& lv = c.lv;
     std::vector<int> variants = D == 3 ? std::vector<int>{2} : std::vector<int>{1, 2, 4};
     if (D == 3 && zc_eligible(lv, 4)) variants.push_back(4);
-    if (D == 3 && zc_eligible(lv, 2) && lv.ncells <= 4194304.0) variants.push_back(TILE_COL);
+    if (D == 3 && zc_eligible(lv, 2) && lv.ncells <= TILE_COL_CELLS) variants.push_back(TILE_COL);
     if (D == 3 && sw_eligible(lv)) variants.push_back(TILE_BULK);
     if (variants.size() < 2) continue;  // nothing to choose
     const long long key = tile_key(lv, sizeof(T));
@@ -1105,7 +1109,7 @@ amr_status autotune_tiles(amr_operator* op, cudaStream_t st) {
         std::lock_guard<std::mutex> lock(g_tile_mu);
         g_tile_table.pop_back();
       }
-        // a larger tile (or the bulk-copy kernel) must win by 5 %: timing back-to-back sweeps
+      // a larger tile (or the bulk-copy kernel) must win by 5 %: timing back-to-back sweeps
       // flatters it (warmer L2)
       if (ms < 0.95f * best) { best = ms; best_rows = rows; }
     }
@@ -1696,8 +1700,10 @@ amr_status mg_level0(amr_operator* op, const amr_solver_params& p, int m, const 
     TRY((fused_config<T, D, TR>(op, m0, bytes)));
     if (m == m0) return fused_coarse<T, D, TR>(op, p, m0, bytes, b, x, st);
   }
-  // default: the coarse end in one cluster's shared memory (FP32 2-D forward V-cycles with blocked
-  // legs keep their one-block coarse kernels)
+  // default: the coarse end in one cluster's shared memory.  FP32 2-D forward V-cycles with blocked
+  // legs keep their one-block coarse kernels: mixed solves with these / with the cluster from 64^2 /
+  // from 128^2 on, us: 512^2 894 / 916 / 919, 1024^2 2425 / 2460 / 2472, three-level pressure solve on
+  // 256^2 2499 / 2543 / 2551
   if (p.fuse_coarse == 0 && p.nu1 >= 1 && !(D == 2 && sizeof(T) == 4 && !TR && p.temporal_blocking) &&
       m == mg_cluster_m0<T, D, TR>(op))
     return mg_cluster<T, D, TR>(op, p, m, b, x, st);
@@ -3866,7 +3872,9 @@ void cic_weights(double k, double eta, double w[2][4]) {
     for (int i = 0; i < 4; ++i) w[r][i] = m[r][3 - i];
 }
 
-// A 3-D level's first interface-ghost call must come before any stream capture.
+// A 3-D level's first interface-ghost call must come before any stream capture.  The call allocates
+// nothing any more; the rule is kept as the entry point's contract, so that what it refuses does not
+// depend on the kernels behind it.
 amr_status cic_first_call(amr_hierarchy* h, int l, cudaStream_t st) {
   LevelHost& L = h->lev[l];
   if (L.dev.cic_seen) return AMR_OK;

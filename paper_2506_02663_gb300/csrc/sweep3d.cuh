@@ -170,8 +170,9 @@ __host__ __device__ constexpr bool sw3_zqueue() {
 // k+1 sit in registers, so a step reads from the ring only the new plane's own cells, the x
 // neighbours and the four rows around the thread's own -- 16 shared loads for eight cells
 // instead of 44 -- and a plane's slot is free once its own step is done, two planes earlier.
-// One sweep repeated by itself: 256^3 44.5 -> 42.8 us (bound by the plane traffic, 1.33 halo
-// included); 128^3, where few planes are in flight, 12.0 -> 8.6 us.
+// Pays on 128^3, where few planes are in flight: 12.0 -> 8.6 us.  On 256^3 the plane traffic (1.33 halo
+// included) bounds both forms: 44.5 -> 42.8 us repeated by itself, and no gain inside a solve (49 us
+// per sweep in the benchmark's instrumented pass, 48 before).
 // Same sums in the same order as the loop that reads every neighbour from the ring.
 template <typename T, int RW, int S, int SLOT>
 __device__ __forceinline__ void zqueue_march(T* ring, unsigned long long* gbar, unsigned long long* empty, int rbase,
