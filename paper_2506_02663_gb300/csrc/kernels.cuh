@@ -3017,28 +3017,29 @@ __global__ void k_avgdown_T2(LevelView fine, LevelView crs, const XferBlock* __r
 }
 
 // ------------------------------------------------------------------------ elementwise
-// A pass over the interior cells of a level: a warp takes rows, a lane up to ROW_K of its cells at
-// once, their loads issued together (F::load), then their stores (F::store).  Bound by memory: as
-// one thread per cell in 65,536 blocks, X += E on 256^3 took 60 us where its bytes take 30 (128^3
-// FP32: 10.1 -> 6.0 us).
+// A pass over the interior cells of a level: a warp takes pieces of 32 ROW_K columns of a row, a lane
+// ROW_K of its cells at once, their loads issued together (F::load), then their stores (F::store).
+// Bound by memory: as one thread per cell in 65,536 blocks, X += E on 256^3 took 60 us where its bytes
+// take 30 (128^3 FP32: 10.1 -> 6.0 us).  Pieces, not whole rows: on 308^2 a warp went through its row in
+// three dependent steps on 39 of the SMs (5.6 us against 3.6; 1024^2 X += E 11.0 against 7.0).
 constexpr int ROW_K = 4;
 template <int D, typename F>
 __global__ void __launch_bounds__(256) k_rows(LevelView lv, F f) {
   pdl_wait();
   const PatchDesc p = lv.npatch == 1 ? lv.p0 : lv.patches[blockIdx.y];
-  const int lane = threadIdx.x & 31, rows = p.n[1] * (D == 3 ? p.n[2] : 1), nw = gridDim.x * 8;
+  const int lane = threadIdx.x & 31, np = (p.n[0] + 32 * ROW_K - 1) / (32 * ROW_K);  // pieces of a row
+  const unsigned n = (unsigned)np * p.n[1] * (D == 3 ? p.n[2] : 1), nw = gridDim.x * 8;
   f.begin();
-  for (int row = blockIdx.x * 8 + (threadIdx.x >> 5); row < rows; row += nw) {
+  for (unsigned u = blockIdx.x * 8 + (threadIdx.x >> 5); u < n; u += nw) {
+    const int row = (int)(u / np), i0 = (int)(u - (unsigned)row * np) * (32 * ROW_K) + lane;
     const long long o0 = poff(p, 0, row % p.n[1], D == 3 ? row / p.n[1] : 0);
-    for (int i0 = lane; i0 < p.n[0]; i0 += 32 * ROW_K) {
-      typename F::V v[ROW_K];
+    typename F::V v[ROW_K];
 #pragma unroll
-      for (int q = 0; q < ROW_K; ++q)
-        if (i0 + 32 * q < p.n[0]) v[q] = f.load(o0 + i0 + 32 * q);
+    for (int q = 0; q < ROW_K; ++q)
+      if (i0 + 32 * q < p.n[0]) v[q] = f.load(o0 + i0 + 32 * q);
 #pragma unroll
-      for (int q = 0; q < ROW_K; ++q)
-        if (i0 + 32 * q < p.n[0]) f.store(o0 + i0 + 32 * q, v[q]);
-    }
+    for (int q = 0; q < ROW_K; ++q)
+      if (i0 + 32 * q < p.n[0]) f.store(o0 + i0 + 32 * q, v[q]);
   }
 }
 

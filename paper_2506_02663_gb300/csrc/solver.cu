@@ -882,11 +882,11 @@ amr_status reflux(const amr_hierarchy* h, int l, const LevelView& crs, const Lev
   return launch_check();
 }
 
-// an elementwise pass over a level's rows: enough blocks to fill the chip, the rest by stride
+// an elementwise pass over a level's row pieces: enough blocks to fill the chip, the rest by stride
 template <int D, typename F>
 amr_status row_pass(const LevelView& lv, const F& f, cudaStream_t st) {
-  const long long rows = (long long)lv.maxn[1] * (D == 3 ? lv.maxn[2] : 1);
-  launch(k_rows<D, F>, dim3((unsigned)std::min<long long>((rows + 7) / 8, 16LL * sm_count()), lv.npatch, 1), 256, 0, st, lv, f);
+  const long long pieces = (long long)((lv.maxn[0] + 32 * ROW_K - 1) / (32 * ROW_K)) * lv.maxn[1] * (D == 3 ? lv.maxn[2] : 1);
+  launch(k_rows<D, F>, dim3((unsigned)std::min<long long>((pieces + 7) / 8, 16LL * sm_count()), lv.npatch, 1), 256, 0, st, lv, f);
   return launch_check();
 }
 
