@@ -4,11 +4,10 @@
 //   k_cfi_tile (3-D) /  the CF ghost cells of level l at an intermediate time t*: AMRCFI of the
 //   k_cic_grp           level-(l-1) data at four equispaced coarse times, combined by the 2 x 4
 //                       matrix I^(4)(k, eta) of Eq. (timeInterp) into the value at t* and its
-//                       time derivative (ratio 2).  Both maps are linear.  Regular face
-//                       rectangles of a 3-D level fold all four times along the face normal,
-//                       combine them there and share the folds along the face (kernels.cuh);
-//                       2-D levels and the other parents take k_cic_grp, which combines each
-//                       window cell and folds dimension by dimension.
+//                       time derivative (ratio 2).  Both maps are linear, and each window cell is
+//                       combined first.  Regular face rectangles of a 3-D level share the folds along the
+//                       normal and the first tangential dimension (kernels.cuh); 2-D levels and
+//                       the other parents take k_cic_grp, which folds dimension by dimension.
 //   k_cic_faces_sum /   the normal face averages n . <w> on the level's coarse-fine interface
 //   k_cic_faces_shift   faces (Eq. cell2face along the face normal, from the two interior
 //                       cells and the two CF ghost layers), corrected per connected component
