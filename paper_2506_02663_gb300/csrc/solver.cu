@@ -726,11 +726,13 @@ amr_status level_op(int mode, const LevelView& lv, const T* x, const T* f, T* ou
   if constexpr (D == 3) {
     if (bc == nullptr && (!TR || vmask == nullptr) && small_offsets(lv)) {
       // any other homogeneous 3-D level: one thread per column and run of kz planes, as many runs
-      // as give every SM 32 warps (half of its slots: enough loads in flight for L2, and long runs
-      // where the grid allows them)
+      // as give every SM 32 warps (half of its slots: enough loads in flight for L2), 64 where the runs
+      // keep eight planes then.  With 32 / with 64, us: two FP64 sweeps of 144^3 333 / 276 (a marching
+      // kernel before this one: 307), its FP64 solve 7419 / 6551, mixed 2385 / 2152; runs of two planes,
+      // mixed solves on 72^3 487 / 510, 96 x 80 x 64 497 / 511
       const long long warps = (long long)lv.npatch * ((lv.maxn[0] * (long long)lv.maxn[1] + 31) / 32);
-      const long long want = 32LL * sm_count();
       const int nz = lv.maxn[2];
+      const long long want = (warps * nz >= 8 * 64LL * sm_count() ? 64LL : 32LL) * sm_count();
       const int kz = (int)std::max<long long>(1, std::min<long long>(nz, (warps * nz + want - 1) / want));
       constexpr int cb = 64;
       const dim3 grid((unsigned)((lv.maxn[0] * (long long)lv.maxn[1] + cb - 1) / cb), (nz + kz - 1) / kz, lv.npatch);

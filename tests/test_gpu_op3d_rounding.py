@@ -11,7 +11,7 @@ import torch
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n0", [(40, 36, 44), (72, 72, 72), (56, 48, 40)])
+@pytest.mark.parametrize("n0", [(40, 36, 44), (72, 72, 72), (56, 48, 40), (144, 160, 144)])
 def test_helmholtz_rounding(n0):
     from paper_2506_02663_gb300 import amr
     alpha, beta, u = 1.0, -1e-8, 2.0 ** -53
