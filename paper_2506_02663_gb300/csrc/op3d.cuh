@@ -15,8 +15,8 @@ namespace amr4 {
 // One dimension of the transposed operator (trans_sums) with what does not depend on the plane
 // formed once per column: which neighbours exist, and the weights of the two cells next to the
 // near face that the cell's rows of the ghost formulas put on it.  Domains of eight cells and
-// more, so that a cell is near one face only.  A transposed FP32 sweep of 128^3: 21.9 -> 18.7
-// us, an FP64 application 98 -> 84 us.
+// more, so that a cell is near one face only.  Against the generic kernel of one thread per cell: a
+// transposed FP32 sweep of 128^3 22.6 -> 17.6 us, an FP64 application 108 -> 82 us.
 template <typename T>
 struct TransLine {
   T a, b;          // ex += a x[f] + b x[f + s]
@@ -77,8 +77,12 @@ struct TransLine {
 // the restriction, prolongation and bottom solve below, the FP64 Helmholtz solve on 72^3 + a
 // 56 x 52 x 72 box went from 6.05 to 2.95 ms and the mixed pressure solve on 96 x 80 x 64 with two
 // ragged boxes from 10.1 to 5.8 ms.
+// FP32 at 64 registers, the 32 warps per SM that the host counts on: left free, the transposed sweep takes
+// 80 and 23.6 us on 128^3 instead of 17.6, the mixed solve on 144^3 2137 instead of 2021 us.  FP64 has no
+// bound (0: its transposed application of 128^3 takes 82 us, at 80 registers 86; a bound of one block makes
+// the compiler take more registers, 72^3 solve 1165 -> 1184 us).
 template <typename T, int MODE, bool TR>
-__global__ void __launch_bounds__(128) k_level_op3d_col(LevelView lv, int kz, const T* __restrict__ x,
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 0) k_level_op3d_col(LevelView lv, int kz, const T* __restrict__ x,
                                                         const T* f, T* out, T alpha, T beta,
                                                         const __grid_constant__ JFac<T, 3> jf,
                                                         const unsigned char* __restrict__ vmask, int lap) {
